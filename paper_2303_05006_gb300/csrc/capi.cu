@@ -158,6 +158,7 @@ void tdbem_destroy(tdbem_ctx* c) {
   for (void* p : c->allocs) cudaFree(p);
   tdbem_fast_free(c);
   tdbem_mlp_free(c);
+  tdbem_sc_free(c);
   if (c->own_stream) cudaStreamDestroy(c->own_stream);
   delete c;
 }

@@ -931,25 +931,29 @@ using namespace tdbem;
 
 static int g_cluster = 0;
 
+// Meshes with at least this many RWG functions solve over a cooperative grid
+// of every SM instead of one cluster: a 16-SM cluster spends about 1 ms per
+// BiCGStab iteration at 120000 unknowns.
+constexpr int64_t kGridSolveRows = 49152;
+static bool use_grid(const tdbem_ctx* c) {
+  return c->p.solve_grid == 2 || (c->p.solve_grid == 0 && c->ne >= kGridSolveRows);
+}
+
 // Triangle-block (additive Schwarz) preconditioner: for every triangle the
 // 3 x 3 block of Z0 among the RWG functions of its three sides is inverted,
 // and P = sum over triangles of the inverses scattered to their rows and
 // columns.  Row i of P couples edge i with the other sides of its two
 // triangles (at most kPc entries).  A triangle whose block is singular adds
 // its diagonal reciprocals instead.
-static tdbem_status build_triangle_precond(tdbem_ctx* c, const std::vector<int32_t>& hp) {
-  const int64_t ne = c->ne, nnz = hp[ne];
-  std::vector<int32_t> hc(nnz);
-  std::vector<double> hv(nnz);
-  TDBEM_CUDA_TRY(c, cudaMemcpy(hc.data(), c->d_z0_col, nnz * sizeof(int32_t), cudaMemcpyDeviceToHost));
-  TDBEM_CUDA_TRY(c, cudaMemcpy(hv.data(), c->d_z0_val, nnz * sizeof(double), cudaMemcpyDeviceToHost));
+static tdbem_status build_triangle_precond(tdbem_ctx* c, const std::vector<int32_t>& hp, const std::vector<int32_t>& hc,
+                                           const std::vector<double>& hv, std::vector<int32_t>& pcol,
+                                           std::vector<double>& pval) {
+  const int64_t ne = c->ne;
   auto z = [&](int32_t i, int32_t j) {
     for (int32_t k = hp[i]; k < hp[i + 1]; ++k)
       if (hc[k] == j) return hv[k];
     return 0.0;
   };
-  std::vector<int32_t> pcol(kPc * ne, 0);
-  std::vector<double> pval(kPc * ne, 0.0);
   std::vector<int> used(ne, 0);
   auto add = [&](int32_t i, int32_t j, double v) {
     for (int k = 0; k < used[i]; ++k)
@@ -1018,8 +1022,26 @@ static tdbem_status tdbem_z0_f32(tdbem_ctx* c) {
                                                                        c->d_ell_val32);
   TDBEM_CUDA_TRY(c, cudaGetLastError());
   TDBEM_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  if (c->p.precond == 1) return build_triangle_precond(c, hp);
-  return TDBEM_OK;
+  const int64_t ne = c->ne, nnz = hp[ne];
+  std::vector<int32_t> hc(nnz);
+  std::vector<double> hv(nnz);
+  TDBEM_CUDA_TRY(c, cudaMemcpy(hc.data(), c->d_z0_col, nnz * sizeof(int32_t), cudaMemcpyDeviceToHost));
+  TDBEM_CUDA_TRY(c, cudaMemcpy(hv.data(), c->d_z0_val, nnz * sizeof(double), cudaMemcpyDeviceToHost));
+  std::vector<int32_t> pcol(kPc * ne, 0);
+  std::vector<double> pval(kPc * ne, 0.0);
+  if (c->p.precond == 1) {
+    if ((s = build_triangle_precond(c, hp, hc, hv, pcol, pval))) return s;
+  } else {
+    for (int64_t i = 0; i < ne; ++i) {
+      double d = 0.0;
+      for (int32_t k = hp[i]; k < hp[i + 1]; ++k)
+        if (hc[k] == i) d = hv[k];
+      pcol[i] = (int32_t)i;
+      pval[i] = d != 0.0 ? 1.0 / d : 1.0;
+    }
+  }
+  if (c->R > 1 || c->p.jacobi_sweeps > 0 || use_grid(c)) return TDBEM_OK;
+  return tdbem_sc_build(c, c->p.solve_cluster > 0 ? c->p.solve_cluster : 16, hp, hc, hv, pcol, pval);
 }
 
 tdbem_status tdbem_build_z0(tdbem_ctx* c) {
@@ -1110,10 +1132,6 @@ static tdbem_status pick_cluster(tdbem_ctx* c) {
   return TDBEM_ECUDA;
 }
 
-// Meshes with at least this many RWG functions solve over a cooperative grid
-// of every SM instead of one cluster: a 16-SM cluster spends about 1 ms per
-// BiCGStab iteration at 120000 unknowns.
-constexpr int64_t kGridSolveRows = 49152;
 static int g_grid = 0;
 static tdbem_status pick_grid(tdbem_ctx* c) {
   if (g_grid) return TDBEM_OK;
@@ -1210,8 +1228,10 @@ tdbem_status tdbem_solve_z0(tdbem_ctx* c, int32_t alpha, int32_t* iters, int32_t
   tdbem_status s;
   if (c->R > 1) {
     if ((s = solve_multi(c, alpha, warm))) return s;
+  } else if (c->sc) {
+    if ((s = tdbem_sc_solve(c, alpha, warm))) return s;
   } else {
-    const bool grid = c->p.solve_grid == 2 || (c->p.solve_grid == 0 && c->ne >= kGridSolveRows);
+    const bool grid = use_grid(c);
     if ((s = grid ? pick_grid(c) : pick_cluster(c))) return s;
     if (grid && !c->d_gslots && (s = c->dalloc(&c->d_gslots, (size_t)2 * g_grid * 4))) return s;
     SolveArgs A;

@@ -1,0 +1,867 @@
+// solve_cluster.cu -- the single-right-hand-side solve Z0 J^{alpha-1} =
+// R^{alpha-1} (paper eq. solve) in one thread-block cluster, with the exchanged
+// vector kept whole in every CTA's shared memory.
+//
+// Scheme.  Iterative refinement: an FP64 residual r = b - Z0 x around an FP32
+// BiCGStab on the right-preconditioned matrix A = Z0 P (P: triangle blocks or
+// the diagonal), which is formed once at setup.  The Krylov vectors live in
+// registers, each thread owning kScRows rows; only the vector that the next
+// product gathers from travels: every owner stores its values into all CTAs'
+// copies through distributed shared memory, so the gathers are shared-memory
+// reads and an iteration meets at four cluster barriers (p, alpha's dots, s,
+// omega's dots).
+//
+// What bounds it: latency.  The products stream A from L2 (the prefetch of
+// four blocks of 8 rows x 16 entries per warp keeps about 50 KB in flight per
+// SM), the reductions are dependent shuffles.  FP64 issues at 1/64 of FP32's
+// rate here (2 per clock and SM), so FP64 is left to the residuals and the
+// iterate; the dots are summed in double-float (FP32 pairs, 48 bits), the
+// Krylov scalars are FP32 and the refinement's scale is a power of two, which
+// needs no FP64 division or square root.
+//
+// Layout.  Rows are put in an order of their own (`perm`): sorted by length,
+// cut into groups of 8 (four lanes per row, so that a warp takes one group at a
+// time), the groups dealt over the CTAs and warps.  A warp's groups are one
+// contiguous run of blocks of 8 rows x 16 entries, zero padded; a lane reads
+// its four entries of a block as one vector, with 16-bit positions.
+#include <cooperative_groups.h>
+
+#include <algorithm>
+#include <new>
+#include <vector>
+
+#include "internal.h"
+
+namespace cg = cooperative_groups;
+
+namespace tdbem {
+
+constexpr int kScThreads = 512, kScWarps = kScThreads / 32;
+constexpr int kScPc = 5;            // entries per row of P
+constexpr int kScPasses = 24;       // groups per warp at most: 6 rows per thread
+constexpr double kScInner2 = 1e-10; // squared relative residual an inner solve stops at
+constexpr int kScPSharedRows = 2;   // rows per thread up to which P is staged in shared memory
+constexpr int kScDepth = 4;          // blocks a warp keeps in flight
+constexpr int kScInnerMax = 80;     // iterations of one inner solve
+
+struct ScArgs {
+  const int32_t* perm;       // [npad] row at a position, -1: padding
+  const int32_t *ab, *ae;    // A: first block of a warp [cs * 16], block ends of its passes [cs * 16][passes]
+  const float4* aval;        // [blocks][32]
+  const uint2* acol;         // [blocks][32] four 16-bit positions
+  const int32_t *zb, *ze;    // Z0, the same
+  const double2* zval;       // [blocks][32][2]
+  const float4 *zhi, *zlo;   // Z0 as (hi, lo) pairs
+  const uint2* zcol;
+  const float* pval;         // P: [kScPc][npad]
+  const uint16_t* pcol;
+  double* w64;               // [2][npad] iterates as the residual gathers them
+  const double* b;           // rows in edge order from here on
+  double* x;
+  double* ring;
+  int32_t L, alpha, warm, gpc, passes, npad, ne, maxit;
+  double tol;
+  int32_t* status;           // as in SolveArgs (solve.cu)
+  double* resid;
+};
+
+// double-float sums
+struct Df {
+  float h, l;
+};
+__device__ __forceinline__ Df df_plus(Df a, Df b) {
+  const float s = __fadd_rn(a.h, b.h);
+  const float bb = __fsub_rn(s, a.h);
+  const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, bb)), __fsub_rn(b.h, bb));
+  return {s, __fadd_rn(__fadd_rn(a.l, b.l), e)};
+}
+__device__ __forceinline__ Df df_xor(Df a, int m) {
+  return {__shfl_xor_sync(0xffffffffu, a.h, m), __shfl_xor_sync(0xffffffffu, a.l, m)};
+}
+
+// Shared memory of a CTA besides the gathered vector.
+struct ScShared {
+  float2 red[kScWarps][4];
+  float4 slots[2][16][2];      // [phase][rank]: four double-float sums
+  double red64[kScWarps][2];
+  double slots64[2][16][2];
+  double bc64[2];
+};
+
+__device__ __forceinline__ uint32_t sc_mapa(uint32_t a, int rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void sc_st(uint32_t a, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+__device__ __forceinline__ void sc_st4(uint32_t a, float x, float y, float z, float w) {
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
+}
+__device__ __forceinline__ void sc_st64(uint32_t a, double x, double y) {
+  asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(a), "d"(x), "d"(y) : "memory");
+}
+
+struct ScCtx {
+  ScShared* sm;
+  int nb, rank, warp, lane, phase;
+
+  __device__ __forceinline__ void sync() {
+    if (nb == 1) {
+      __syncthreads();
+    } else {
+      asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+      asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+  }
+
+  // Cluster-wide sums of v[0..3] over all threads (same bits in every thread).
+  // The four values are folded together: each shuffle step halves the values a
+  // lane carries, 6 double-float additions per lane instead of 20.
+  __device__ __forceinline__ void dots4(float v0, float v1, float v2, float v3, float (&out)[4]) {
+    Df k0, k1;
+    {
+      const bool up = lane & 16;
+      k0 = {up ? v2 : v0, 0.f};
+      k1 = {up ? v3 : v1, 0.f};
+      k0 = df_plus(k0, {__shfl_xor_sync(0xffffffffu, up ? v0 : v2, 16), 0.f});
+      k1 = df_plus(k1, {__shfl_xor_sync(0xffffffffu, up ? v1 : v3, 16), 0.f});
+    }
+    {
+      const bool up = lane & 8;
+      const Df s = up ? k0 : k1;
+      k0 = df_plus(up ? k1 : k0, df_xor(s, 8));
+    }
+    k0 = df_plus(k0, df_xor(k0, 4));
+    k0 = df_plus(k0, df_xor(k0, 2));
+    k0 = df_plus(k0, df_xor(k0, 1));
+    if ((lane & 7) == 0) sm->red[warp][lane >> 3] = make_float2(k0.h, k0.l);  // value lane >> 3
+    __syncthreads();
+    const int ph = phase++ & 1, id = lane & 3, k = lane >> 2;
+    Df t;
+    if (nb == 1) {  // one CTA: every warp sums the warps' values itself
+      const float2 a = sm->red[k][id], b = sm->red[k + 8][id];
+      t = df_plus({a.x, a.y}, {b.x, b.y});
+    } else {
+      if (warp == 0) {
+        const float2 a = sm->red[k][id], b = sm->red[k + 8][id];
+        t = df_plus({a.x, a.y}, {b.x, b.y});
+        t = df_plus(t, df_xor(t, 4));
+        t = df_plus(t, df_xor(t, 8));
+        t = df_plus(t, df_xor(t, 16));
+        // lane r < nb sends the four sums to CTA r
+        const uint32_t dst = sc_mapa((uint32_t)__cvta_generic_to_shared(&sm->slots[ph][rank][0]), lane < nb ? lane : 0);
+        const float a0 = __shfl_sync(0xffffffffu, t.h, 0), a1 = __shfl_sync(0xffffffffu, t.l, 0);
+        const float b0 = __shfl_sync(0xffffffffu, t.h, 1), b1 = __shfl_sync(0xffffffffu, t.l, 1);
+        const float c0 = __shfl_sync(0xffffffffu, t.h, 2), c1 = __shfl_sync(0xffffffffu, t.l, 2);
+        const float d0 = __shfl_sync(0xffffffffu, t.h, 3), d1 = __shfl_sync(0xffffffffu, t.l, 3);
+        if (lane < nb) {
+          sc_st4(dst, a0, a1, b0, b1);
+          sc_st4(dst + 16, c0, c1, d0, d1);
+        }
+      }
+      sync();
+      const float2* sl = reinterpret_cast<const float2*>(&sm->slots[ph][0][0]);  // [16][4]
+      t = {0.f, 0.f};
+      if (k < nb) t = {sl[k * 4 + id].x, sl[k * 4 + id].y};
+      if (k + 8 < nb) t = df_plus(t, {sl[(k + 8) * 4 + id].x, sl[(k + 8) * 4 + id].y});
+    }
+    t = df_plus(t, df_xor(t, 4));
+    t = df_plus(t, df_xor(t, 8));
+    t = df_plus(t, df_xor(t, 16));
+    const float s = t.h + t.l;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) out[i] = __shfl_sync(0xffffffffu, s, i);
+    if (nb == 1) __syncthreads();  // red is rewritten by the next sums
+  }
+
+  // Cluster-wide FP64 sums of a and b (same bits in every thread).
+  __device__ __forceinline__ void sums64(double& a, double& b) {
+    const bool up = lane & 16;
+    double k = up ? b : a;
+    k += __shfl_xor_sync(0xffffffffu, up ? a : b, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
+    if ((lane & 15) == 0) sm->red64[warp][lane >> 4] = k;
+    __syncthreads();
+    const int ph = phase++ & 1;
+    if (warp == 0) {
+      double t = sm->red64[lane >> 1][lane & 1];
+#pragma unroll
+      for (int o = 2; o < 32; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      const double t0 = __shfl_sync(0xffffffffu, t, 0), t1 = __shfl_sync(0xffffffffu, t, 1);
+      const uint32_t dst = sc_mapa((uint32_t)__cvta_generic_to_shared(&sm->slots64[ph][rank][0]), lane < nb ? lane : 0);
+      if (lane < nb) sc_st64(dst, t0, t1);
+    }
+    sync();
+    if (warp == 0) {
+      const int r = lane >> 1;
+      double t = r < nb ? sm->slots64[ph][r][lane & 1] : 0.0;
+#pragma unroll
+      for (int o = 2; o < 32; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      if (lane < 2) sm->bc64[lane] = t;
+    }
+    __syncthreads();
+    a = sm->bc64[0];
+    b = sm->bc64[1];
+  }
+};
+
+// A warp's rows of a matrix times the gathered vector.  Ld: the matrix's
+// entries of a block (load), its products added to an accumulator (mul), the
+// accumulator's sum over a row's four lanes (fold).  kScDepth blocks are in
+// flight: a warp's run is a multiple of that long (zero blocks behind its last
+// group), and the loads ahead of its end stay inside the padded array.
+// out[e] of lane (row, q) is the row of pass 4 e + q.
+template <int RPT, class Ld, class Out>
+__device__ __forceinline__ void sc_spmv(Ld ld, int b, int tot, int ends, int lane, Out (&out)[RPT]) {
+  typename Ld::Block buf[kScDepth];
+  asm volatile("" : "+r"(b));  // the addresses are formed here, not kept in registers over the solver's loops
+  int left = tot - b, j = 0, gleft = __shfl_sync(0xffffffffu, ends, 0) - b, gend = gleft + b;
+  ld.seek(b, lane);
+#pragma unroll
+  for (int i = 0; i < kScDepth; ++i) ld.load(buf[i], i);
+  typename Ld::Acc acc;
+  acc.zero();
+#pragma unroll
+  for (int e = 0; e < RPT; ++e) out[e] = 0;
+  for (; left > 0; left -= kScDepth) {
+    ld.skip();
+#pragma unroll
+    for (int i = 0; i < kScDepth; ++i) {
+      ld.mul(buf[i], acc);
+      ld.load(buf[i], i);
+      if (--gleft == 0) {
+        const Out s = acc.fold();
+        acc.zero();
+#pragma unroll
+        for (int e = 0; e < RPT; ++e)
+          if (j == 4 * e + (lane & 3)) out[e] = s;
+        ++j;
+        const int g2 = __shfl_sync(0xffffffffu, ends, j & 31);
+        gleft = g2 - gend;
+        gend = g2;
+      }
+    }
+  }
+}
+
+struct LdA {  // FP32 matrix, FP32 vector in shared memory
+  const float4* v;
+  const uint2* c;
+  const float* X;
+  struct Block {
+    float4 v;
+    uint2 c;
+  };
+  struct Acc {
+    float a, b;
+    __device__ __forceinline__ void zero() { a = b = 0.f; }
+    __device__ __forceinline__ float fold() {
+      float s = a + b;
+      s += __shfl_xor_sync(0xffffffffu, s, 1);
+      return s + __shfl_xor_sync(0xffffffffu, s, 2);
+    }
+  };
+  __device__ __forceinline__ void seek(int b, int lane) {
+    v += (int64_t)b * 32 + lane;
+    c += (int64_t)b * 32 + lane;
+  }
+  __device__ __forceinline__ void skip() {
+    v += kScDepth * 32;
+    c += kScDepth * 32;
+  }
+  __device__ __forceinline__ void load(Block& k, int i) const {
+    k.v = __ldg(v + i * 32);
+    k.c = __ldg(c + i * 32);
+  }
+  __device__ __forceinline__ void mul(const Block& k, Acc& s) const {
+    s.a = fmaf(k.v.x, X[k.c.x & 0xffff], s.a);
+    s.b = fmaf(k.v.y, X[k.c.x >> 16], s.b);
+    s.a = fmaf(k.v.z, X[k.c.y & 0xffff], s.a);
+    s.b = fmaf(k.v.w, X[k.c.y >> 16], s.b);
+  }
+};
+
+struct LdZ64 {  // FP64 matrix, FP64 vector in global memory
+  const double2* v;
+  const uint2* c;
+  const double* x;
+  struct Block {
+    double2 v0, v1;
+    uint2 c;
+  };
+  struct Acc {
+    double a;
+    __device__ __forceinline__ void zero() { a = 0.0; }
+    __device__ __forceinline__ double fold() {
+      double s = a;
+      s += __shfl_xor_sync(0xffffffffu, s, 1);
+      return s + __shfl_xor_sync(0xffffffffu, s, 2);
+    }
+  };
+  __device__ __forceinline__ void seek(int b, int lane) {
+    v += ((int64_t)b * 32 + lane) * 2;
+    c += (int64_t)b * 32 + lane;
+  }
+  __device__ __forceinline__ void skip() {
+    v += kScDepth * 64;
+    c += kScDepth * 32;
+  }
+  __device__ __forceinline__ void load(Block& k, int i) const {
+    k.v0 = __ldg(v + i * 64);
+    k.v1 = __ldg(v + i * 64 + 1);
+    k.c = __ldg(c + i * 32);
+  }
+  __device__ __forceinline__ void mul(const Block& k, Acc& s) const {
+    const double x0 = x[k.c.x & 0xffff], x1 = x[k.c.x >> 16], x2 = x[k.c.y & 0xffff], x3 = x[k.c.y >> 16];
+    s.a += k.v0.x * x0;
+    s.a += k.v0.y * x1;
+    s.a += k.v1.x * x2;
+    s.a += k.v1.y * x3;
+  }
+};
+
+struct LdZdf {  // (hi, lo) matrix, FP32 vector in shared memory, double-float products and sums
+  const float4 *h, *l;
+  const uint2* c;
+  const float* X;
+  struct Block {
+    float4 h, l;
+    uint2 c;
+  };
+  struct Acc {
+    float h, l;
+    __device__ __forceinline__ void zero() { h = l = 0.f; }
+    __device__ __forceinline__ void add(float zh, float zl, float x) {
+      const float p = __fmul_rn(zh, x);
+      const float e = __fmaf_rn(zl, x, __fmaf_rn(zh, x, -p));
+      const Df t = df_plus({h, l}, {p, e});
+      h = t.h;
+      l = t.l;
+    }
+    __device__ __forceinline__ double fold() {
+      Df t = {h, l};
+      t = df_plus(t, df_xor(t, 1));
+      t = df_plus(t, df_xor(t, 2));
+      return (double)t.h + (double)t.l;
+    }
+  };
+  __device__ __forceinline__ void seek(int b, int lane) {
+    h += (int64_t)b * 32 + lane;
+    l += (int64_t)b * 32 + lane;
+    c += (int64_t)b * 32 + lane;
+  }
+  __device__ __forceinline__ void skip() {
+    h += kScDepth * 32;
+    l += kScDepth * 32;
+    c += kScDepth * 32;
+  }
+  __device__ __forceinline__ void load(Block& k, int i) const {
+    k.h = __ldg(h + i * 32);
+    k.l = __ldg(l + i * 32);
+    k.c = __ldg(c + i * 32);
+  }
+  __device__ __forceinline__ void mul(const Block& k, Acc& s) const {
+    s.add(k.h.x, k.l.x, X[k.c.x & 0xffff]);
+    s.add(k.h.y, k.l.y, X[k.c.x >> 16]);
+    s.add(k.h.z, k.l.z, X[k.c.y & 0xffff]);
+    s.add(k.h.w, k.l.w, X[k.c.y >> 16]);
+  }
+};
+
+template <int RPT>
+__global__ void __launch_bounds__(kScThreads) k_solve_cluster(const ScArgs A) {
+  extern __shared__ __align__(16) float sc_X[];
+  __shared__ ScShared sm;
+  ScCtx S;
+  S.sm = &sm;
+  {
+    uint32_t n, r;
+    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(n));
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    S.nb = (int)n;
+    S.rank = (int)r;
+  }
+  S.warp = (int)threadIdx.x >> 5;
+  S.lane = (int)threadIdx.x & 31;
+  S.phase = 0;
+  const int lane = S.lane, q = lane & 3, W = S.rank * kScWarps + S.warp;
+  const uint32_t Xa = (uint32_t)__cvta_generic_to_shared(sc_X);
+  // P of this thread's rows, and Z0's and A's runs of this warp
+  float* pvs = sc_X + A.npad;  // [kScPc][RPT][threads]
+  uint16_t* pcs = reinterpret_cast<uint16_t*>(pvs + kScPc * RPT * kScThreads);
+  constexpr bool kPShared = RPT <= kScPSharedRows;
+  // this thread's rows: position and edge of each (-1: none)
+  int pos[RPT], row[RPT];
+#pragma unroll
+  for (int e = 0; e < RPT; ++e) {
+    const int g = (4 * e + q) * kScWarps + S.warp;
+    pos[e] = g < A.gpc ? (S.rank * A.gpc + g) * 8 + (lane >> 2) : -1;
+    row[e] = pos[e] >= 0 ? A.perm[pos[e]] : -1;
+    if constexpr (kPShared)
+#pragma unroll
+    for (int k = 0; k < kScPc; ++k) {
+      pvs[(k * RPT + e) * kScThreads + threadIdx.x] = pos[e] >= 0 ? A.pval[k * A.npad + pos[e]] : 0.f;
+      pcs[(k * RPT + e) * kScThreads + threadIdx.x] = pos[e] >= 0 ? A.pcol[k * A.npad + pos[e]] : (uint16_t)0;
+    }
+  }
+  const int ab = A.ab[W], zb = A.zb[W];
+  const int aends = lane < A.passes ? A.ae[W * A.passes + lane] : 0;
+  const int zends = lane < A.passes ? A.ze[W * A.passes + lane] : 0;
+  const int atot = __shfl_sync(0xffffffffu, aends, A.passes - 1), ztot = __shfl_sync(0xffffffffu, zends, A.passes - 1);
+  // every CTA's copy of this thread's values
+  auto push = [&](const float(&v)[RPT]) {
+#pragma unroll 1
+    for (int k = 0; k < S.nb; ++k) {
+      int r = S.rank + k;
+      if (r >= S.nb) r -= S.nb;
+      const uint32_t d = sc_mapa(Xa, r);
+#pragma unroll
+      for (int e = 0; e < RPT; ++e)
+        if (pos[e] >= 0) sc_st(d + 4 * pos[e], v[e]);
+    }
+  };
+  const int msk = A.L - 1;
+  double x[RPT], r64[RPT], b[RPT];
+#pragma unroll
+  for (int e = 0; e < RPT; ++e) {
+    x[e] = b[e] = 0.0;
+    if (row[e] < 0) continue;
+    b[e] = A.b[row[e]];
+    if (A.warm) {  // cubic extrapolation of the last four currents (zero before step 0)
+      const double* J = A.ring + (int64_t)row[e] * A.L;
+      const int s = A.alpha - 2;
+      const double j1 = s >= 0 ? J[s & msk] : 0.0, j2 = s >= 1 ? J[(s - 1) & msk] : 0.0;
+      const double j3 = s >= 2 ? J[(s - 2) & msk] : 0.0, j4 = s >= 3 ? J[(s - 3) & msk] : 0.0;
+      x[e] = 4.0 * j1 - 6.0 * j2 + 4.0 * j3 - j4;
+    }
+  }
+  // r = b - Z0 y in FP64, y published through w (a barrier before it is read)
+  auto residual = [&](const double(&y)[RPT], double* w, double(&r)[RPT]) {
+#pragma unroll
+    for (int e = 0; e < RPT; ++e)
+      if (pos[e] >= 0) w[pos[e]] = y[e];
+    S.sync();
+    sc_spmv<RPT>(LdZ64{A.zval, A.zcol, w}, zb, ztot, zends, lane, r);
+#pragma unroll
+    for (int e = 0; e < RPT; ++e) r[e] = row[e] >= 0 ? b[e] - r[e] : 0.0;
+  };
+  auto norm2 = [&](const double(&r)[RPT], double& rr, double& bb) {
+    rr = bb = 0.0;
+#pragma unroll
+    for (int e = 0; e < RPT; ++e) {
+      rr += r[e] * r[e];
+      bb += b[e] * b[e];
+    }
+    S.sums64(rr, bb);
+  };
+  double rr = 0.0, bb = 0.0;
+  int inner_total = 0;
+  bool conv = false;
+  // The start: the extrapolation; with warm 2 also the caller's guess in A.x,
+  // kept only if its FP64 residual is smaller (a NaN never is).
+#pragma unroll 1
+  for (int outer = -1;; ++outer) {
+    double nr, nbb;
+    if (outer < 0 || !(rr <= 0x1p-16 * bb)) {
+      residual(x, A.w64, r64);
+    } else {
+      // The correction (y: its FP32 digits) is at most about 2^-8 of the iterate:
+      // Z0 d in double-float (46 bits) is then as exact as b - Z0 x anew in FP64.
+      double zd[RPT];
+      sc_spmv<RPT>(LdZdf{A.zhi, A.zlo, A.zcol, sc_X}, zb, ztot, zends, lane, zd);
+      const int kx = max((((__double2hiint(rr) >> 20) & 0x7ff) - 1023) >> 1, -500);
+      const double sc = __hiloint2double((1023 + kx) << 20, 0);
+#pragma unroll
+      for (int e = 0; e < RPT; ++e) r64[e] = row[e] >= 0 ? r64[e] - sc * zd[e] : 0.0;
+    }
+    norm2(r64, nr, nbb);
+    rr = nr;
+    bb = nbb;
+    if (outer < 0 && A.warm == 2) {
+      double g[RPT], rg[RPT], gg, b2;
+#pragma unroll
+      for (int e = 0; e < RPT; ++e) g[e] = row[e] >= 0 ? A.x[row[e]] : 0.0;
+      residual(g, A.w64 + A.npad, rg);
+      norm2(rg, gg, b2);
+      const bool keep = gg < rr;
+      if (keep) {
+        rr = gg;
+#pragma unroll
+        for (int e = 0; e < RPT; ++e) {
+          x[e] = g[e];
+          r64[e] = rg[e];
+        }
+      }
+      if (S.rank == 0 && threadIdx.x == 0) A.status[keep ? 8 : 9] += 1;
+    }
+    const double tol2bb = A.tol * A.tol * bb;
+    if (rr <= tol2bb) {
+      conv = true;
+      break;
+    }
+    if (outer == 7 || inner_total >= A.maxit) break;
+    if (!(rr < 1.7e308)) {  // non-finite data: so is the result
+#pragma unroll
+      for (int e = 0; e < RPT; ++e) x[e] = __longlong_as_double(0x7ff8000000000000LL);
+      break;
+    }
+    // scale 2^k, k the exponent of |r|: the inner right-hand side has norm in [1, 2)
+    const int kx = max((((__double2hiint(rr) >> 20) & 0x7ff) - 1023) >> 1, -500);
+    const double sc = __hiloint2double((1023 + kx) << 20, 0), inv = __hiloint2double((1023 - kx) << 20, 0);
+    // u: r, then s = r - alpha v, of each iteration
+    float u[RPT], rh[RPT], p[RPT], v[RPT], y[RPT], w[RPT], d[4];
+    // inner target: the reduction that brings the FP64 residual to half the outer
+    // tolerance, within [1e-5, 0.5] (1e-5: what FP32 reliably reaches)
+    const float rin = (float)(rr * inv * inv);
+    const float tin2 = fminf(fmaxf(0.25f * (float)(tol2bb * inv * inv) / rin, (float)kScInner2), 0.25f) * rin;
+#pragma unroll
+    for (int e = 0; e < RPT; ++e) {
+      u[e] = rh[e] = p[e] = (float)(r64[e] * inv);
+      v[e] = y[e] = 0.f;
+    }
+    push(p);  // X is free: the barrier of the last sums lies behind every gather
+    S.sync();
+    float rho = 0.f, alp = 1.f;
+    int half = 0, left = kScInnerMax;
+    bool first = true;
+#pragma unroll 1
+    for (;;) {
+      if (half == 0) {
+        if (inner_total >= A.maxit || left-- == 0) break;
+        ++inner_total;
+      }
+      sc_spmv<RPT>(LdA{A.aval, A.acol, sc_X}, ab, atot, aends, lane, w);
+      float q0 = 0.f, q1 = 0.f, q2 = 0.f, q3 = 0.f;
+#pragma unroll
+      for (int e = 0; e < RPT; ++e) {
+        q0 = fmaf(rh[e], w[e], q0);
+        q1 = fmaf(u[e], u[e], q1);
+        q2 = fmaf(u[e], w[e], q2);
+        q3 = fmaf(w[e], w[e], q3);
+      }
+      S.dots4(q0, q1, q2, q3, d);
+      if (half == 0) {
+        if (first) rho = d[1];  // rh = r
+        first = false;
+        if (d[0] == 0.f || rho == 0.f) break;
+        alp = rho / d[0];
+#pragma unroll
+        for (int e = 0; e < RPT; ++e) {
+          v[e] = w[e];
+          y[e] = fmaf(alp, p[e], y[e]);
+          u[e] = fmaf(-alp, w[e], u[e]);
+        }
+        // |s|^2 from the same sums: the half step may end the inner solve
+        if (d[1] - alp * (2.f * d[2] - alp * d[3]) <= tin2) break;
+        push(u);
+      } else {
+        if (d[3] == 0.f) break;
+        const float om = d[2] / d[3];
+        // (rh, s) = 0 by the choice of alpha
+        const float rho_new = -om * d[0], beta = (rho_new / rho) * (alp / om);
+        rho = rho_new;
+#pragma unroll
+        for (int e = 0; e < RPT; ++e) {
+          y[e] = fmaf(om, u[e], y[e]);
+          u[e] = fmaf(-om, w[e], u[e]);
+          p[e] = fmaf(beta, fmaf(-om, v[e], p[e]), u[e]);
+        }
+        if (om == 0.f || d[1] - om * (2.f * d[2] - om * d[3]) <= tin2) break;
+        push(p);
+      }
+      half ^= 1;
+      S.sync();
+    }
+    // d = P y, x += 2^k d; every gather of X lies behind the last sums' barrier
+    push(y);
+    S.sync();
+#pragma unroll
+    for (int e = 0; e < RPT; ++e) {
+      float de = 0.f;
+#pragma unroll
+      for (int k = 0; k < kScPc; ++k) {
+        if constexpr (kPShared) {
+          const int o = (k * RPT + e) * kScThreads + threadIdx.x;
+          de = fmaf(pvs[o], sc_X[pcs[o]], de);
+        } else if (pos[e] >= 0) {
+          de = fmaf(A.pval[k * A.npad + pos[e]], sc_X[A.pcol[k * A.npad + pos[e]]], de);
+        }
+      }
+      y[e] = de;
+      x[e] += sc * (double)de;
+    }
+    if (rr <= 0x1p-16 * bb) {
+      S.sync();  // every CTA has gathered y
+      push(y);
+      S.sync();
+    }
+  }
+#pragma unroll
+  for (int e = 0; e < RPT; ++e)
+    if (row[e] >= 0) {
+      A.x[row[e]] = x[e];
+      A.ring[(int64_t)row[e] * A.L + ((A.alpha - 1) & msk)] = x[e];
+    }
+  if (S.rank == 0 && threadIdx.x == 0) {
+    A.status[0] = inner_total;
+    A.status[6] = 0;
+    A.status[1] = conv ? 1 : 0;
+    A.status[2] += conv ? 0 : 1;
+    A.status[3] += inner_total;
+    A.resid[0] = bb > 0 ? sqrt(rr / bb) : 0.0;
+  }
+  S.sync();  // no CTA leaves while another may still store into its shared memory
+}
+
+struct ScPlan {
+  int cs = 0, gpc = 0, passes = 0, npad = 0;
+  int32_t *perm = nullptr, *ab = nullptr, *ae = nullptr, *zb = nullptr, *ze = nullptr;
+  float4 *aval = nullptr, *zhi = nullptr, *zlo = nullptr;
+  double2* zval = nullptr;
+  uint2 *acol = nullptr, *zcol = nullptr;
+  float* pval = nullptr;
+  uint16_t* pcol = nullptr;
+  double* w64 = nullptr;
+};
+
+}  // namespace tdbem
+
+using namespace tdbem;
+
+using ScFn = void (*)(ScArgs);
+static ScFn sc_fn(int passes) {
+  return passes <= 4 ? k_solve_cluster<1> : passes <= 8 ? k_solve_cluster<2> : passes <= 12 ? k_solve_cluster<3>
+                                                                                       : k_solve_cluster<6>;
+}
+
+static size_t sc_smem(const ScPlan& P) {
+  const int rpt = P.passes <= 12 ? (P.passes + 3) / 4 : 6;
+  return (size_t)P.npad * sizeof(float) + (rpt <= kScPSharedRows ? (size_t)kScPc * rpt * kScThreads * 6 : 0);
+}
+
+static void sc_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* at, int cs, size_t smem, cudaStream_t st) {
+  *cfg = {};
+  cfg->gridDim = dim3(cs);
+  cfg->blockDim = dim3(kScThreads);
+  cfg->dynamicSmemBytes = smem;
+  cfg->stream = st;
+  at->id = cudaLaunchAttributeClusterDimension;
+  at->val.clusterDim.x = cs;
+  at->val.clusterDim.y = 1;
+  at->val.clusterDim.z = 1;
+  cfg->attrs = at;
+  cfg->numAttrs = 1;
+}
+
+// One matrix in blocks of 8 rows x 16 entries along the order `slot` of the
+// groups; put(block * 128 + place, entry) stores an entry.
+template <class Len, class Put>
+static void sc_blocks(const ScPlan& P, const std::vector<int32_t>& perm, Len len, Put put, std::vector<int32_t>* begin,
+                      std::vector<int32_t>* end, int32_t* nblk) {
+  int32_t b = 0;
+  begin->assign(P.cs * kScWarps, 0);
+  end->assign(P.cs * kScWarps * P.passes, 0);
+  for (int k = 0; k < P.cs; ++k)
+    for (int w = 0; w < kScWarps; ++w) {
+      (*begin)[k * kScWarps + w] = b;
+      for (int j = 0; j < P.passes; ++j) {
+        const int g = j * kScWarps + w;
+        if (g < P.gpc) {
+          const int64_t p0 = ((int64_t)k * P.gpc + g) * 8;
+          int most = 1;
+          for (int t = 0; t < 8; ++t)
+            if (perm[p0 + t] >= 0) most = std::max(most, (int)len(perm[p0 + t]));
+          const int nb = (most + 15) / 16;
+          for (int t = 0; t < 8; ++t)
+            if (perm[p0 + t] >= 0)
+              for (int m = 0; m < len(perm[p0 + t]); ++m)
+                put((int64_t)(b + m / 16) * 128 + t * 16 + m % 16, perm[p0 + t], m);
+          b += nb;
+        }
+        if (j == P.passes - 1)  // whole prefetch rounds: zero blocks behind the last group
+          while ((b - (*begin)[k * kScWarps + w]) % kScDepth) ++b;
+        (*end)[(k * kScWarps + w) * P.passes + j] = b;
+      }
+    }
+  *nblk = b + kScDepth;  // loads run ahead of the last warp's end
+}
+
+template <class T>
+static tdbem_status sc_upload(tdbem_ctx* c, T** d, const std::vector<T>& h) {
+  tdbem_status s = c->dalloc(d, h.size());
+  if (s) return s;
+  // on the context's stream and waited for: the host array goes out of scope
+  TDBEM_CUDA_TRY(c, cudaMemcpyAsync(*d, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice, c->stream));
+  TDBEM_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  return TDBEM_OK;
+}
+
+tdbem_status tdbem_sc_build(tdbem_ctx* c, int want, const std::vector<int32_t>& zp, const std::vector<int32_t>& zc,
+                            const std::vector<double>& zv, const std::vector<int32_t>& pcol,
+                            const std::vector<double>& pval) {
+  const int ne = (int)c->ne;
+  ScPlan P;
+  // the largest cluster the device schedules, at most the wanted one
+  for (P.cs = want; P.cs >= 1; P.cs >>= 1) {
+    const int groups = (ne + 7) / 8;
+    P.gpc = (groups + P.cs - 1) / P.cs;
+    P.passes = (P.gpc + kScWarps - 1) / kScWarps;
+    P.npad = P.cs * P.gpc * 8;
+    if (P.passes > kScPasses || P.npad > 65535 || sc_smem(P) > 200 * 1024) return TDBEM_OK;
+    const ScFn fn = sc_fn(P.passes);
+    TDBEM_CUDA_TRY(c, cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    TDBEM_CUDA_TRY(c, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at;
+    sc_config(&cfg, &at, P.cs, sc_smem(P), c->stream);
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) == cudaSuccess && n > 0) break;
+    cudaGetLastError();
+  }
+  if (P.cs < 1) return TDBEM_OK;
+  // A = Z0 P, row by row
+  std::vector<int64_t> ap(ne + 1, 0);
+  std::vector<int32_t> ac, at(ne, -1);
+  std::vector<double> av;
+  ac.reserve(zc.size() * 2);
+  av.reserve(zc.size() * 2);
+  for (int i = 0; i < ne; ++i) {
+    const int64_t r0 = (int64_t)ac.size();
+    for (int k = zp[i]; k < zp[i + 1]; ++k) {
+      const int j = zc[k];
+      for (int m = 0; m < kScPc; ++m) {
+        const double pv = pval[(size_t)m * ne + j];
+        if (pv == 0.0) continue;
+        const int l = pcol[(size_t)m * ne + j];
+        if (at[l] < r0) {
+          at[l] = (int32_t)ac.size();
+          ac.push_back(l);
+          av.push_back(0.0);
+        }
+        av[at[l]] += zv[k] * pv;
+      }
+    }
+    ap[i + 1] = (int64_t)ac.size();
+  }
+  if (ap[ne] >= (1ll << 31)) return TDBEM_OK;
+  // order: rows by their blocks of A, longest first (stable), in groups of 8 dealt over the CTAs
+  std::vector<int32_t> ord(ne);
+  for (int i = 0; i < ne; ++i) ord[i] = i;
+  std::stable_sort(ord.begin(), ord.end(), [&](int32_t a, int32_t b) {
+    return (ap[a + 1] - ap[a] + 15) / 16 > (ap[b + 1] - ap[b] + 15) / 16;
+  });
+  std::vector<int32_t> perm(P.npad, -1), at_pos(ne);
+  int next = 0;
+  for (int j = 0; j < P.passes && next < ne; ++j)
+    for (int u = 0; u < P.cs * kScWarps && next < ne; ++u) {
+      const int f = j & 1 ? P.cs * kScWarps - 1 - u : u;  // there and back: long and short groups meet
+      const int k = f % P.cs, g = j * kScWarps + f / P.cs;
+      if (g >= P.gpc) continue;
+      for (int t = 0; t < 8 && next < ne; ++t, ++next) {
+        const int64_t p = ((int64_t)k * P.gpc + g) * 8 + t;
+        perm[p] = ord[next];
+        at_pos[ord[next]] = (int32_t)p;
+      }
+    }
+  std::vector<int32_t> ab, ae, zb, ze;
+  int32_t na = 0, nz = 0;
+  auto alen = [&](int i) { return (int)(ap[i + 1] - ap[i]); };
+  auto zlen = [&](int i) { return zp[i + 1] - zp[i]; };
+  auto none = [](int64_t, int, int) {};
+  sc_blocks(P, perm, alen, none, &ab, &ae, &na);
+  sc_blocks(P, perm, zlen, none, &zb, &ze, &nz);
+  tdbem_status s;
+  if ((s = sc_upload(c, &P.perm, perm)) || (s = sc_upload(c, &P.ab, ab)) || (s = sc_upload(c, &P.ae, ae)) ||
+      (s = sc_upload(c, &P.zb, zb)) || (s = sc_upload(c, &P.ze, ze)))
+    return s;
+  {
+    std::vector<float4> v((size_t)na * 32, make_float4(0, 0, 0, 0));
+    std::vector<uint2> col((size_t)na * 32, make_uint2(0, 0));
+    float* fv = (float*)v.data();
+    uint16_t* fc = (uint16_t*)col.data();
+    sc_blocks(P, perm, alen, [&](int64_t o, int i, int m) {
+      fv[o] = (float)av[ap[i] + m];
+      fc[o] = (uint16_t)at_pos[ac[ap[i] + m]];
+    }, &ab, &ae, &na);
+    if ((s = sc_upload(c, &P.aval, v)) || (s = sc_upload(c, &P.acol, col))) return s;
+  }
+  {
+    std::vector<double2> v((size_t)nz * 64, make_double2(0, 0));
+    std::vector<float4> hi((size_t)nz * 32, make_float4(0, 0, 0, 0)), lo = hi;
+    std::vector<uint2> col((size_t)nz * 32, make_uint2(0, 0));
+    double* dv = (double*)v.data();
+    float *fh = (float*)hi.data(), *fl = (float*)lo.data();
+    uint16_t* fc = (uint16_t*)col.data();
+    sc_blocks(P, perm, zlen, [&](int64_t o, int i, int m) {
+      const double z = zv[zp[i] + m];
+      dv[o] = z;
+      fh[o] = (float)z;
+      fl[o] = (float)(z - (double)fh[o]);
+      fc[o] = (uint16_t)at_pos[zc[zp[i] + m]];
+    }, &zb, &ze, &nz);
+    if ((s = sc_upload(c, &P.zval, v)) || (s = sc_upload(c, &P.zhi, hi)) || (s = sc_upload(c, &P.zlo, lo)) ||
+        (s = sc_upload(c, &P.zcol, col)))
+      return s;
+  }
+  {
+    std::vector<float> pv((size_t)kScPc * P.npad, 0.f);
+    std::vector<uint16_t> pc((size_t)kScPc * P.npad, 0);
+    for (int m = 0; m < kScPc; ++m)
+      for (int i = 0; i < ne; ++i) {
+        pv[(size_t)m * P.npad + at_pos[i]] = (float)pval[(size_t)m * ne + i];
+        pc[(size_t)m * P.npad + at_pos[i]] = (uint16_t)at_pos[pcol[(size_t)m * ne + i]];
+      }
+    if ((s = sc_upload(c, &P.pval, pv)) || (s = sc_upload(c, &P.pcol, pc)) || (s = c->dalloc(&P.w64, 2 * (size_t)P.npad)))
+      return s;
+  }
+  TDBEM_CUDA_TRY(c, cudaMemsetAsync(P.w64, 0, 2 * (size_t)P.npad * sizeof(double), c->stream));
+  c->sc = new (std::nothrow) ScPlan(P);
+  return c->sc ? TDBEM_OK : TDBEM_ENOMEM;
+}
+
+tdbem_status tdbem_sc_solve(tdbem_ctx* c, int32_t alpha, int32_t warm) {
+  const ScPlan& P = *c->sc;
+  ScArgs A;
+  A.perm = P.perm;
+  A.ab = P.ab;
+  A.ae = P.ae;
+  A.aval = P.aval;
+  A.acol = P.acol;
+  A.zb = P.zb;
+  A.ze = P.ze;
+  A.zval = P.zval;
+  A.zhi = P.zhi;
+  A.zlo = P.zlo;
+  A.zcol = P.zcol;
+  A.pval = P.pval;
+  A.pcol = P.pcol;
+  A.w64 = P.w64;
+  A.b = c->d_R;
+  A.x = c->d_J;
+  A.ring = c->d_Jring;
+  A.L = c->L;
+  A.alpha = alpha;
+  A.warm = warm;
+  A.gpc = P.gpc;
+  A.passes = P.passes;
+  A.npad = P.npad;
+  A.ne = (int32_t)c->ne;
+  A.maxit = c->p.solve_maxit;
+  A.tol = c->p.solve_tol;
+  A.status = c->d_status;
+  A.resid = c->d_dots;
+  c->cluster = P.cs;
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute at;
+  sc_config(&cfg, &at, P.cs, sc_smem(P), c->stream);
+  TDBEM_CUDA_TRY(c, cudaLaunchKernelEx(&cfg, sc_fn(P.passes), A));
+  return TDBEM_OK;
+}
+
+void tdbem_sc_free(tdbem_ctx* c) {
+  delete c->sc;
+  c->sc = nullptr;
+}
