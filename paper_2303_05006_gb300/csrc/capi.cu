@@ -766,6 +766,7 @@ tdbem_status tdbem_reset(tdbem_ctx* c) {
   if (s0) return s0;
   const int64_t NR = c->ne * (int64_t)c->R;
   TDBEM_CUDA_TRY(c, cudaMemsetAsync(c->d_Jring, 0, NR * c->L * sizeof(double), c->stream));
+  if (c->d_rs) TDBEM_CUDA_TRY(c, cudaMemsetAsync(c->d_rs, 0, NR * c->L * sizeof(float2), c->stream));
   TDBEM_CUDA_TRY(c, cudaMemsetAsync(c->d_J, 0, NR * sizeof(double), c->stream));
   TDBEM_CUDA_TRY(c, cudaMemsetAsync(c->d_status, 0, 16 * sizeof(int32_t), c->stream));
   if (c->p.mode == TDBEM_FAST) {
@@ -863,8 +864,9 @@ tdbem_status tdbem_load(tdbem_ctx* c, const char* path) {
   }
   // every size checked: now overwrite the state
   for (size_t k = 0; k < bufs.size(); ++k)
-    TDBEM_CUDA_TRY(c, cudaMemcpy(bufs[k].first, host[k].data(), host[k].size(), cudaMemcpyHostToDevice));
+    TDBEM_CUDA_TRY(c, cudaMemcpyAsync(bufs[k].first, host[k].data(), host[k].size(), cudaMemcpyHostToDevice, c->stream));
   TDBEM_CUDA_TRY(c, cudaMemsetAsync(c->d_status, 0, 16 * sizeof(int32_t), c->stream));
+  if ((s = tdbem_direct_resplit(c))) return s;
   TDBEM_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   c->alpha = h.alpha;
   return TDBEM_OK;

@@ -61,6 +61,12 @@ struct PairStore {
   double* val = nullptr;    // [nval]; direct mode with one right-hand side: (hi, lo) FP32 pairs after setup
 };
 
+// an FP64 value as an unevaluated sum of two FP32 numbers, |lo| <= ulp(hi) / 2
+__device__ __forceinline__ float2 split_pair(double v) {
+  const float h = __double2float_rn(v);
+  return make_float2(h, __double2float_rn(v - (double)h));
+}
+
 struct FmmPlan;
 struct ScPlan;
 
@@ -111,26 +117,47 @@ struct tdbem_ctx {
   int32_t L = 0;                    // ring length (power of two)
   double* d_Jring = nullptr;        // [ne][L][R]
   float2* d_ring2 = nullptr;        // direct mode, R = 1: split history [L][ne] (hi, lo) (untiled kernel)
-  // direct mode, R = 1, tiled history sum (lags >= 3) plus the lag-2 entries in the reduction
-  double* d_dpart = nullptr;        // partial sums [3][ncb][ne]: march steps alpha & 1, evaluations 2
   // direct mode, R = 1, row-tile store of the lags >= 3 (rows in tiles of 32,
-  // one lane per row; see k_direct_history_rt)
-  int32_t rt_prec = 0;              // 0: untiled (ring > 128 steps), 1: FP32 values, 2: (hi, lo) pairs, 3: 24-bit
+  // one lane per row; see k_direct_history_rt): the far pairs by column blocks,
+  // rt_B steps per pass, and the near pairs as a list, plus the lag-2 entries in
+  // the reduction
+  int32_t rt_prec = 0;              // 0: untiled, 1: FP32 values, 2: (hi, lo) pairs, 3: 24-bit
+  int32_t rt_B = 1;                 // steps per pass of the far pairs
+  int32_t rt_nrt = 0;               // row tiles
+  int32_t* d_rt_row = nullptr;      // [nrt * 32] row at a position (-1: padding)
   unsigned char* d_rt_val = nullptr;  // [groups] of 32 values (128, 256 or 96 bytes)
   uint32_t* d_rt_goff = nullptr;    // [nrt * ne + 1] first group of (tile, column)
-  uint8_t* d_rt_lo = nullptr;       // [nrt * ne][32] first stored lag (>= 3) of (row, column)
-  int32_t rt_Lh = 0;                // history rows staged per column (every lag a group reaches)
-  int32_t rt_ncb = 0, rt_nrg = 0;   // column blocks and row-tile groups of its grid
-  int32_t rt_tiles = 0;             // row tiles per block
-  int64_t rt_bytes = 0;             // bytes streamed per launch (values, lag bytes, group offsets)
+  uint8_t* d_rt_lo = nullptr;       // [nrt * ne][32] first stored lag of (row, column)
+  int32_t rt_Lh = 0;                // lags a far group reaches
+  int32_t rt_ncb = 0, rt_cbw = 0;   // column blocks of its grid, columns per block
+  int32_t* d_rt_list = nullptr;     // row tiles of the launches: far parts 0 .. B - 1, then the near units, by column block
+  int32_t* d_rt_loff = nullptr;     // [(B + 1) * ncb + 1] their starts
+  int32_t rt_lmost[9] = {}, rt_ltiles[9] = {};  // most tiles of a column block; tiles per block of threads
+  int32_t rt_units = 0;             // tiers by whole (tile, column block) units of one store, columns in edge order
+  int64_t rt_bytes = 0;             // bytes streamed per step (values, lag bytes, group offsets)
+  int32_t* d_rt_lomin = nullptr;    // [nrt][ncb] smallest far lag of (tile, column block)
+  unsigned char* d_nt_val = nullptr;  // near pairs: groups of the quads (8 rows x 4 columns)
+  uint32_t* d_nt_qoff = nullptr;    // first group of a quad
+  uint32_t* d_nt_meta = nullptr;    // [quads][32] column | first lag << 24
+  int4* d_nt_chunk = nullptr;       // [rt_nchunk] {sub-tile, first quad, end, partial slot}
+  int32_t rt_nchunk = 0, rt_nslot = 0;
+  double* d_dpart = nullptr;        // near partial sums [3][rt_nslot][nrt * 32]: march steps alpha & 1, evaluations 2
+  double* d_fpart = nullptr;        // far partial sums [2][rt_B][ncb][nrt * 32], then [ncb][nrt * 32] of evaluations
+  float2* d_rs = nullptr;           // [ne][L] the ring's values as (hi, lo) pairs, kept up to date by the solve
+  float2* d_rs_eval = nullptr;      // the same for evaluations of another history
+  int32_t far_blk[2] = {0, 0};      // first step of the block whose far sums buffer b holds (0: none)
+  int32_t far_done[2] = {0, 0};     // its parts (row-tile ranges) launched, one bit each
+  bool far_wait[2] = {false, false};  // launched on the side stream, not yet waited for
+  cudaEvent_t ev_far[2] = {nullptr, nullptr};
   int32_t* d_dt_err = nullptr;      // set by a bounded wait of the history sum that expired
-  int64_t* d_l2_ptr = nullptr;      // lag-2 coefficients, CSR over rows [ne + 1]
+  double* d_pre = nullptr;          // [3][8][nrt * 32] a position's sums of partials: march steps alpha & 1, evaluations 2
+  int32_t* d_l2_ptr = nullptr;      // lag-2 coefficients, CSR over the positions [nrt * 32 + 1]
   int32_t* d_l2_col = nullptr;
   double* d_l2_val = nullptr;
-  cudaStream_t dstream = nullptr;   // far_overlap: the lags >= 3 of step alpha + 2 run here during step alpha + 1
+  cudaStream_t dstream = nullptr;   // far_overlap: the lags >= 3 of later steps are summed here beside step alpha + 1
   cudaEvent_t ev_dsolved = nullptr;
   cudaEvent_t ev_dahead[2] = {nullptr, nullptr};
-  int32_t dahead[2] = {0, 0};       // step whose lags >= 3 sit in partial buffer b (0: none)
+  int32_t dahead[2] = {0, 0};       // step whose near pairs sit in partial buffer b (0: none)
   double* d_R = nullptr;            // [ne][R]
   double* d_J = nullptr;            // [ne][R] current solution
   double* d_Vall = nullptr;         // [Nt-1][ne][R] or null
@@ -214,6 +241,7 @@ tdbem_status tdbem_build_direct(tdbem_ctx* c);
 tdbem_status tdbem_direct_history(tdbem_ctx* c, int32_t alpha, const double* d_ring, const double* V);
 tdbem_status tdbem_direct_split(tdbem_ctx* c);
 tdbem_status tdbem_direct_after_solve(tdbem_ctx* c, int32_t alpha);
+tdbem_status tdbem_direct_resplit(tdbem_ctx* c);  // the split history anew from the ring
 tdbem_status tdbem_direct_join(tdbem_ctx* c);
 tdbem_status tdbem_direct_check(tdbem_ctx* c);
 tdbem_status tdbem_direct_invalidate(tdbem_ctx* c);

@@ -99,6 +99,7 @@ struct SolveArgs {
   const double* b;
   double* x;        // solution (also written to the ring)
   double* ring;     // [ne][L]
+  float2* rs;       // the ring's values as (hi, lo) pairs (may be null)
   int32_t L;
   int32_t alpha;    // solving J^{alpha-1}
   int32_t warm;     // 1: cubic extrapolation of J^{alpha-2..alpha-5}; 2: x holds another guess,
@@ -471,7 +472,11 @@ __device__ __forceinline__ void bicgstab_body(const SolveArgs& A, Sync& cl, doub
     for (int64_t i = r0 + threadIdx.x; i < r1; i += blockDim.x) A.x[i] += sc * (double)d[i];
     cl.sync();
   }
-  for (int64_t i = r0 + threadIdx.x; i < r1; i += blockDim.x) A.ring[i * L + ((A.alpha - 1) & msk)] = A.x[i];
+  for (int64_t i = r0 + threadIdx.x; i < r1; i += blockDim.x) {
+    const int64_t o = i * L + ((A.alpha - 1) & msk);
+    A.ring[o] = A.x[i];
+    if (A.rs) A.rs[o] = split_pair(A.x[i]);
+  }
   if (rk == 0 && threadIdx.x == 0) {
     A.status[0] = inner_total;
     A.status[6] = sweeps;
@@ -1040,7 +1045,12 @@ static tdbem_status tdbem_z0_f32(tdbem_ctx* c) {
       pval[i] = d != 0.0 ? 1.0 / d : 1.0;
     }
   }
-  if (c->R > 1 || c->p.jacobi_sweeps > 0 || use_grid(c)) return TDBEM_OK;
+  // The FP32 and 24-bit stores' marches round every current to FP32 in the next
+  // steps' sums, so they carry any difference in the solve's rounding on at the level
+  // of the store's own rounding (1e-8 after 80 steps on the 7680-RWG sphere, from
+  // 1e-13): they keep k_bicgstab and with it their currents.
+  const bool f32 = c->p.mode == TDBEM_DIRECT && c->p.p2p_prec != TDBEM_P_FP64;
+  if (c->R > 1 || c->p.jacobi_sweeps > 0 || f32 || use_grid(c)) return TDBEM_OK;
   return tdbem_sc_build(c, c->p.solve_cluster > 0 ? c->p.solve_cluster : 16, hp, hc, hv, pcol, pval);
 }
 
@@ -1245,6 +1255,7 @@ tdbem_status tdbem_solve_z0(tdbem_ctx* c, int32_t alpha, int32_t* iters, int32_t
     A.b = c->d_R;
     A.x = c->d_J;
     A.ring = c->d_Jring;
+    A.rs = c->d_rs;
     A.L = c->L;
     A.alpha = alpha;
     A.warm = warm;
@@ -1262,18 +1273,7 @@ tdbem_status tdbem_solve_z0(tdbem_ctx* c, int32_t alpha, int32_t* iters, int32_t
       TDBEM_CUDA_TRY(c, cudaLaunchCooperativeKernel((void*)k_bicgstab_grid, dim3(g_grid), dim3(kSolveThreads), args,
                                                     0, c->stream));
     } else {
-      // Default: the largest cluster, except in the pipelined direct march with
-      // a history sum streaming at least 3 GB per step (about 0.5 ms).  There
-      // the solve overlaps that sum on its own SMs, and a cluster of 4 leaves
-      // 12 more SMs to it while the solve still hides behind it (7680-RWG
-      // sphere, (hi, lo) store of 4.6 GB: 1145 steps/s against 1106 with 16).
-      // A shorter sum (the FP32 store's 2.3 GB) leaves the solve on the
-      // critical path, where 16 CTAs win (2160 steps/s against 1855 with 4).
-      int cs = g_cluster;
-      if (c->p.solve_cluster > 0)
-        cs = std::min(c->p.solve_cluster, g_cluster);
-      else if (c->p.mode == TDBEM_DIRECT && c->p.far_overlap && c->rt_bytes >= (3LL << 30))
-        cs = std::min(4, g_cluster);
+      const int cs = c->p.solve_cluster > 0 ? std::min(c->p.solve_cluster, g_cluster) : g_cluster;
       c->cluster = cs;
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(cs);

@@ -59,6 +59,7 @@ struct ScArgs {
   const double* b;           // rows in edge order from here on
   double* x;
   double* ring;
+  float2* rs;                // the ring's values as (hi, lo) pairs (may be null)
   int32_t L, alpha, warm, gpc, passes, npad, ne, maxit;
   double tol;
   int32_t* status;           // as in SolveArgs (solve.cu)
@@ -603,7 +604,9 @@ __global__ void __launch_bounds__(kScThreads) k_solve_cluster(const ScArgs A) {
   for (int e = 0; e < RPT; ++e)
     if (row[e] >= 0) {
       A.x[row[e]] = x[e];
-      A.ring[(int64_t)row[e] * A.L + ((A.alpha - 1) & msk)] = x[e];
+      const int64_t o = (int64_t)row[e] * A.L + ((A.alpha - 1) & msk);
+      A.ring[o] = x[e];
+      if (A.rs) A.rs[o] = split_pair(x[e]);
     }
   if (S.rank == 0 && threadIdx.x == 0) {
     A.status[0] = inner_total;
@@ -842,6 +845,7 @@ tdbem_status tdbem_sc_solve(tdbem_ctx* c, int32_t alpha, int32_t warm) {
   A.b = c->d_R;
   A.x = c->d_J;
   A.ring = c->d_Jring;
+  A.rs = c->d_rs;
   A.L = c->L;
   A.alpha = alpha;
   A.warm = warm;
