@@ -300,12 +300,10 @@ void tdbem_mlp_free(tdbem_ctx* c);
 tdbem_status tdbem_build_z0(tdbem_ctx* c);
 tdbem_status tdbem_build_z0_csr(tdbem_ctx* c);
 tdbem_status tdbem_solve_z0(tdbem_ctx* c, int32_t alpha, int32_t* iters, int32_t warm);
-// solve_cluster.cu: the cluster solve of one right-hand side for a Z0 given in
-// CSR (host) and a preconditioner in ELL ([5][ne], FP64); want: CTAs of the
-// cluster at most.  No plan is made (c->sc stays null) where the mesh does not
-// fit it.
+// solve_cluster.cu: the cluster solve of one right-hand side for the context's Z0
+// (CSR on the device, and here on the host); want: CTAs of the cluster at most.
+// No plan is made (c->sc stays null) where the mesh does not fit it.
 tdbem_status tdbem_sc_build(tdbem_ctx* c, int want, const std::vector<int32_t>& zp, const std::vector<int32_t>& zc,
-                            const std::vector<double>& zv, const std::vector<int32_t>& pcol,
-                            const std::vector<double>& pval);
+                            const std::vector<double>& zv);
 tdbem_status tdbem_sc_solve(tdbem_ctx* c, int32_t alpha, int32_t warm);
 void tdbem_sc_free(tdbem_ctx* c);

@@ -951,14 +951,15 @@ static bool use_grid(const tdbem_ctx* c) {
 // triangles (at most kPc entries).  A triangle whose block is singular adds
 // its diagonal reciprocals instead.
 static tdbem_status build_triangle_precond(tdbem_ctx* c, const std::vector<int32_t>& hp, const std::vector<int32_t>& hc,
-                                           const std::vector<double>& hv, std::vector<int32_t>& pcol,
-                                           std::vector<double>& pval) {
+                                           const std::vector<double>& hv) {
   const int64_t ne = c->ne;
   auto z = [&](int32_t i, int32_t j) {
     for (int32_t k = hp[i]; k < hp[i + 1]; ++k)
       if (hc[k] == j) return hv[k];
     return 0.0;
   };
+  std::vector<int32_t> pcol(kPc * ne, 0);
+  std::vector<double> pval(kPc * ne, 0.0);
   std::vector<int> used(ne, 0);
   auto add = [&](int32_t i, int32_t j, double v) {
     for (int k = 0; k < used[i]; ++k)
@@ -1027,31 +1028,20 @@ static tdbem_status tdbem_z0_f32(tdbem_ctx* c) {
                                                                        c->d_ell_val32);
   TDBEM_CUDA_TRY(c, cudaGetLastError());
   TDBEM_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  const int64_t ne = c->ne, nnz = hp[ne];
+  const int64_t nnz = hp[c->ne];
   std::vector<int32_t> hc(nnz);
   std::vector<double> hv(nnz);
   TDBEM_CUDA_TRY(c, cudaMemcpy(hc.data(), c->d_z0_col, nnz * sizeof(int32_t), cudaMemcpyDeviceToHost));
   TDBEM_CUDA_TRY(c, cudaMemcpy(hv.data(), c->d_z0_val, nnz * sizeof(double), cudaMemcpyDeviceToHost));
-  std::vector<int32_t> pcol(kPc * ne, 0);
-  std::vector<double> pval(kPc * ne, 0.0);
-  if (c->p.precond == 1) {
-    if ((s = build_triangle_precond(c, hp, hc, hv, pcol, pval))) return s;
-  } else {
-    for (int64_t i = 0; i < ne; ++i) {
-      double d = 0.0;
-      for (int32_t k = hp[i]; k < hp[i + 1]; ++k)
-        if (hc[k] == i) d = hv[k];
-      pcol[i] = (int32_t)i;
-      pval[i] = d != 0.0 ? 1.0 / d : 1.0;
-    }
-  }
   // The FP32 and 24-bit stores' marches round every current to FP32 in the next
   // steps' sums, so they carry any difference in the solve's rounding on at the level
   // of the store's own rounding (1e-8 after 80 steps on the 7680-RWG sphere, from
   // 1e-13): they keep k_bicgstab and with it their currents.
   const bool f32 = c->p.mode == TDBEM_DIRECT && c->p.p2p_prec != TDBEM_P_FP64;
-  if (c->R > 1 || c->p.jacobi_sweeps > 0 || f32 || use_grid(c)) return TDBEM_OK;
-  return tdbem_sc_build(c, c->p.solve_cluster > 0 ? c->p.solve_cluster : 16, hp, hc, hv, pcol, pval);
+  if (c->R == 1 && c->p.jacobi_sweeps == 0 && !f32 && !use_grid(c)) {
+    if ((s = tdbem_sc_build(c, c->p.solve_cluster > 0 ? c->p.solve_cluster : 16, hp, hc, hv)) || c->sc) return s;
+  }
+  return c->p.precond == 1 ? build_triangle_precond(c, hp, hc, hv) : TDBEM_OK;
 }
 
 tdbem_status tdbem_build_z0(tdbem_ctx* c) {

@@ -3,8 +3,15 @@
 // vector kept whole in every CTA's shared memory.
 //
 // Scheme.  Iterative refinement: an FP64 residual r = b - Z0 x around an FP32
-// BiCGStab on the right-preconditioned matrix A = Z0 P (P: triangle blocks or
-// the diagonal), which is formed once at setup.  The Krylov vectors live in
+// BiCGStab on the right-preconditioned matrix A = Z0 P, which is formed once at
+// setup.  Row i of P is row i of the inverse of the block of Z0 among edge i and
+// its kScK - 1 strongest couplings (k_local_inverse), or the diagonal's inverse.
+// Against the triangle blocks used before, 32 couplings take a third of the
+// iterations (to 1e-5: 7680-RWG sphere 3 to 1, cone-capped cylinder 14.5 to 3.5,
+// octahedral ellipsoid 12.5 to 4.5, UV ellipsoid 44.5 to 10.5), and A has about as
+// many entries, as it is close to the identity: entries below 1e-6 are left out
+// (they would change a correction by less than the 1e-5 it is computed to; the
+// FP64 residual decides).  The Krylov vectors live in
 // registers, each thread owning kScRows rows; only the vector that the next
 // product gathers from travels: every owner stores its values into all CTAs'
 // copies through distributed shared memory, so the gathers are shared-memory
@@ -27,6 +34,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <cmath>
 #include <new>
 #include <vector>
 
@@ -37,10 +45,10 @@ namespace cg = cooperative_groups;
 namespace tdbem {
 
 constexpr int kScThreads = 512, kScWarps = kScThreads / 32;
-constexpr int kScPc = 5;            // entries per row of P
+constexpr int kScK = 32;            // entries per row of P at most
+constexpr double kScDrop = 1e-6;    // entries of A left out (A is close to the identity)
 constexpr int kScPasses = 24;       // groups per warp at most: 6 rows per thread
 constexpr double kScInner2 = 1e-10; // squared relative residual an inner solve stops at
-constexpr int kScPSharedRows = 2;   // rows per thread up to which P is staged in shared memory
 constexpr int kScDepth = 4;          // blocks a warp keeps in flight
 constexpr int kScInnerMax = 80;     // iterations of one inner solve
 
@@ -53,8 +61,9 @@ struct ScArgs {
   const double2* zval;       // [blocks][32][2]
   const float4 *zhi, *zlo;   // Z0 as (hi, lo) pairs
   const uint2* zcol;
-  const float* pval;         // P: [kScPc][npad]
-  const uint16_t* pcol;
+  const int32_t *pb, *pe;    // P, as A
+  const float4* pval;
+  const uint2* pcol;
   double* w64;               // [2][npad] iterates as the residual gathers them
   const double* b;           // rows in edge order from here on
   double* x;
@@ -390,10 +399,6 @@ __global__ void __launch_bounds__(kScThreads) k_solve_cluster(const ScArgs A) {
   S.phase = 0;
   const int lane = S.lane, q = lane & 3, W = S.rank * kScWarps + S.warp;
   const uint32_t Xa = (uint32_t)__cvta_generic_to_shared(sc_X);
-  // P of this thread's rows, and Z0's and A's runs of this warp
-  float* pvs = sc_X + A.npad;  // [kScPc][RPT][threads]
-  uint16_t* pcs = reinterpret_cast<uint16_t*>(pvs + kScPc * RPT * kScThreads);
-  constexpr bool kPShared = RPT <= kScPSharedRows;
   // this thread's rows: position and edge of each (-1: none)
   int pos[RPT], row[RPT];
 #pragma unroll
@@ -401,16 +406,12 @@ __global__ void __launch_bounds__(kScThreads) k_solve_cluster(const ScArgs A) {
     const int g = (4 * e + q) * kScWarps + S.warp;
     pos[e] = g < A.gpc ? (S.rank * A.gpc + g) * 8 + (lane >> 2) : -1;
     row[e] = pos[e] >= 0 ? A.perm[pos[e]] : -1;
-    if constexpr (kPShared)
-#pragma unroll
-    for (int k = 0; k < kScPc; ++k) {
-      pvs[(k * RPT + e) * kScThreads + threadIdx.x] = pos[e] >= 0 ? A.pval[k * A.npad + pos[e]] : 0.f;
-      pcs[(k * RPT + e) * kScThreads + threadIdx.x] = pos[e] >= 0 ? A.pcol[k * A.npad + pos[e]] : (uint16_t)0;
-    }
   }
-  const int ab = A.ab[W], zb = A.zb[W];
+  const int ab = A.ab[W], zb = A.zb[W], pb = A.pb[W];
   const int aends = lane < A.passes ? A.ae[W * A.passes + lane] : 0;
   const int zends = lane < A.passes ? A.ze[W * A.passes + lane] : 0;
+  const int pends = lane < A.passes ? A.pe[W * A.passes + lane] : 0;
+  const int ptot = __shfl_sync(0xffffffffu, pends, A.passes - 1);
   const int atot = __shfl_sync(0xffffffffu, aends, A.passes - 1), ztot = __shfl_sync(0xffffffffu, zends, A.passes - 1);
   // every CTA's copy of this thread's values
   auto push = [&](const float(&v)[RPT]) {
@@ -579,21 +580,9 @@ __global__ void __launch_bounds__(kScThreads) k_solve_cluster(const ScArgs A) {
     // d = P y, x += 2^k d; every gather of X lies behind the last sums' barrier
     push(y);
     S.sync();
+    sc_spmv<RPT>(LdA{A.pval, A.pcol, sc_X}, pb, ptot, pends, lane, y);
 #pragma unroll
-    for (int e = 0; e < RPT; ++e) {
-      float de = 0.f;
-#pragma unroll
-      for (int k = 0; k < kScPc; ++k) {
-        if constexpr (kPShared) {
-          const int o = (k * RPT + e) * kScThreads + threadIdx.x;
-          de = fmaf(pvs[o], sc_X[pcs[o]], de);
-        } else if (pos[e] >= 0) {
-          de = fmaf(A.pval[k * A.npad + pos[e]], sc_X[A.pcol[k * A.npad + pos[e]]], de);
-        }
-      }
-      y[e] = de;
-      x[e] += sc * (double)de;
-    }
+    for (int e = 0; e < RPT; ++e) x[e] += sc * (double)y[e];
     if (rr <= 0x1p-16 * bb) {
       S.sync();  // every CTA has gathered y
       push(y);
@@ -621,12 +610,10 @@ __global__ void __launch_bounds__(kScThreads) k_solve_cluster(const ScArgs A) {
 
 struct ScPlan {
   int cs = 0, gpc = 0, passes = 0, npad = 0;
-  int32_t *perm = nullptr, *ab = nullptr, *ae = nullptr, *zb = nullptr, *ze = nullptr;
-  float4 *aval = nullptr, *zhi = nullptr, *zlo = nullptr;
+  int32_t *perm = nullptr, *ab = nullptr, *ae = nullptr, *zb = nullptr, *ze = nullptr, *pb = nullptr, *pe = nullptr;
+  float4 *aval = nullptr, *zhi = nullptr, *zlo = nullptr, *pval = nullptr;
   double2* zval = nullptr;
-  uint2 *acol = nullptr, *zcol = nullptr;
-  float* pval = nullptr;
-  uint16_t* pcol = nullptr;
+  uint2 *acol = nullptr, *zcol = nullptr, *pcol = nullptr;
   double* w64 = nullptr;
 };
 
@@ -636,14 +623,10 @@ using namespace tdbem;
 
 using ScFn = void (*)(ScArgs);
 static ScFn sc_fn(int passes) {
-  return passes <= 4 ? k_solve_cluster<1> : passes <= 8 ? k_solve_cluster<2> : passes <= 12 ? k_solve_cluster<3>
-                                                                                       : k_solve_cluster<6>;
+  return passes <= 4 ? k_solve_cluster<1> : passes <= 8 ? k_solve_cluster<2> : k_solve_cluster<6>;
 }
 
-static size_t sc_smem(const ScPlan& P) {
-  const int rpt = P.passes <= 12 ? (P.passes + 3) / 4 : 6;
-  return (size_t)P.npad * sizeof(float) + (rpt <= kScPSharedRows ? (size_t)kScPc * rpt * kScThreads * 6 : 0);
-}
+static size_t sc_smem(const ScPlan& P) { return (size_t)P.npad * sizeof(float); }
 
 static void sc_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* at, int cs, size_t smem, cudaStream_t st) {
   *cfg = {};
@@ -702,9 +685,147 @@ static tdbem_status sc_upload(tdbem_ctx* c, T** d, const std::vector<T>& h) {
   return TDBEM_OK;
 }
 
+// A CSR matrix in blocks of the plan's order: FP32 values (and, with lo, the low
+// parts of (hi, lo) pairs; with f64, the FP64 values), positions, block runs.
+struct ScMat {
+  const std::vector<int64_t>& ptr;
+  const std::vector<int32_t>& col;
+  const std::vector<double>& val;
+};
+static tdbem_status sc_matrix(tdbem_ctx* c, const ScPlan& P, const std::vector<int32_t>& perm,
+                              const std::vector<int32_t>& at, const ScMat& M, int32_t** begin, int32_t** end,
+                              float4** hi, float4** lo, double2** f64, uint2** col) {
+  std::vector<int32_t> b, e;
+  int32_t n = 0;
+  auto len = [&](int i) { return (int)(M.ptr[i + 1] - M.ptr[i]); };
+  sc_blocks(P, perm, len, [](int64_t, int, int) {}, &b, &e, &n);
+  std::vector<float4> vh((size_t)n * 32, make_float4(0, 0, 0, 0)), vl(lo ? (size_t)n * 32 : 0, make_float4(0, 0, 0, 0));
+  std::vector<double2> vd(f64 ? (size_t)n * 64 : 0, make_double2(0, 0));
+  std::vector<uint2> vc((size_t)n * 32, make_uint2(0, 0));
+  float *fh = (float*)vh.data(), *fl = (float*)vl.data();
+  double* fd = (double*)vd.data();
+  uint16_t* fc = (uint16_t*)vc.data();
+  sc_blocks(P, perm, len, [&](int64_t o, int i, int m) {
+    const double z = M.val[M.ptr[i] + m];
+    fh[o] = (float)z;
+    if (lo) fl[o] = (float)(z - (double)fh[o]);
+    if (f64) fd[o] = z;
+    fc[o] = (uint16_t)at[M.col[M.ptr[i] + m]];
+  }, &b, &e, &n);
+  tdbem_status s;
+  if ((s = sc_upload(c, begin, b)) || (s = sc_upload(c, end, e)) || (s = sc_upload(c, hi, vh)) ||
+      (s = sc_upload(c, col, vc)) || (lo && (s = sc_upload(c, lo, vl))) || (f64 && (s = sc_upload(c, f64, vd))))
+    return s;
+  return TDBEM_OK;
+}
+
+// Row i of P: row 0 of the inverse of the block of Z0 among J = {i, then the
+// columns of row i's largest entries}, at most kScK in all; the solution of
+// B^T y = e_0 by Gauss-Jordan elimination with partial pivoting in FP32, lane r
+// holding row r of B^T.  A block without a usable pivot gives the reciprocal of
+// the diagonal.  One warp per row.
+constexpr int kLiWarps = 8;
+
+__global__ void __launch_bounds__(kLiWarps * 32) k_local_inverse(const int32_t* ptr, const int32_t* col,
+                                                                const double* val, int32_t ne, int32_t* pcol,
+                                                                float* pval) {
+  __shared__ float Bs[kLiWarps][32][33];
+  __shared__ int Js[kLiWarps][32];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int i = blockIdx.x * kLiWarps + w;
+  if (i >= ne) return;  // whole warps; only warp-wide synchronisation below
+  const int p0 = ptr[i], p1 = ptr[i + 1];
+  // the largest entries, one after the other: each round takes the largest below the last taken
+  // (ties: the smaller index first)
+  int n = 1, myj = lane == 0 ? i : -1, last = -1;
+  float lastv = 3e38f;
+  for (; n < kScK; ++n) {
+    float bv = 0.f;
+    int bk = -1;
+    for (int k = p0 + lane; k < p1; k += 32) {
+      const float v = fabsf((float)val[k]);
+      if (col[k] == i || v == 0.f) continue;
+      const bool below = v < lastv || (v == lastv && k > last);
+      if (below && v > bv) {  // the lane's own entries ascend: the first of equals stays
+        bv = v;
+        bk = k;
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
+      const int ok = __shfl_xor_sync(0xffffffffu, bk, o);
+      if (ok >= 0 && (ov > bv || (ov == bv && ok < bk) || bk < 0)) {
+        bv = ov;
+        bk = ok;
+      }
+    }
+    if (bk < 0) break;
+    last = bk;
+    lastv = bv;
+    if (lane == n) myj = col[bk];
+  }
+  Js[w][lane] = myj;
+  for (int r = 0; r < 32; ++r) Bs[w][r][lane] = r == lane && lane >= n ? 1.f : 0.f;
+  __syncwarp();
+  // Bs[r][k] = Z0[J_k][J_r]
+  float diag = 1.f;
+  for (int k = 0; k < n; ++k) {
+    const int row = Js[w][k];
+    for (int q = ptr[row] + lane; q < ptr[row + 1]; q += 32) {
+      const int cc = col[q];
+      for (int r = 0; r < n; ++r)
+        if (Js[w][r] == cc) Bs[w][r][k] = (float)val[q];
+    }
+  }
+  __syncwarp();
+  if (Bs[w][0][0] != 0.f) diag = Bs[w][0][0];
+  float rhs = lane == 0 ? 1.f : 0.f;
+  int mine = -1;  // the column this row was the pivot of
+  bool ok = true;
+  for (int k = 0; k < 32 && ok; ++k) {
+    float v = mine < 0 ? fabsf(Bs[w][lane][k]) : -1.f;
+    int who = lane;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const float ov = __shfl_xor_sync(0xffffffffu, v, o);
+      const int oi = __shfl_xor_sync(0xffffffffu, who, o);
+      if (ov > v || (ov == v && oi < who)) {
+        v = ov;
+        who = oi;
+      }
+    }
+    ok = v > 0.f && v < 3e38f;  // the same in every lane
+    if (!ok) break;
+    const float piv = Bs[w][who][k];
+    const float prhs = __shfl_sync(0xffffffffu, rhs, who);
+    if (lane == who) {
+      mine = k;
+    } else {
+      const float f = Bs[w][lane][k] / piv;
+      for (int m = k + 1; m < 32; ++m) Bs[w][lane][m] = fmaf(-f, Bs[w][who][m], Bs[w][lane][m]);
+      rhs = fmaf(-f, prhs, rhs);
+    }
+    __syncwarp();
+  }
+  // y_k of the row that was column k's pivot
+  float y = 0.f;
+  if (ok) {
+    const float u = rhs / Bs[w][lane][mine];
+    for (int r = 0; r < 32; ++r) {
+      const int k = __shfl_sync(0xffffffffu, mine, r);
+      const float v = __shfl_sync(0xffffffffu, u, r);
+      if (lane == k) y = v;
+    }
+    ok = __all_sync(0xffffffffu, fabsf(y) < 3e38f);
+  }
+  if (!ok) y = lane == 0 ? 1.f / diag : 0.f;
+  pcol[(int64_t)i * kScK + lane] = myj;
+  pval[(int64_t)i * kScK + lane] = lane < n ? y : 0.f;
+}
+
 tdbem_status tdbem_sc_build(tdbem_ctx* c, int want, const std::vector<int32_t>& zp, const std::vector<int32_t>& zc,
-                            const std::vector<double>& zv, const std::vector<int32_t>& pcol,
-                            const std::vector<double>& pval) {
+                            const std::vector<double>& zv) {
   const int ne = (int)c->ne;
   ScPlan P;
   // the largest cluster the device schedules, at most the wanted one
@@ -725,31 +846,85 @@ tdbem_status tdbem_sc_build(tdbem_ctx* c, int want, const std::vector<int32_t>& 
     cudaGetLastError();
   }
   if (P.cs < 1) return TDBEM_OK;
+  // Z0 without the stored zeros (pairs whose lag window holds lag 1 but whose
+  // supports lie beyond c dt of each other: about 40% of the entries)
+  std::vector<int64_t> np(ne + 1, 0);
+  std::vector<int32_t> nc;
+  std::vector<double> nv;
+  nc.reserve(zc.size());
+  nv.reserve(zc.size());
+  for (int i = 0; i < ne; ++i) {
+    for (int k = zp[i]; k < zp[i + 1]; ++k)
+      if (zv[k] != 0.0) {
+        nc.push_back(zc[k]);
+        nv.push_back(zv[k]);
+      }
+    np[i + 1] = (int64_t)nc.size();
+  }
+  // P
+  std::vector<int64_t> pp(ne + 1, 0);
+  std::vector<int32_t> pc;
+  std::vector<double> pv;
+  tdbem_status s;
+  if (c->p.precond == 1) {
+    int32_t* d_pc = nullptr;
+    float* d_pv = nullptr;
+    const size_t n = (size_t)ne * kScK;
+    if ((s = c->dalloc(&d_pc, n)) || (s = c->dalloc(&d_pv, n))) return s;
+    k_local_inverse<<<(ne + kLiWarps - 1) / kLiWarps, kLiWarps * 32, 0, c->stream>>>(c->d_z0_ptr, c->d_z0_col,
+                                                                                    c->d_z0_val, ne, d_pc, d_pv);
+    TDBEM_CUDA_TRY(c, cudaGetLastError());
+    std::vector<int32_t> hc(n);
+    std::vector<float> hv(n);
+    TDBEM_CUDA_TRY(c, cudaMemcpyAsync(hc.data(), d_pc, n * sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
+    TDBEM_CUDA_TRY(c, cudaMemcpyAsync(hv.data(), d_pv, n * sizeof(float), cudaMemcpyDeviceToHost, c->stream));
+    TDBEM_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+    c->dfree(d_pc);
+    c->dfree(d_pv);
+    for (int i = 0; i < ne; ++i) {
+      for (int k = 0; k < kScK; ++k)
+        if (hv[(size_t)i * kScK + k] != 0.f) {
+          pc.push_back(hc[(size_t)i * kScK + k]);
+          pv.push_back(hv[(size_t)i * kScK + k]);
+        }
+      pp[i + 1] = (int64_t)pc.size();
+    }
+  } else {
+    for (int i = 0; i < ne; ++i) {
+      double d = 0.0;
+      for (int64_t k = np[i]; k < np[i + 1]; ++k)
+        if (nc[k] == i) d = nv[k];
+      pc.push_back(i);
+      pv.push_back(d != 0.0 ? 1.0 / d : 1.0);
+      pp[i + 1] = (int64_t)pc.size();
+    }
+  }
   // A = Z0 P, row by row
   std::vector<int64_t> ap(ne + 1, 0);
-  std::vector<int32_t> ac, at(ne, -1);
-  std::vector<double> av;
-  ac.reserve(zc.size() * 2);
-  av.reserve(zc.size() * 2);
+  std::vector<int32_t> ac, at(ne, -1), rowc;
+  std::vector<double> av, acc(ne, 0.0);
   for (int i = 0; i < ne; ++i) {
-    const int64_t r0 = (int64_t)ac.size();
-    for (int k = zp[i]; k < zp[i + 1]; ++k) {
-      const int j = zc[k];
-      for (int m = 0; m < kScPc; ++m) {
-        const double pv = pval[(size_t)m * ne + j];
-        if (pv == 0.0) continue;
-        const int l = pcol[(size_t)m * ne + j];
-        if (at[l] < r0) {
-          at[l] = (int32_t)ac.size();
-          ac.push_back(l);
-          av.push_back(0.0);
+    rowc.clear();
+    for (int64_t k = np[i]; k < np[i + 1]; ++k) {
+      const double z = nv[k];
+      const int j = nc[k];
+      for (int64_t m = pp[j]; m < pp[j + 1]; ++m) {
+        const int l = pc[m];
+        if (at[l] != i) {
+          at[l] = i;
+          acc[l] = 0.0;
+          rowc.push_back(l);
         }
-        av[at[l]] += zv[k] * pv;
+        acc[l] += z * pv[m];
       }
     }
+    for (int l : rowc)
+      if (std::fabs(acc[l]) > kScDrop) {
+        ac.push_back(l);
+        av.push_back(acc[l]);
+      }
     ap[i + 1] = (int64_t)ac.size();
   }
-  if (ap[ne] >= (1ll << 31)) return TDBEM_OK;
   // order: rows by their blocks of A, longest first (stable), in groups of 8 dealt over the CTAs
   std::vector<int32_t> ord(ne);
   for (int i = 0; i < ne; ++i) ord[i] = i;
@@ -769,57 +944,12 @@ tdbem_status tdbem_sc_build(tdbem_ctx* c, int want, const std::vector<int32_t>& 
         at_pos[ord[next]] = (int32_t)p;
       }
     }
-  std::vector<int32_t> ab, ae, zb, ze;
-  int32_t na = 0, nz = 0;
-  auto alen = [&](int i) { return (int)(ap[i + 1] - ap[i]); };
-  auto zlen = [&](int i) { return zp[i + 1] - zp[i]; };
-  auto none = [](int64_t, int, int) {};
-  sc_blocks(P, perm, alen, none, &ab, &ae, &na);
-  sc_blocks(P, perm, zlen, none, &zb, &ze, &nz);
-  tdbem_status s;
-  if ((s = sc_upload(c, &P.perm, perm)) || (s = sc_upload(c, &P.ab, ab)) || (s = sc_upload(c, &P.ae, ae)) ||
-      (s = sc_upload(c, &P.zb, zb)) || (s = sc_upload(c, &P.ze, ze)))
+  if ((s = sc_upload(c, &P.perm, perm)) ||
+      (s = sc_matrix(c, P, perm, at_pos, {ap, ac, av}, &P.ab, &P.ae, &P.aval, nullptr, nullptr, &P.acol)) ||
+      (s = sc_matrix(c, P, perm, at_pos, {pp, pc, pv}, &P.pb, &P.pe, &P.pval, nullptr, nullptr, &P.pcol)) ||
+      (s = sc_matrix(c, P, perm, at_pos, {np, nc, nv}, &P.zb, &P.ze, &P.zhi, &P.zlo, &P.zval, &P.zcol)) ||
+      (s = c->dalloc(&P.w64, 2 * (size_t)P.npad)))
     return s;
-  {
-    std::vector<float4> v((size_t)na * 32, make_float4(0, 0, 0, 0));
-    std::vector<uint2> col((size_t)na * 32, make_uint2(0, 0));
-    float* fv = (float*)v.data();
-    uint16_t* fc = (uint16_t*)col.data();
-    sc_blocks(P, perm, alen, [&](int64_t o, int i, int m) {
-      fv[o] = (float)av[ap[i] + m];
-      fc[o] = (uint16_t)at_pos[ac[ap[i] + m]];
-    }, &ab, &ae, &na);
-    if ((s = sc_upload(c, &P.aval, v)) || (s = sc_upload(c, &P.acol, col))) return s;
-  }
-  {
-    std::vector<double2> v((size_t)nz * 64, make_double2(0, 0));
-    std::vector<float4> hi((size_t)nz * 32, make_float4(0, 0, 0, 0)), lo = hi;
-    std::vector<uint2> col((size_t)nz * 32, make_uint2(0, 0));
-    double* dv = (double*)v.data();
-    float *fh = (float*)hi.data(), *fl = (float*)lo.data();
-    uint16_t* fc = (uint16_t*)col.data();
-    sc_blocks(P, perm, zlen, [&](int64_t o, int i, int m) {
-      const double z = zv[zp[i] + m];
-      dv[o] = z;
-      fh[o] = (float)z;
-      fl[o] = (float)(z - (double)fh[o]);
-      fc[o] = (uint16_t)at_pos[zc[zp[i] + m]];
-    }, &zb, &ze, &nz);
-    if ((s = sc_upload(c, &P.zval, v)) || (s = sc_upload(c, &P.zhi, hi)) || (s = sc_upload(c, &P.zlo, lo)) ||
-        (s = sc_upload(c, &P.zcol, col)))
-      return s;
-  }
-  {
-    std::vector<float> pv((size_t)kScPc * P.npad, 0.f);
-    std::vector<uint16_t> pc((size_t)kScPc * P.npad, 0);
-    for (int m = 0; m < kScPc; ++m)
-      for (int i = 0; i < ne; ++i) {
-        pv[(size_t)m * P.npad + at_pos[i]] = (float)pval[(size_t)m * ne + i];
-        pc[(size_t)m * P.npad + at_pos[i]] = (uint16_t)at_pos[pcol[(size_t)m * ne + i]];
-      }
-    if ((s = sc_upload(c, &P.pval, pv)) || (s = sc_upload(c, &P.pcol, pc)) || (s = c->dalloc(&P.w64, 2 * (size_t)P.npad)))
-      return s;
-  }
   TDBEM_CUDA_TRY(c, cudaMemsetAsync(P.w64, 0, 2 * (size_t)P.npad * sizeof(double), c->stream));
   c->sc = new (std::nothrow) ScPlan(P);
   return c->sc ? TDBEM_OK : TDBEM_ENOMEM;
@@ -839,6 +969,8 @@ tdbem_status tdbem_sc_solve(tdbem_ctx* c, int32_t alpha, int32_t warm) {
   A.zhi = P.zhi;
   A.zlo = P.zlo;
   A.zcol = P.zcol;
+  A.pb = P.pb;
+  A.pe = P.pe;
   A.pval = P.pval;
   A.pcol = P.pcol;
   A.w64 = P.w64;
