@@ -92,7 +92,7 @@ struct tdbem_ctx {
   // direct coefficients: rows i, all j (direct mode)
   tdbem::PairStore direct;
   tdbem::FmmPlan* fmm = nullptr;    // fast mode
-  tdbem::ScPlan* sc = nullptr;      // single-right-hand-side cluster solve (solve_cluster.cu)
+  tdbem::ScPlan* sc = nullptr;      // cluster solve, a cluster per right-hand side (solve_cluster.cu)
   int32_t max_lag = 0;
   // Z0 in CSR
   int32_t* d_z0_ptr = nullptr;
@@ -300,7 +300,7 @@ void tdbem_mlp_free(tdbem_ctx* c);
 tdbem_status tdbem_build_z0(tdbem_ctx* c);
 tdbem_status tdbem_build_z0_csr(tdbem_ctx* c);
 tdbem_status tdbem_solve_z0(tdbem_ctx* c, int32_t alpha, int32_t* iters, int32_t warm);
-// solve_cluster.cu: the cluster solve of one right-hand side for the context's Z0
+// solve_cluster.cu: the cluster solve, a cluster per right-hand side, for the context's Z0
 // (CSR on the device, and here on the host); want: CTAs of the cluster at most.
 // No plan is made (c->sc stays null) where the mesh does not fit it.
 tdbem_status tdbem_sc_build(tdbem_ctx* c, int want, const std::vector<int32_t>& zp, const std::vector<int32_t>& zc,

@@ -1038,8 +1038,8 @@ static tdbem_status tdbem_z0_f32(tdbem_ctx* c) {
   // of the store's own rounding (1e-8 after 80 steps on the 7680-RWG sphere, from
   // 1e-13): they keep k_bicgstab and with it their currents.
   const bool f32 = c->p.mode == TDBEM_DIRECT && c->p.p2p_prec != TDBEM_P_FP64;
-  if (c->R == 1 && c->p.jacobi_sweeps == 0 && !f32 && !use_grid(c)) {
-    if ((s = tdbem_sc_build(c, c->p.solve_cluster > 0 ? c->p.solve_cluster : 16, hp, hc, hv)) || c->sc) return s;
+  if (c->p.jacobi_sweeps == 0 && !f32 && !(c->R == 1 && use_grid(c))) {
+    if ((s = tdbem_sc_build(c, c->p.solve_cluster > 0 && c->R == 1 ? c->p.solve_cluster : 16, hp, hc, hv)) || c->sc) return s;
   }
   return c->p.precond == 1 ? build_triangle_precond(c, hp, hc, hv) : TDBEM_OK;
 }
@@ -1226,10 +1226,10 @@ static tdbem_status solve_multi(tdbem_ctx* c, int32_t alpha, int32_t warm) {
 
 tdbem_status tdbem_solve_z0(tdbem_ctx* c, int32_t alpha, int32_t* iters, int32_t warm) {
   tdbem_status s;
-  if (c->R > 1) {
-    if ((s = solve_multi(c, alpha, warm))) return s;
-  } else if (c->sc) {
+  if (c->sc) {
     if ((s = tdbem_sc_solve(c, alpha, warm))) return s;
+  } else if (c->R > 1) {
+    if ((s = solve_multi(c, alpha, warm))) return s;
   } else {
     const bool grid = use_grid(c);
     if ((s = grid ? pick_grid(c) : pick_cluster(c))) return s;

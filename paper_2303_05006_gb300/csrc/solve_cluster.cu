@@ -1,6 +1,6 @@
-// solve_cluster.cu -- the single-right-hand-side solve Z0 J^{alpha-1} =
-// R^{alpha-1} (paper eq. solve) in one thread-block cluster, with the exchanged
-// vector kept whole in every CTA's shared memory.
+// solve_cluster.cu -- the solve Z0 J^{alpha-1} = R^{alpha-1} (paper eq. solve),
+// one thread-block cluster per right-hand side, with the exchanged vector kept
+// whole in every CTA's shared memory.
 //
 // Scheme.  Iterative refinement: an FP64 residual r = b - Z0 x around an FP32
 // BiCGStab on the right-preconditioned matrix A = Z0 P, which is formed once at
@@ -64,12 +64,12 @@ struct ScArgs {
   const int32_t *pb, *pe;    // P, as A
   const float4* pval;
   const uint2* pcol;
-  double* w64;               // [2][npad] iterates as the residual gathers them
-  const double* b;           // rows in edge order from here on
+  double* w64;               // [R][2][npad] iterates as the residual gathers them
+  const double* b;           // [ne][R], rows in edge order from here on
   double* x;
   double* ring;
   float2* rs;                // the ring's values as (hi, lo) pairs (may be null)
-  int32_t L, alpha, warm, gpc, passes, npad, ne, maxit;
+  int32_t L, alpha, warm, gpc, passes, npad, ne, maxit, R;
   double tol;
   int32_t* status;           // as in SolveArgs (solve.cu)
   double* resid;
@@ -397,6 +397,8 @@ __global__ void __launch_bounds__(kScThreads) k_solve_cluster(const ScArgs A) {
   S.warp = (int)threadIdx.x >> 5;
   S.lane = (int)threadIdx.x & 31;
   S.phase = 0;
+  const int R = A.R, rhs = (int)blockIdx.x / S.nb;  // this cluster's right-hand side
+  double* const w64 = A.w64 + (int64_t)rhs * 2 * A.npad;
   const int lane = S.lane, q = lane & 3, W = S.rank * kScWarps + S.warp;
   const uint32_t Xa = (uint32_t)__cvta_generic_to_shared(sc_X);
   // this thread's rows: position and edge of each (-1: none)
@@ -431,12 +433,12 @@ __global__ void __launch_bounds__(kScThreads) k_solve_cluster(const ScArgs A) {
   for (int e = 0; e < RPT; ++e) {
     x[e] = b[e] = 0.0;
     if (row[e] < 0) continue;
-    b[e] = A.b[row[e]];
+    b[e] = A.b[(int64_t)row[e] * R + rhs];
     if (A.warm) {  // cubic extrapolation of the last four currents (zero before step 0)
-      const double* J = A.ring + (int64_t)row[e] * A.L;
+      const double* J = A.ring + (int64_t)row[e] * A.L * R + rhs;
       const int s = A.alpha - 2;
-      const double j1 = s >= 0 ? J[s & msk] : 0.0, j2 = s >= 1 ? J[(s - 1) & msk] : 0.0;
-      const double j3 = s >= 2 ? J[(s - 2) & msk] : 0.0, j4 = s >= 3 ? J[(s - 3) & msk] : 0.0;
+      const double j1 = s >= 0 ? J[(s & msk) * R] : 0.0, j2 = s >= 1 ? J[((s - 1) & msk) * R] : 0.0;
+      const double j3 = s >= 2 ? J[((s - 2) & msk) * R] : 0.0, j4 = s >= 3 ? J[((s - 3) & msk) * R] : 0.0;
       x[e] = 4.0 * j1 - 6.0 * j2 + 4.0 * j3 - j4;
     }
   }
@@ -468,7 +470,7 @@ __global__ void __launch_bounds__(kScThreads) k_solve_cluster(const ScArgs A) {
   for (int outer = -1;; ++outer) {
     double nr, nbb;
     if (outer < 0 || !(rr <= 0x1p-16 * bb)) {
-      residual(x, A.w64, r64);
+      residual(x, w64, r64);
     } else {
       // The correction (y: its FP32 digits) is at most about 2^-8 of the iterate:
       // Z0 d in double-float (46 bits) is then as exact as b - Z0 x anew in FP64.
@@ -485,8 +487,8 @@ __global__ void __launch_bounds__(kScThreads) k_solve_cluster(const ScArgs A) {
     if (outer < 0 && A.warm == 2) {
       double g[RPT], rg[RPT], gg, b2;
 #pragma unroll
-      for (int e = 0; e < RPT; ++e) g[e] = row[e] >= 0 ? A.x[row[e]] : 0.0;
-      residual(g, A.w64 + A.npad, rg);
+      for (int e = 0; e < RPT; ++e) g[e] = row[e] >= 0 ? A.x[(int64_t)row[e] * R + rhs] : 0.0;
+      residual(g, w64 + A.npad, rg);
       norm2(rg, gg, b2);
       const bool keep = gg < rr;
       if (keep) {
@@ -497,7 +499,7 @@ __global__ void __launch_bounds__(kScThreads) k_solve_cluster(const ScArgs A) {
           r64[e] = rg[e];
         }
       }
-      if (S.rank == 0 && threadIdx.x == 0) A.status[keep ? 8 : 9] += 1;
+      if (S.rank == 0 && threadIdx.x == 0) atomicAdd(&A.status[keep ? 8 : 9], 1);
     }
     const double tol2bb = A.tol * A.tol * bb;
     if (rr <= tol2bb) {
@@ -592,18 +594,35 @@ __global__ void __launch_bounds__(kScThreads) k_solve_cluster(const ScArgs A) {
 #pragma unroll
   for (int e = 0; e < RPT; ++e)
     if (row[e] >= 0) {
-      A.x[row[e]] = x[e];
-      const int64_t o = (int64_t)row[e] * A.L + ((A.alpha - 1) & msk);
+      A.x[(int64_t)row[e] * R + rhs] = x[e];
+      const int64_t o = ((int64_t)row[e] * A.L + ((A.alpha - 1) & msk)) * R + rhs;
       A.ring[o] = x[e];
       if (A.rs) A.rs[o] = split_pair(x[e]);
     }
   if (S.rank == 0 && threadIdx.x == 0) {
-    A.status[0] = inner_total;
-    A.status[6] = 0;
-    A.status[1] = conv ? 1 : 0;
-    A.status[2] += conv ? 0 : 1;
-    A.status[3] += inner_total;
-    A.resid[0] = bb > 0 ? sqrt(rr / bb) : 0.0;
+    if (R == 1) {
+      A.status[0] = inner_total;
+      A.status[6] = 0;
+      A.status[1] = conv ? 1 : 0;
+      A.status[2] += conv ? 0 : 1;
+      A.status[3] += inner_total;
+      A.resid[0] = bb > 0 ? sqrt(rr / bb) : 0.0;
+    } else {
+      // status[0] (the most iterations of any right-hand side) is zero at launch;
+      // the last cluster to finish publishes the step's verdict
+      atomicMax(&A.status[0], inner_total);
+      if (!conv) atomicAdd(&A.status[4], 1);
+      __threadfence();
+      if (atomicAdd(&A.status[5], 1) == R - 1) {
+        __threadfence();
+        const int miss = atomicExch(&A.status[4], 0), it = atomicAdd(&A.status[0], 0);
+        A.status[6] = 0;
+        A.status[1] = miss == 0 ? 1 : 0;
+        A.status[2] += miss == 0 ? 0 : 1;
+        A.status[3] += it;
+        A.status[5] = 0;
+      }
+    }
   }
   S.sync();  // no CTA leaves while another may still store into its shared memory
 }
@@ -628,9 +647,9 @@ static ScFn sc_fn(int passes) {
 
 static size_t sc_smem(const ScPlan& P) { return (size_t)P.npad * sizeof(float); }
 
-static void sc_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* at, int cs, size_t smem, cudaStream_t st) {
+static void sc_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* at, int cs, int ctas, size_t smem, cudaStream_t st) {
   *cfg = {};
-  cfg->gridDim = dim3(cs);
+  cfg->gridDim = dim3(ctas);
   cfg->blockDim = dim3(kScThreads);
   cfg->dynamicSmemBytes = smem;
   cfg->stream = st;
@@ -828,22 +847,36 @@ tdbem_status tdbem_sc_build(tdbem_ctx* c, int want, const std::vector<int32_t>& 
                             const std::vector<double>& zv) {
   const int ne = (int)c->ne;
   ScPlan P;
-  // the largest cluster the device schedules, at most the wanted one
-  for (P.cs = want; P.cs >= 1; P.cs >>= 1) {
-    const int groups = (ne + 7) / 8;
-    P.gpc = (groups + P.cs - 1) / P.cs;
-    P.passes = (P.gpc + kScWarps - 1) / kScWarps;
-    P.npad = P.cs * P.gpc * 8;
-    if (P.passes > kScPasses || P.npad > 65535 || sc_smem(P) > 200 * 1024) return TDBEM_OK;
-    const ScFn fn = sc_fn(P.passes);
+  // Cluster size: the one of least cost among those the device schedules, at most
+  // the wanted one.  An iteration costs about 8 us of barriers and latency (4.5 in a
+  // single CTA, which has no cluster barriers) and 9 ns per row and CTA for the
+  // products, whatever the number of clusters that run side by side; right-hand
+  // sides beyond those queue.
+  double best = 1e300;
+  for (int cs = want; cs >= 1; cs >>= 1) {
+    ScPlan T;
+    T.cs = cs;
+    T.gpc = ((ne + 7) / 8 + cs - 1) / cs;
+    T.passes = (T.gpc + kScWarps - 1) / kScWarps;
+    T.npad = cs * T.gpc * 8;
+    if (T.passes > kScPasses || T.npad > 65535 || sc_smem(T) > 200 * 1024) break;
+    const ScFn fn = sc_fn(T.passes);
     TDBEM_CUDA_TRY(c, cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     TDBEM_CUDA_TRY(c, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute at;
-    sc_config(&cfg, &at, P.cs, sc_smem(P), c->stream);
+    sc_config(&cfg, &at, cs, cs, sc_smem(T), c->stream);
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) == cudaSuccess && n > 0) break;
-    cudaGetLastError();
+    if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess || n < 1) {
+      cudaGetLastError();
+      continue;
+    }
+    const double cost = (double)((c->R + n - 1) / n) * ((cs > 1 ? 8.0 : 4.5) + 0.009 * ne / cs);
+    if (cost < best) {
+      best = cost;
+      P = T;
+    }
+    if (c->p.solve_cluster > 0 && c->R == 1) break;  // the caller's choice
   }
   if (P.cs < 1) return TDBEM_OK;
   // Z0 without the stored zeros (pairs whose lag window holds lag 1 but whose
@@ -948,9 +981,9 @@ tdbem_status tdbem_sc_build(tdbem_ctx* c, int want, const std::vector<int32_t>& 
       (s = sc_matrix(c, P, perm, at_pos, {ap, ac, av}, &P.ab, &P.ae, &P.aval, nullptr, nullptr, &P.acol)) ||
       (s = sc_matrix(c, P, perm, at_pos, {pp, pc, pv}, &P.pb, &P.pe, &P.pval, nullptr, nullptr, &P.pcol)) ||
       (s = sc_matrix(c, P, perm, at_pos, {np, nc, nv}, &P.zb, &P.ze, &P.zhi, &P.zlo, &P.zval, &P.zcol)) ||
-      (s = c->dalloc(&P.w64, 2 * (size_t)P.npad)))
+      (s = c->dalloc(&P.w64, 2 * (size_t)P.npad * c->R)))
     return s;
-  TDBEM_CUDA_TRY(c, cudaMemsetAsync(P.w64, 0, 2 * (size_t)P.npad * sizeof(double), c->stream));
+  TDBEM_CUDA_TRY(c, cudaMemsetAsync(P.w64, 0, 2 * (size_t)P.npad * c->R * sizeof(double), c->stream));
   c->sc = new (std::nothrow) ScPlan(P);
   return c->sc ? TDBEM_OK : TDBEM_ENOMEM;
 }
@@ -985,6 +1018,7 @@ tdbem_status tdbem_sc_solve(tdbem_ctx* c, int32_t alpha, int32_t warm) {
   A.passes = P.passes;
   A.npad = P.npad;
   A.ne = (int32_t)c->ne;
+  A.R = c->R;
   A.maxit = c->p.solve_maxit;
   A.tol = c->p.solve_tol;
   A.status = c->d_status;
@@ -992,7 +1026,8 @@ tdbem_status tdbem_sc_solve(tdbem_ctx* c, int32_t alpha, int32_t warm) {
   c->cluster = P.cs;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute at;
-  sc_config(&cfg, &at, P.cs, sc_smem(P), c->stream);
+  sc_config(&cfg, &at, P.cs, P.cs * c->R, sc_smem(P), c->stream);
+  if (c->R > 1) TDBEM_CUDA_TRY(c, cudaMemsetAsync(c->d_status, 0, sizeof(int32_t), c->stream));
   TDBEM_CUDA_TRY(c, cudaLaunchKernelEx(&cfg, sc_fn(P.passes), A));
   return TDBEM_OK;
 }
