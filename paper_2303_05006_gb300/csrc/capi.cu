@@ -173,6 +173,10 @@ static tdbem_status finish_create(tdbem_ctx* c) {
   if ((s = c->dalloc(&c->d_Jring, NR * L)) || (s = c->dalloc(&c->d_R, NR)) || (s = c->dalloc(&c->d_J, NR)) ||
       (s = c->dalloc(&c->d_pulse, 10 * (int64_t)c->R)) || (c->R > 1 && (s = c->dalloc(&c->d_stage, NR))))
     return s;
+  if (c->p.mode == TDBEM_FAST && c->R > 1) {
+    if ((s = c->dalloc(&c->d_rf, NR * L))) return s;
+    TDBEM_CUDA_TRY(c, cudaMemsetAsync(c->d_rf, 0, NR * L * sizeof(float), c->stream));
+  }
   TDBEM_CUDA_TRY(c, cudaMemsetAsync(c->d_Jring, 0, NR * L * sizeof(double), c->stream));
   TDBEM_CUDA_TRY(c, cudaMemsetAsync(c->d_J, 0, NR * sizeof(double), c->stream));
   TDBEM_CUDA_TRY(c, cudaMemsetAsync(c->d_status, 0, 16 * sizeof(int32_t), c->stream));
@@ -285,6 +289,11 @@ tdbem_status tdbem_set_incident_plane(tdbem_ctx* c, int32_t rhs, const double* p
 __global__ void k_put_column(const double* x, int64_t n, int32_t R, int32_t r, double* y) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i < n) y[i * R + r] = x[i];
+}
+
+__global__ void k_ring_f32(const double* x, int64_t n, float* y) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i < n) y[i] = (float)x[i];
 }
 
 // [ne][R] (device layout) -> [R][ne] (host layout) and back
@@ -767,6 +776,7 @@ tdbem_status tdbem_reset(tdbem_ctx* c) {
   const int64_t NR = c->ne * (int64_t)c->R;
   TDBEM_CUDA_TRY(c, cudaMemsetAsync(c->d_Jring, 0, NR * c->L * sizeof(double), c->stream));
   if (c->d_rs) TDBEM_CUDA_TRY(c, cudaMemsetAsync(c->d_rs, 0, NR * c->L * sizeof(float2), c->stream));
+  if (c->d_rf) TDBEM_CUDA_TRY(c, cudaMemsetAsync(c->d_rf, 0, NR * c->L * sizeof(float), c->stream));
   TDBEM_CUDA_TRY(c, cudaMemsetAsync(c->d_J, 0, NR * sizeof(double), c->stream));
   TDBEM_CUDA_TRY(c, cudaMemsetAsync(c->d_status, 0, 16 * sizeof(int32_t), c->stream));
   if (c->p.mode == TDBEM_FAST) {
@@ -867,6 +877,11 @@ tdbem_status tdbem_load(tdbem_ctx* c, const char* path) {
     TDBEM_CUDA_TRY(c, cudaMemcpyAsync(bufs[k].first, host[k].data(), host[k].size(), cudaMemcpyHostToDevice, c->stream));
   TDBEM_CUDA_TRY(c, cudaMemsetAsync(c->d_status, 0, 16 * sizeof(int32_t), c->stream));
   if ((s = tdbem_direct_resplit(c))) return s;
+  if (c->d_rf) {
+    const int64_t n = c->ne * (int64_t)c->L * c->R;
+    k_ring_f32<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(c->d_Jring, n, c->d_rf);
+    TDBEM_CUDA_TRY(c, cudaGetLastError());
+  }
   TDBEM_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   c->alpha = h.alpha;
   return TDBEM_OK;

@@ -907,37 +907,56 @@ __global__ void k_near_seg_reduce(const int64_t* rseg_ptr, const int32_t* rseg, 
   if (i < ne && sub == 0) R[i] = -t;
 }
 
-// Batched near field on the flattened entries: one block per row; thread t
-// takes right-hand side r0 + t mod RL (RL = R rounded up to a power of two,
-// at most 32) and the row's entries sub, sub + nsub, ... (sub = t / RL), so
-// each entry's coefficient is read once per lane group and its history
-// R-vector contiguously; partial sums meet in shared memory.
-__global__ void __launch_bounds__(256) k_near_history_flat_multi(const int64_t* hrow, const float* hval,
-                                                                const int32_t* hmeta, int64_t ne, const double* ring,
-                                                                int L, int alpha, int R, int RL, const double* V,
-                                                                double* Rfar_slot, double* Rout) {
-  __shared__ double red[8][32];
+// Batched near field on the flattened entries: one block per row, its 8 warps
+// taking interleaved runs of 32 entries.  A lane loads one entry of the run
+// (coalesced); then RL lanes (R rounded up to a power of two, at most 32) share an
+// entry at a time, 32 / RL entries side by side, its coefficient and place passed by
+// shuffles and its history R-vector read contiguously.  What bounds it is the
+// history's L2 traffic and latency: the run's reads are independent of each other,
+// so up to 32 are in flight per warp, and the march reads its ring in FP32 (rf, the
+// values the FP64 ring would be rounded to here; kept by the solve).  A chain of
+// FP32 additions is 1 / (8 * 32 / RL) of the row; the chains meet in FP64.
+template <int RL, typename T>
+__global__ void __launch_bounds__(256) k_near_history_flat_multi(const int64_t* __restrict__ hrow,
+                                                                const float* __restrict__ hval,
+                                                                const int32_t* __restrict__ hmeta, int64_t ne,
+                                                                const T* __restrict__ ring, int L, int alpha, int R,
+                                                                const double* V, double* Rfar_slot, double* Rout) {
+  __shared__ double red[8][RL];
   const int64_t i = blockIdx.x;
-  const int rr = threadIdx.x % RL, sub = threadIdx.x / RL, nsub = blockDim.x / RL;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rr = lane % RL, sub = lane / RL;
   const int64_t e0 = hrow[i], e1 = hrow[i + 1];
   for (int r0 = 0; r0 < R; r0 += RL) {
-    const int r = r0 + rr;
+    const int r = min(r0 + rr, R - 1);  // lanes past R repeat the last column and are not stored
     float s = 0.f;
-    if (r < R) {
-      for (int64_t e = e0 + sub; e < e1; e += nsub) {
+    for (int64_t eb = e0 + warp * 32; eb < e1; eb += 256) {
+      const int64_t e = eb + lane;
+      float z = 0.f;
+      int o = 0;  // place in the ring, in units of R
+      if (e < e1) {
         const int q = __ldg(hmeta + e);
         const int b = alpha - (q & 0xff);
-        if (b >= 0) s += __ldg(hval + e) * (float)ring[((int64_t)(q >> 8) * L + (b & (L - 1))) * R + r];
+        if (b >= 0) {  // (no history yet: a zero coefficient at a place that exists)
+          z = __ldg(hval + e);
+          o = (q >> 8) * L + (b & (L - 1));
+        }
+      }
+#pragma unroll 8
+      for (int k = 0; k < 32; k += 32 / RL) {
+        const float zk = __shfl_sync(0xffffffffu, z, k + sub);
+        const int ok = __shfl_sync(0xffffffffu, o, k + sub);
+        s = fmaf(zk, (float)ring[(int64_t)ok * R + r], s);
       }
     }
     double d = s;
-    for (int o = 16; o >= RL; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+#pragma unroll
+    for (int t = 16; t >= RL; t >>= 1) d += __shfl_xor_sync(0xffffffffu, d, t);
     if (lane < RL) red[warp][lane] = d;
     __syncthreads();
     if (threadIdx.x < RL && r0 + (int)threadIdx.x < R) {
       double t = 0.0;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w][threadIdx.x];
+#pragma unroll
+      for (int w = 0; w < 8; ++w) t += red[w][threadIdx.x];
       const int64_t q = i * R + r0 + threadIdx.x;
       const double far = Rfar_slot ? Rfar_slot[q] : 0.0;
       Rout[q] = (V ? V[q] : 0.0) + far - t;
@@ -945,6 +964,19 @@ __global__ void __launch_bounds__(256) k_near_history_flat_multi(const int64_t* 
     }
     __syncthreads();
   }
+}
+
+template <typename T>
+static void near_multi(tdbem_ctx* c, const FmmPlan* F, const T* ring, int alpha, const double* V, double* slot) {
+  const unsigned g = (unsigned)c->ne;
+  auto run = [&](auto fn) {
+    fn<<<g, 256, 0, c->stream>>>(F->d_hrow, F->d_hval, F->d_hmeta, c->ne, ring, c->L, alpha, c->R, V, slot, c->d_R);
+  };
+  if (c->R <= 2) run(k_near_history_flat_multi<2, T>);
+  else if (c->R <= 4) run(k_near_history_flat_multi<4, T>);
+  else if (c->R <= 8) run(k_near_history_flat_multi<8, T>);
+  else if (c->R <= 16) run(k_near_history_flat_multi<16, T>);
+  else run(k_near_history_flat_multi<32, T>);
 }
 
 __global__ void k_f64_to_f32(const double* a, float* b, int64_t n) {
@@ -1998,10 +2030,10 @@ tdbem_status tdbem_fast_history(tdbem_ctx* c, int32_t alpha, const double* ring,
                                                                              ring, c->L, alpha, V, nullptr, slot,
                                                                              c->d_R);
   } else {
-    int RL = 1;
-    while (RL < c->R && RL < 32) RL <<= 1;
-    k_near_history_flat_multi<<<(unsigned)c->ne, 256, 0, c->stream>>>(F->d_hrow, F->d_hval, F->d_hmeta, c->ne, ring,
-                                                                        c->L, alpha, c->R, RL, V, slot, c->d_R);
+    if (ring == c->d_Jring && c->d_rf)
+      near_multi(c, F, c->d_rf, alpha, V, slot);
+    else
+      near_multi(c, F, ring, alpha, V, slot);
   }
   c->prof_end(1, e);
   TDBEM_CUDA_TRY(c, cudaGetLastError());

@@ -529,6 +529,7 @@ struct MultiArgs {
   const double* b;   // [ne][R]
   double* x;         // [ne][R]
   double* ring;      // [ne][L][R]
+  float* rf;         // the same in FP32 (may be null)
   int32_t L, alpha, warm, R;
   double* w;         // FP64 residual [ne][R], then 9 FP32 vectors [9][ne][R]
   int64_t ne;
@@ -888,7 +889,11 @@ __global__ void __launch_bounds__(kSolveThreads) k_bicgstab_multi(MultiArgs A) {
   }
   int nconv = 0;
   for (int m = 0; m < Rl; ++m) nconv += conv[m] ? 1 : 0;
-  ROWS A.ring[(i * L + ((A.alpha - 1) & msk)) * R + rl] = A.x[i * R + rl];
+  ROWS {
+    const int64_t o = (i * L + ((A.alpha - 1) & msk)) * R + rl;
+    A.ring[o] = A.x[i * R + rl];
+    if (A.rf) A.rf[o] = (float)A.x[i * R + rl];
+  }
 #undef ROWS
   if (rk == 0 && threadIdx.x == 0) {
     atomicMax(&A.status[0], inner_total);
@@ -1190,6 +1195,7 @@ static tdbem_status solve_multi(tdbem_ctx* c, int32_t alpha, int32_t warm) {
   A.b = c->d_R;
   A.x = c->d_J;
   A.ring = c->d_Jring;
+  A.rf = c->d_rf;
   A.L = c->L;
   A.alpha = alpha;
   A.warm = warm;

@@ -69,6 +69,7 @@ struct ScArgs {
   double* x;
   double* ring;
   float2* rs;                // the ring's values as (hi, lo) pairs (may be null)
+  float* rf;                 // the ring's values in FP32 (may be null)
   int32_t L, alpha, warm, gpc, passes, npad, ne, maxit, R;
   double tol;
   int32_t* status;           // as in SolveArgs (solve.cu)
@@ -598,6 +599,7 @@ __global__ void __launch_bounds__(kScThreads) k_solve_cluster(const ScArgs A) {
       const int64_t o = ((int64_t)row[e] * A.L + ((A.alpha - 1) & msk)) * R + rhs;
       A.ring[o] = x[e];
       if (A.rs) A.rs[o] = split_pair(x[e]);
+      if (A.rf) A.rf[o] = (float)x[e];
     }
   if (S.rank == 0 && threadIdx.x == 0) {
     if (R == 1) {
@@ -1011,6 +1013,7 @@ tdbem_status tdbem_sc_solve(tdbem_ctx* c, int32_t alpha, int32_t warm) {
   A.x = c->d_J;
   A.ring = c->d_Jring;
   A.rs = c->d_rs;
+  A.rf = c->d_rf;
   A.L = c->L;
   A.alpha = alpha;
   A.warm = warm;
