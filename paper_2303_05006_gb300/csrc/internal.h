@@ -306,5 +306,8 @@ tdbem_status tdbem_solve_z0(tdbem_ctx* c, int32_t alpha, int32_t* iters, int32_t
 // No plan is made (c->sc stays null) where the mesh does not fit it.
 tdbem_status tdbem_sc_build(tdbem_ctx* c, int want, const std::vector<int32_t>& zp, const std::vector<int32_t>& zc,
                             const std::vector<double>& zv);
+// the same for the FP32 and 24-bit direct marches: k_bicgstab's own arithmetic
+tdbem_status tdbem_bx_build(tdbem_ctx* c, int want, const std::vector<int32_t>& zp, const std::vector<int32_t>& zc,
+                            const std::vector<double>& zv);
 tdbem_status tdbem_sc_solve(tdbem_ctx* c, int32_t alpha, int32_t warm);
 void tdbem_sc_free(tdbem_ctx* c);

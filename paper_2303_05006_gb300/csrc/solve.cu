@@ -940,6 +940,7 @@ __global__ void k_z0_f32(const double* z, const double* inv_diag, int64_t nnz, i
 using namespace tdbem;
 
 static int g_cluster = 0;
+static tdbem_status pick_cluster(tdbem_ctx* c);
 
 // Meshes with at least this many RWG functions solve over a cooperative grid
 // of every SM instead of one cluster: a 16-SM cluster spends about 1 ms per
@@ -1041,12 +1042,18 @@ static tdbem_status tdbem_z0_f32(tdbem_ctx* c) {
   // The FP32 and 24-bit stores' marches round every current to FP32 in the next
   // steps' sums, so they carry any difference in the solve's rounding on at the level
   // of the store's own rounding (1e-8 after 80 steps on the 7680-RWG sphere, from
-  // 1e-13): they keep k_bicgstab and with it their currents.
+  // 1e-13): they keep k_bicgstab's arithmetic (k_bicgstab_x) and with it
+  // their currents.
   const bool f32 = c->p.mode == TDBEM_DIRECT && c->p.p2p_prec != TDBEM_P_FP64;
   if (c->p.jacobi_sweeps == 0 && !f32 && !(c->R == 1 && use_grid(c))) {
     if ((s = tdbem_sc_build(c, c->p.solve_cluster > 0 && c->R == 1 ? c->p.solve_cluster : 16, hp, hc, hv)) || c->sc) return s;
   }
-  return c->p.precond == 1 ? build_triangle_precond(c, hp, hc, hv) : TDBEM_OK;
+  if (c->p.precond != 1) return TDBEM_OK;
+  if ((s = build_triangle_precond(c, hp, hc, hv))) return s;
+  // (the same cluster size as k_bicgstab would take: the sums' tree depends on it)
+  if (f32 && c->R == 1 && c->p.jacobi_sweeps == 0 && !use_grid(c) && !(s = pick_cluster(c)))
+    s = tdbem_bx_build(c, c->p.solve_cluster > 0 ? std::min(c->p.solve_cluster, g_cluster) : g_cluster, hp, hc, hv);
+  return s;
 }
 
 tdbem_status tdbem_build_z0(tdbem_ctx* c) {

@@ -629,6 +629,403 @@ __global__ void __launch_bounds__(kScThreads) k_solve_cluster(const ScArgs A) {
   S.sync();  // no CTA leaves while another may still store into its shared memory
 }
 
+// ---------------------------------------------------------------------------
+// The solve of the FP32 and 24-bit direct marches: the arithmetic of k_bicgstab
+// (solve.cu) rounding for rounding, so that their currents stay what they are (see
+// tdbem_z0_f32), in the exchange form above.  What k_bicgstab spent its time on is
+// gone: every thread's FP64 divisions and square roots (one warp computes the
+// scalars now), two FP64 shuffle trees per pair of sums (folded into one tree with
+// the same additions), Krylov vectors in L2 and one dependent gather after the other
+// (registers, whole copies in shared memory, four blocks of entries in flight).
+// Rows stay in edge order, thread t of CTA k owning the rows k ceil(ne / CTAs) + t,
+// + 512, ..; a row's entries go to four chains as there (chain m of the entries
+// m, m + 4, .., the last ne mod 4 to chain 0), one lane each.
+struct BxArgs {
+  const int32_t *zb, *ze;    // first block of a warp [cs * 16], block ends of its passes [cs * 16][passes]
+  const float4* z32;
+  const double2* z64;
+  const uint2* zcol;
+  const int32_t* pcol;       // triangle blocks [5][ne]
+  const float* pval;
+  const double* b;
+  double* x;
+  double* ring;
+  float2* rs;
+  int32_t L, alpha, warm, rows, passes, ne, maxit;
+  double tol;
+  int32_t* status;
+  double* resid;
+};
+constexpr int kBxPc = 5;
+
+struct LdB32 {  // FP32, one chain per lane
+  const float4* v;
+  const uint2* c;
+  const float* X;
+  struct Block {
+    float4 v;
+    uint2 c;
+  };
+  struct Acc {
+    float a;
+    __device__ __forceinline__ void zero() { a = 0.f; }
+    __device__ __forceinline__ float fold() {
+      float s = a;
+      s += __shfl_xor_sync(0xffffffffu, s, 1);
+      return s + __shfl_xor_sync(0xffffffffu, s, 2);
+    }
+  };
+  __device__ __forceinline__ void seek(int b, int lane) {
+    v += (int64_t)b * 32 + lane;
+    c += (int64_t)b * 32 + lane;
+  }
+  __device__ __forceinline__ void skip() {
+    v += kScDepth * 32;
+    c += kScDepth * 32;
+  }
+  __device__ __forceinline__ void load(Block& k, int i) const {
+    k.v = __ldg(v + i * 32);
+    k.c = __ldg(c + i * 32);
+  }
+  __device__ __forceinline__ void mul(const Block& k, Acc& s) const {
+    s.a = fmaf(k.v.x, X[k.c.x & 0xffff], s.a);
+    s.a = fmaf(k.v.y, X[k.c.x >> 16], s.a);
+    s.a = fmaf(k.v.z, X[k.c.y & 0xffff], s.a);
+    s.a = fmaf(k.v.w, X[k.c.y >> 16], s.a);
+  }
+};
+
+// The warp's rows times the gathered vector into out[local row] (shared memory).
+template <class Ld, class Out>
+__device__ __forceinline__ void bx_spmv(Ld ld, int b, int tot, int ends, int gpc, int warp, int lane, Out* out) {
+  typename Ld::Block buf[kScDepth];
+  asm volatile("" : "+r"(b));
+  int left = tot - b, g = warp, gend = __shfl_sync(0xffffffffu, ends, 0), gleft = gend - b, j = 0;
+  ld.seek(b, lane);
+#pragma unroll
+  for (int i = 0; i < kScDepth; ++i) ld.load(buf[i], i);
+  typename Ld::Acc acc;
+  acc.zero();
+  for (; left > 0; left -= kScDepth) {
+    ld.skip();
+#pragma unroll
+    for (int i = 0; i < kScDepth; ++i) {
+      ld.mul(buf[i], acc);
+      ld.load(buf[i], i);
+      if (--gleft == 0) {
+        const Out s = acc.fold();
+        acc.zero();
+        // (the zero blocks behind a warp's last group may close a pass without one)
+        if ((lane & 3) == 0 && g < gpc) out[g * 8 + (lane >> 2)] = s;
+        g += kScWarps;
+        const int g2 = __shfl_sync(0xffffffffu, ends, ++j & 31);
+        gleft = g2 - gend;
+        gend = g2;
+      }
+    }
+  }
+}
+
+struct __align__(16) BxShared {  // (sums are sent as 16-byte pairs)
+  double red[kScWarps][2];
+  double slots[2][16][2];
+  double rr, inv, sc;
+  float alf, omf, beta;
+  int stop;
+};
+
+template <int RPT>
+__global__ void __launch_bounds__(kScThreads) k_bicgstab_x(const BxArgs A) {
+  extern __shared__ __align__(16) float bx_sm[];
+  __shared__ BxShared sm;
+  int nb, rank;
+  asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(nb));
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31, W = rank * kScWarps + warp;
+  const int ne = A.ne, r0 = rank * A.rows, nr = max(0, min(ne - r0, A.rows));
+  const int nx = (ne + 3) & ~3, gpc = (A.rows + 7) / 8;
+  float *Xa = bx_sm, *Xb = bx_sm + nx;                     // p then s; P p then P s
+  double* prod = reinterpret_cast<double*>(bx_sm + 2 * nx);  // a product's rows
+  float* prodf = reinterpret_cast<float*>(prod);
+  const int zb = A.zb[W], zends = lane < A.passes ? A.ze[W * A.passes + lane] : 0;
+  const int ztot = __shfl_sync(0xffffffffu, zends, A.passes - 1);
+  auto sync = [&]() {
+    if (nb == 1) {
+      __syncthreads();
+    } else {
+      asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+      asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+  };
+  auto own = [&](int e) { return t + e * kScThreads < nr; };
+  auto row = [&](int e) { return r0 + t + e * kScThreads; };
+  auto push = [&](float* X, const float(&v)[RPT]) {
+    const uint32_t a = (uint32_t)__cvta_generic_to_shared(X);
+#pragma unroll 1
+    for (int k = 0; k < nb; ++k) {
+      int r = rank + k;
+      if (r >= nb) r -= nb;
+      const uint32_t d = sc_mapa(a, r);
+#pragma unroll
+      for (int e = 0; e < RPT; ++e)
+        if (own(e)) sc_st(d + 4 * row(e), v[e]);
+    }
+  };
+  // Sums over all rows of a and b, with the additions of the tree that k_bicgstab
+  // takes for either; warp 0 gets both and runs f on them before the CTA goes on.
+  int phase = 0;
+  auto sums = [&](double a, double b, auto f) {
+    const bool up = lane & 16;
+    double k = (up ? b : a) + __shfl_xor_sync(0xffffffffu, up ? a : b, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) k += __shfl_down_sync(0xffffffffu, k, o);
+    if ((lane & 15) == 0) sm.red[warp][lane >> 4] = k;
+    __syncthreads();
+    const int ph = phase++ & 1;
+    if (warp == 0) {
+      double u = sm.red[lane & 15][lane >> 4];
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) u += __shfl_down_sync(0xffffffffu, u, o);
+      const double u0 = __shfl_sync(0xffffffffu, u, 0), u1 = __shfl_sync(0xffffffffu, u, 16);
+      const uint32_t dst = sc_mapa((uint32_t)__cvta_generic_to_shared(&sm.slots[ph][rank][0]), lane < nb ? lane : 0);
+      if (lane < nb) sc_st64(dst, u0, u1);
+    }
+    sync();
+    if (warp == 0) {
+      double u = (lane & 15) < nb ? sm.slots[ph][lane & 15][lane >> 4] : 0.0;
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) u += __shfl_down_sync(0xffffffffu, u, o);
+      f(__shfl_sync(0xffffffffu, u, 0), __shfl_sync(0xffffffffu, u, 16));
+    }
+    __syncthreads();
+  };
+  auto spmv32 = [&](float(&v)[RPT]) {  // Z0 Xb
+    bx_spmv(LdB32{A.z32, A.zcol, Xb}, zb, ztot, zends, gpc, warp, lane, prodf);
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < RPT; ++e) v[e] = own(e) ? prodf[t + e * kScThreads] : 0.f;
+  };
+  auto spmv64 = [&](const double* x, double(&v)[RPT]) {  // Z0 x, x in global memory
+    bx_spmv(LdZ64{A.z64, A.zcol, x}, zb, ztot, zends, gpc, warp, lane, prod);
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < RPT; ++e) v[e] = own(e) ? prod[t + e * kScThreads] : 0.0;
+    __syncthreads();  // prod is written again before the next barrier of the sums
+  };
+  auto precond = [&](float(&v)[RPT]) {  // the triangle blocks times Xa
+#pragma unroll
+    for (int e = 0; e < RPT; ++e) {
+      float s = 0.f;
+      if (own(e)) {
+        const int i = row(e);
+#pragma unroll
+        for (int k = 0; k < kBxPc; ++k)
+          s += __ldg(A.pval + (int64_t)k * ne + i) * Xa[__ldg(A.pcol + (int64_t)k * ne + i)];
+      }
+      v[e] = s;
+    }
+  };
+  const int L = A.L, msk = A.L - 1;
+  double x[RPT], b[RPT], r64[RPT], z[RPT];
+#pragma unroll
+  for (int e = 0; e < RPT; ++e) {
+    b[e] = x[e] = 0.0;
+    if (!own(e)) continue;
+    b[e] = A.b[row(e)];
+    double x0 = 0.0;
+    if (A.warm) {
+      const double* J = A.ring + (int64_t)row(e) * L;
+      int bt = A.alpha - 2;  // J^{alpha-2}, J^{alpha-3}, ... (zero before step 0)
+      double j1 = bt >= 0 ? J[bt & msk] : 0.0, j2 = bt >= 1 ? J[(bt - 1) & msk] : 0.0;
+      double j3 = bt >= 2 ? J[(bt - 2) & msk] : 0.0, j4 = bt >= 3 ? J[(bt - 3) & msk] : 0.0;
+      x0 = 4.0 * j1 - 6.0 * j2 + 4.0 * j3 - j4;
+    }
+    x[e] = x0;
+    if (A.warm != 2) A.x[row(e)] = x0;
+  }
+  sync();
+  if (A.warm == 2) {
+    // keep the guess in A.x only if its FP64 residual is smaller (a NaN never is)
+    double g[RPT], qg = 0.0, qc = 0.0;
+    spmv64(A.x, z);
+#pragma unroll
+    for (int e = 0; e < RPT; ++e) {
+      g[e] = own(e) ? A.x[row(e)] : 0.0;
+      const double rg = b[e] - z[e];
+      if (own(e)) qg += rg * rg;
+    }
+    sync();  // every CTA has read the guess
+#pragma unroll
+    for (int e = 0; e < RPT; ++e)
+      if (own(e)) A.x[row(e)] = x[e];
+    sync();
+    spmv64(A.x, z);
+#pragma unroll
+    for (int e = 0; e < RPT; ++e) {
+      const double rc = b[e] - z[e];
+      if (own(e)) qc += rc * rc;
+    }
+    sums(qg, qc, [&](double a, double c) { sm.stop = a < c ? 1 : 0; });
+    const bool keep = sm.stop;
+    if (keep) {
+#pragma unroll
+      for (int e = 0; e < RPT; ++e) {
+        x[e] = g[e];
+        if (own(e)) A.x[row(e)] = g[e];
+      }
+    }
+    if (rank == 0 && t == 0) A.status[keep ? 8 : 9] += 1;
+    sync();
+  }
+  // scalars of warp 0 (its lanes hold the same values)
+  double bb = -1.0, rr = 0.0, rho = 0.0, rho_old = 1.0, alp = 1.0, om = 1.0, want2 = 0.0, tin2 = 0.0;
+  int inner_total = 0;
+  bool conv = false;
+#pragma unroll 1
+  for (int outer = 0; outer < 8; ++outer) {
+    double q0 = 0.0, q1 = 0.0;
+    spmv64(A.x, z);
+#pragma unroll
+    for (int e = 0; e < RPT; ++e) {
+      const double ri = b[e] - z[e];
+      r64[e] = own(e) ? ri : 0.0;
+      if (own(e)) {
+        q0 += ri * ri;
+        q1 += b[e] * b[e];
+      }
+    }
+    sums(q0, q1, [&](double a, double c) {
+      rr = a;
+      if (bb < 0) bb = c;
+      sm.stop = rr <= A.tol * A.tol * bb;
+      sm.inv = 1.0 / sqrt(rr);
+      sm.sc = sqrt(rr);
+      want2 = 0.25 * A.tol * A.tol * bb / rr;
+    });
+    if (sm.stop) {
+      conv = true;
+      break;
+    }
+    if (inner_total >= A.maxit) break;
+    const double inv = sm.inv, sc = sm.sc;
+    float r[RPT], rh[RPT], p[RPT], v[RPT], s[RPT], tt[RPT], ph[RPT], sh[RPT], d[RPT];
+    q0 = 0.0;
+#pragma unroll
+    for (int e = 0; e < RPT; ++e) {
+      float ri = (float)(r64[e] * inv);  // unit-norm right-hand side
+      r[e] = rh[e] = own(e) ? ri : 0.f;
+      p[e] = v[e] = d[e] = 0.f;
+      if (own(e)) q0 += (double)ri * ri;
+    }
+    sums(q0, 0.0, [&](double a, double) {
+      rho = a;
+      rho_old = alp = om = 1.0;
+      tin2 = fmin(fmax(want2, kScInner2), 0.25) * a;
+      sm.stop = rho == 0.0;
+      sm.beta = (float)((rho / rho_old) * (alp / om));
+      sm.omf = (float)om;
+    });
+#pragma unroll 1
+    for (int it = 0; it < kScInnerMax && inner_total < A.maxit; ++it) {
+      ++inner_total;
+      if (sm.stop) break;  // rho = 0
+      const float beta = sm.beta;
+      float omf = sm.omf;
+#pragma unroll
+      for (int e = 0; e < RPT; ++e) p[e] = r[e] + beta * (p[e] - omf * v[e]);
+      push(Xa, p);
+      sync();
+      precond(ph);
+      push(Xb, ph);
+      sync();
+      spmv32(v);
+      q0 = 0.0;
+#pragma unroll
+      for (int e = 0; e < RPT; ++e)
+        if (own(e)) q0 += (double)(rh[e] * v[e]);
+      sums(q0, 0.0, [&](double a, double) {
+        sm.stop = a == 0.0;
+        alp = rho / a;
+        sm.alf = (float)alp;
+      });
+      if (sm.stop) break;
+      const float alf = sm.alf;
+      q0 = 0.0;
+#pragma unroll
+      for (int e = 0; e < RPT; ++e) {
+        float si = r[e] - alf * v[e];
+        s[e] = si;
+        if (own(e)) q0 += (double)(si * si);
+      }
+      push(Xa, s);  // published by the barrier of the sums
+      sums(q0, 0.0, [&](double a, double) { sm.stop = a <= tin2; });
+      if (sm.stop) {
+#pragma unroll
+        for (int e = 0; e < RPT; ++e) d[e] += alf * ph[e];
+        break;
+      }
+      precond(sh);
+      push(Xb, sh);
+      sync();
+      spmv32(tt);
+      q0 = q1 = 0.0;
+#pragma unroll
+      for (int e = 0; e < RPT; ++e)
+        if (own(e)) {
+          q0 += (double)(tt[e] * s[e]);
+          q1 += (double)(tt[e] * tt[e]);
+        }
+      sums(q0, q1, [&](double a, double c) {
+        sm.stop = c == 0.0;
+        om = a / c;
+        sm.omf = (float)om;
+      });
+      if (sm.stop) break;
+      omf = sm.omf;
+      q0 = q1 = 0.0;
+#pragma unroll
+      for (int e = 0; e < RPT; ++e) {
+        d[e] += alf * ph[e] + omf * sh[e];
+        float ri = s[e] - omf * tt[e];
+        r[e] = ri;
+        if (own(e)) {
+          q0 += (double)(ri * ri);
+          q1 += (double)(rh[e] * ri);
+        }
+      }
+      sums(q0, q1, [&](double a, double c) {
+        rho_old = rho;
+        rho = c;
+        sm.stop = (a <= tin2 || om == 0.0 ? 1 : 0) | (rho == 0.0 ? 2 : 0);
+        sm.beta = (float)((rho / rho_old) * (alp / om));
+      });
+      if (sm.stop & 1) break;
+    }
+#pragma unroll
+    for (int e = 0; e < RPT; ++e) {
+      x[e] += sc * (double)d[e];
+      if (own(e)) A.x[row(e)] = x[e];
+    }
+    sync();
+  }
+#pragma unroll
+  for (int e = 0; e < RPT; ++e)
+    if (own(e)) {
+      const int64_t o = (int64_t)row(e) * L + ((A.alpha - 1) & msk);
+      A.ring[o] = x[e];
+      if (A.rs) A.rs[o] = split_pair(x[e]);
+    }
+  if (rank == 0 && t == 0) {
+    A.status[0] = inner_total;
+    A.status[6] = 0;
+    A.status[1] = conv ? 1 : 0;
+    A.status[2] += conv ? 0 : 1;
+    A.status[3] += inner_total;
+    A.resid[0] = bb > 0 ? sqrt(rr / bb) : 0.0;
+  }
+  sync();  // no CTA leaves while another may still store into its shared memory
+}
+
 struct ScPlan {
   int cs = 0, gpc = 0, passes = 0, npad = 0;
   int32_t *perm = nullptr, *ab = nullptr, *ae = nullptr, *zb = nullptr, *ze = nullptr, *pb = nullptr, *pe = nullptr;
@@ -636,6 +1033,9 @@ struct ScPlan {
   double2* zval = nullptr;
   uint2 *acol = nullptr, *zcol = nullptr, *pcol = nullptr;
   double* w64 = nullptr;
+  bool bx = false;                 // k_bicgstab_x: rows per CTA, Z0's FP32 blocks, the triangle blocks are the context's
+  int rows = 0;
+  float4* z32 = nullptr;
 };
 
 }  // namespace tdbem
@@ -990,7 +1390,123 @@ tdbem_status tdbem_sc_build(tdbem_ctx* c, int want, const std::vector<int32_t>& 
   return c->sc ? TDBEM_OK : TDBEM_ENOMEM;
 }
 
+using BxFn = void (*)(BxArgs);
+static BxFn bx_fn(int rows) {
+  return rows <= kScThreads ? k_bicgstab_x<1> : rows <= 2 * kScThreads ? k_bicgstab_x<2> : k_bicgstab_x<4>;
+}
+static size_t bx_smem(int ne, int rows) { return (size_t)((ne + 3) / 4 * 4) * 2 * sizeof(float) + (size_t)(rows + 8) * sizeof(double); }
+
+// The plan of k_bicgstab_x: Z0 in edge order in blocks of 8 rows x 16 entries, the
+// four chains of a row in its four lanes.
+tdbem_status tdbem_bx_build(tdbem_ctx* c, int want, const std::vector<int32_t>& zp, const std::vector<int32_t>& zc,
+                            const std::vector<double>& zv) {
+  const int ne = (int)c->ne;
+  ScPlan P;
+  P.bx = true;
+  for (P.cs = want; P.cs >= 1; P.cs >>= 1) {
+    P.rows = (ne + P.cs - 1) / P.cs;
+    P.gpc = (P.rows + 7) / 8;
+    P.passes = (P.gpc + kScWarps - 1) / kScWarps;
+    if (P.rows > 4 * kScThreads || ne > 65535 || bx_smem(ne, P.rows) > 200 * 1024) return TDBEM_OK;
+    const BxFn fn = bx_fn(P.rows);
+    TDBEM_CUDA_TRY(c, cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    TDBEM_CUDA_TRY(c, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at;
+    sc_config(&cfg, &at, P.cs, P.cs, bx_smem(ne, P.rows), c->stream);
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) == cudaSuccess && n > 0) break;
+    cudaGetLastError();
+  }
+  if (P.cs < 1) return TDBEM_OK;
+  // lane m's chain of a row of n entries: m, m + 4, .. below 4 (n / 4), then (m = 0) the rest
+  auto chain = [](int n, int m) { return n / 4 + (m == 0 ? n % 4 : 0); };
+  std::vector<int32_t> begin(P.cs * kScWarps), end((size_t)P.cs * kScWarps * P.passes);
+  std::vector<float4> z32;
+  std::vector<double2> z64;
+  std::vector<uint2> zcol;
+  int32_t nblk = 0;
+  for (int fill = 0; fill < 2; ++fill) {
+    if (fill) {
+      z32.assign((size_t)(nblk + kScDepth) * 32, make_float4(0, 0, 0, 0));
+      z64.assign((size_t)(nblk + kScDepth) * 64, make_double2(0, 0));
+      zcol.assign((size_t)(nblk + kScDepth) * 32, make_uint2(0, 0));
+    }
+    int32_t blk = 0;
+    for (int k = 0; k < P.cs; ++k)
+      for (int w = 0; w < kScWarps; ++w) {
+        const int32_t b0 = blk;
+        begin[k * kScWarps + w] = blk;
+        for (int j = 0; j < P.passes; ++j) {
+          const int g = j * kScWarps + w;
+          if (g < P.gpc) {
+            int most = 1;
+            for (int t = 0; t < 8; ++t) {
+              const int li = g * 8 + t, i = k * P.rows + li;
+              if (li >= P.rows || i >= ne) continue;
+              const int n = zp[i + 1] - zp[i];
+              for (int m = 0; m < 4; ++m) {
+                most = std::max(most, chain(n, m));
+                for (int u = 0; fill && u < chain(n, m); ++u) {
+                  const int q = zp[i] + (u < n / 4 ? 4 * u + m : n / 4 * 4 + u - n / 4);
+                  const size_t o = (size_t)(blk + u / 4) * 128 + (t * 4 + m) * 4 + u % 4;
+                  ((float*)z32.data())[o] = (float)zv[q];
+                  ((double*)z64.data())[o] = zv[q];
+                  ((uint16_t*)zcol.data())[o] = (uint16_t)zc[q];
+                }
+              }
+            }
+            blk += (most + 3) / 4;
+          }
+          if (j == P.passes - 1)
+            while ((blk - b0) % kScDepth) ++blk;
+          end[(size_t)(k * kScWarps + w) * P.passes + j] = blk;
+        }
+      }
+    nblk = blk;
+  }
+  tdbem_status s;
+  if ((s = sc_upload(c, &P.zb, begin)) || (s = sc_upload(c, &P.ze, end)) || (s = sc_upload(c, &P.z32, z32)) ||
+      (s = sc_upload(c, &P.zval, z64)) || (s = sc_upload(c, &P.zcol, zcol)))
+    return s;
+  c->sc = new (std::nothrow) ScPlan(P);
+  return c->sc ? TDBEM_OK : TDBEM_ENOMEM;
+}
+
+static tdbem_status bx_solve(tdbem_ctx* c, int32_t alpha, int32_t warm) {
+  const ScPlan& P = *c->sc;
+  BxArgs A;
+  A.zb = P.zb;
+  A.ze = P.ze;
+  A.z32 = P.z32;
+  A.z64 = P.zval;
+  A.zcol = P.zcol;
+  A.pcol = c->d_pc_col;
+  A.pval = c->d_pc_val;
+  A.b = c->d_R;
+  A.x = c->d_J;
+  A.ring = c->d_Jring;
+  A.rs = c->d_rs;
+  A.L = c->L;
+  A.alpha = alpha;
+  A.warm = warm;
+  A.rows = P.rows;
+  A.passes = P.passes;
+  A.ne = (int32_t)c->ne;
+  A.maxit = c->p.solve_maxit;
+  A.tol = c->p.solve_tol;
+  A.status = c->d_status;
+  A.resid = c->d_dots;
+  c->cluster = P.cs;
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute at;
+  sc_config(&cfg, &at, P.cs, P.cs, bx_smem((int)c->ne, P.rows), c->stream);
+  TDBEM_CUDA_TRY(c, cudaLaunchKernelEx(&cfg, bx_fn(P.rows), A));
+  return TDBEM_OK;
+}
+
 tdbem_status tdbem_sc_solve(tdbem_ctx* c, int32_t alpha, int32_t warm) {
+  if (c->sc->bx) return bx_solve(c, alpha, warm);
   const ScPlan& P = *c->sc;
   ScArgs A;
   A.perm = P.perm;
