@@ -101,6 +101,7 @@ struct FmmLevel {
   float* d_pack = nullptr;          // packed moments of this level's event (tensor-core M2L)
   float* d_pkinv = nullptr;         // their inverse row scales (FP16 form)
   float* d_opinv = nullptr;         // inverse operator scales (FP16 form)
+  unsigned long long* d_live = nullptr;  // K chunks of each operator row tile that are not zero
   // FP16 form with P <= 256: the resident-operator kernel k_m2l_res, its work
   // units {gemm, 128-row tile, first 128-column tile, column tiles} (lag-1
   // units first) and its packed FP16 hi/lo moments
@@ -1675,7 +1676,8 @@ tdbem_status tdbem_build_fast(tdbem_ctx* c) {
                                                                       a_kernel_derivs(c->p.a_deriv), c->p.s_interp,
                                                                       c->p.t_interp, L.ops);
       TDBEM_CUDA_TRY(c, cudaGetLastError());
-      if (c->p.m2l_prec != TDBEM_P_FP32 && (s = tdbem_m2l_tc_images(c, L.ops, L.nop, P, c->p.m2l_prec, &L.ops_img, &L.d_opinv)))
+      if (c->p.m2l_prec != TDBEM_P_FP32 && (s = tdbem_m2l_tc_images(c, L.ops, L.nop, P, c->p.m2l_prec, &L.ops_img, &L.d_opinv,
+                                                                      &L.d_live)))
         return s;
     }
     // moment and local-coefficient storage (march state and history_eval state)
@@ -1817,7 +1819,7 @@ tdbem_status tdbem_build_fast(tdbem_ctx* c) {
           if (v < 2)
             s = tdbem_m2l_tc(c, v + 1, L.d_gemm, L.d_tiles_tc[v], L.ntiles_tc[v], L.ops_img, P, pt, PS, L.d_pO,
                              L.d_pC, L.d_psym, F->d_smap, L.d_pack, 0, L.loc, L.Q, c->R, c->p.m2l_prec, L.d_opinv,
-                             L.d_pkinv, F->d_err);
+                             L.d_pkinv, L.d_live, F->d_err);
           else
             s = tdbem_m2l_res(c, L.d_gemm, L.d_units, 0, L.nunits, L.ops_img, P, pt, PS, L.d_pO, L.d_pC, L.d_psym,
                               F->d_smap, L.d_pk16, 0, L.loc, L.Q, c->R, L.d_opinv, L.d_pkinv, F->d_err, 0);
@@ -1926,7 +1928,7 @@ static tdbem_status far_events(tdbem_ctx* c, int32_t alpha, const double* ring, 
         } else {
           tdbem_status s = tdbem_m2l_tc(c, L.tc_mt, L.d_gemm, L.d_tiles_tc[v] + t0, n, L.ops_img, P, pt, PS, L.d_pO,
                                         L.d_pC, L.d_psym, F->d_smap, L.d_pack, k, LOC(l), L.Q, R, c->p.m2l_prec,
-                                        L.d_opinv, L.d_pkinv, F->d_err);
+                                        L.d_opinv, L.d_pkinv, L.d_live, F->d_err);
           if (s) return s;
         }
         c->prof_end(5, e);

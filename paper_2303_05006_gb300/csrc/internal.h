@@ -276,12 +276,12 @@ tdbem_status tdbem_fast_check(tdbem_ctx* c);
 tdbem_status tdbem_m2l_tc(tdbem_ctx* c, int mt, const int4* gemm, const int4* tiles, int ntiles, const uint4* img, int P,
                           int pt, int PS, const int32_t* pO, const int32_t* pC, const int16_t* psym,
                           const int16_t* smap, const float* pk, int k, float* loc, int Q, int R, int prec,
-                          const float* opinv, const float* pkinv, int32_t* err);
+                          const float* opinv, const float* pkinv, const unsigned long long* live, int32_t* err);
 // pkinv: the FP16 form's per-row inverse scales (null for the other forms)
 tdbem_status tdbem_m2l_pack(tdbem_ctx* c, const int32_t* cS, const int16_t* csym, int ncombo, const int16_t* smap,
                             const float* mom, int k, int R, int PS, int pt, float* pk, float* pkinv);
 tdbem_status tdbem_m2l_tc_images(tdbem_ctx* c, const float* ops, int nop, int P, int prec, uint4** img,
-                                 float** opinv);
+                                 float** opinv, unsigned long long** live);
 // the FP16 form with the operator rows resident in shared memory (P <= 256):
 // units [u0, u0 + n) of the level's list, and the FP16 hi/lo moment pack it reads
 tdbem_status tdbem_m2l_res(tdbem_ctx* c, const int4* gemm, const int4* units, int u0, int n, const uint4* img, int P,

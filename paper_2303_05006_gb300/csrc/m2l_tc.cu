@@ -173,13 +173,36 @@ __global__ void k_m2l_images(const float* ops, int64_t nunits, int P, int nrt, i
   img[t] = part == 0 ? hi : lo;
 }
 
+// Bit ch of live[(op * 2 + kind) * nrt + rt]: whether the operator's 128 rows of
+// row tile rt have an entry in the K chunk ch (KC columns) that is not zero.  The
+// kernels vanish ahead of the light cone (c tau < r), so about a sixth of the blocks
+// of 128 x 64 are exactly zero at p = 4, and none of their operands need be read: the M2L
+// of the p = 6 march of 1,920 RWG went from 1102 to 1039 us a step.
+// One block per (operator, row tile).
+__global__ void k_m2l_live(const float* ops, int P, int nrt, int KC, unsigned long long* live) {
+  __shared__ unsigned long long m;
+  if (threadIdx.x == 0) m = 0;
+  __syncthreads();
+  const int64_t opk = blockIdx.x / nrt;
+  const int rt = (int)(blockIdx.x - opk * nrt), r1 = min(P, (rt + 1) * kTileM);
+  unsigned long long mine = 0;
+  for (int r = rt * kTileM + (int)(threadIdx.x >> 5); r < r1; r += (int)(blockDim.x >> 5))
+    for (int c = threadIdx.x & 31; c < P; c += 32)
+      if (ops[(opk * P + r) * P + c] != 0.f) mine |= 1ull << (c / KC);
+  atomicOr(&m, mine);
+  __syncthreads();
+  if (threadIdx.x == 0) live[blockIdx.x] = m;
+}
+
 // prec: 1 = TF32, 2 = BF16, 3 = BF16 x 3, 4 = TF32 x 3 (split: hi*hi + hi*lo + lo*hi)
+// live: the K chunks that hold anything (k_m2l_live; null: all), the others are passed over
 template <int kMT>
 __global__ void __launch_bounds__(kThreads) k_m2l_tc(const int4* gemm, const int4* tiles, const uint4* img, int P,
                                                      int pt, int PS, const int32_t* pO, const int32_t* pC,
                                                      const int16_t* psym, const int16_t* smap, const float* pk,
                                                      int k, float* loc, int Q, int R, int prec, const float* opinv,
-                                                     const float* pkinv, int32_t* err) {
+                                                     const float* pkinv, const unsigned long long* live,
+                                                     int32_t* err) {
   constexpr uint32_t kTmemCols = 128 * kMT;
   extern __shared__ __align__(1024) uint8_t dsm[];
   __shared__ int64_t src_off[kTileN];
@@ -193,6 +216,17 @@ __global__ void __launch_bounds__(kThreads) k_m2l_tc(const int4* gemm, const int
   uint8_t* tB = dsm + 2 * kMT * kTileBytes;
   uint8_t* tB2 = tB + kTileBytes;
 
+  // the K chunks to do (at most 64 when live is given); an operator that is zero adds nothing
+  unsigned long long todo = ~0ull;
+  if (live) {
+    const int4 t0 = tiles[blockIdx.x], g0 = gemm[t0.x];
+    const int nrt0 = (P + kTileM - 1) / kTileM;
+    const unsigned long long* l = live + ((int64_t)g0.x * 2 + (g0.w & 0xff)) * nrt0;
+    todo = 0;
+    for (int mt = 0; mt < kMT; ++mt)
+      if (t0.y * kMT + mt < nrt0) todo |= l[t0.y * kMT + mt];
+    if (todo == 0) return;  // the whole CTA, nothing allocated yet
+  }
   // the symmetry node maps, staged in shared memory when they fit
   const int16_t* smp = smap;
   if (48 * PS * 2 <= kSmapSmem) {
@@ -279,9 +313,16 @@ __global__ void __launch_bounds__(kThreads) k_m2l_tc(const int4* gemm, const int
       }
     }
   };
-  if (vec) load_b(0);
-  for (int ch = 0; ch < nchunks && ok; ++ch) {
-    const int k0 = ch * KC;
+  // chunk after chunk ch of those to do (nchunks: none)
+  auto after = [&](int ch) {
+    if (!live) return ch + 1;
+    const unsigned long long m = ch >= 63 ? 0ull : todo >> (ch + 1);
+    return m ? ch + __ffsll((long long)m) : nchunks;
+  };
+  int ch = after(-1);
+  if (vec) load_b(ch);
+  for (int it = 0; ch < nchunks && ok; ++it) {
+    const int next = after(ch), k0 = ch * KC;
     // operator rows: the pre-converted images of this chunk (hi and lo parts
     // contiguous, nparts x 16 KB per row tile) brought in by the TMA bulk-copy
     // engine while the threads gather the moments; the previous chunk's MMAs
@@ -323,7 +364,7 @@ __global__ void __launch_bounds__(kThreads) k_m2l_tc(const int4* gemm, const int
     __syncthreads();
     bool a_ok = true;
     if (tid == 0) {
-      a_ok = mbar_wait(ab, (uint32_t)(ch & 1));
+      a_ok = mbar_wait(ab, (uint32_t)(it & 1));
       a_pending = !a_ok;
       tc_fence_after();
       const uint32_t b0 = smem_u32(tB), b1 = smem_u32(tB2);
@@ -331,7 +372,7 @@ __global__ void __launch_bounds__(kThreads) k_m2l_tc(const int4* gemm, const int
         const uint32_t a0 = smem_u32(dsm + 2 * mt * kTileBytes), a1 = a0 + kTileBytes;
         const uint32_t d = tmem + (uint32_t)(mt * kTileN);  // this row tile's accumulator columns
         for (int s = 0; s < 4; ++s) {
-          uint32_t acc = (ch > 0 || s > 0) ? 1u : 0u;
+          uint32_t acc = (it > 0 || s > 0) ? 1u : 0u;
           uint32_t off = 256u * s;  // two core matrices (32 bytes of K) per instruction
           if (tf) {
             mma_tf32(d, make_desc(a0 + off), make_desc(b0 + off), idesc, acc);
@@ -350,19 +391,20 @@ __global__ void __launch_bounds__(kThreads) k_m2l_tc(const int4* gemm, const int
       }
       mma_commit(mb);
     }
-    if (vec && ch + 1 < nchunks) load_b(ch + 1);
+    if (vec && next < nchunks) load_b(next);
     // the next chunk overwrites the tiles: wait for the MMAs to finish; the
     // verdict is made uniform across the CTA before anyone acts on it
     // (with no MMA issued the commit arrives at once)
-    bool mine = mbar_wait(mb, (uint32_t)(ch & 1)) && a_ok;
+    bool mine = mbar_wait(mb, (uint32_t)(it & 1)) && a_ok;
     ok = __syncthreads_and(mine) != 0;
     if (!ok) {
       if (tid == 0) atomicExch(err, 1);
       // give the tensor core and the copy engine a last bounded chance to
       // drain this chunk before TMEM is freed and the CTA exits
-      mbar_wait(mb, (uint32_t)(ch & 1));
-      if (tid == 0 && a_pending) mbar_wait(ab, (uint32_t)(ch & 1));
+      mbar_wait(mb, (uint32_t)(it & 1));
+      if (tid == 0 && a_pending) mbar_wait(ab, (uint32_t)(it & 1));
     }
+    ch = next;
   }
   tc_fence_after();
   // With both 128-row tiles of a 256-row operator in this CTA every column's
@@ -843,7 +885,8 @@ template <int kMT>
 static tdbem_status launch_m2l_tc(tdbem_ctx* c, const int4* gemm, const int4* tiles, int ntiles, const uint4* img,
                                   int P, int pt, int PS, const int32_t* pO, const int32_t* pC, const int16_t* psym,
                                   const int16_t* smap, const float* pk, int k, float* loc, int Q, int R, int prec,
-                                  const float* opinv, const float* pkinv, int32_t* err) {
+                                  const float* opinv, const float* pkinv, const unsigned long long* live,
+                                  int32_t* err) {
   using namespace tdbem;
   static bool attr = false;
   if (!attr) {
@@ -854,7 +897,7 @@ static tdbem_status launch_m2l_tc(tdbem_ctx* c, const int4* gemm, const int4* ti
   if (ntiles == 0) return TDBEM_OK;
   const size_t smem = smem_tiles<kMT>() + (48 * PS * 2 <= kSmapSmem ? 48 * PS * 2 : 0) + 1024;
   k_m2l_tc<kMT><<<ntiles, kThreads, smem, c->stream>>>(gemm, tiles, img, P, pt, PS, pO, pC, psym, smap, pk, k, loc,
-                                                        Q, R, prec, opinv, pkinv, err);
+                                                        Q, R, prec, opinv, pkinv, live, err);
   TDBEM_CUDA_TRY(c, cudaGetLastError());
   return TDBEM_OK;
 }
@@ -862,23 +905,25 @@ static tdbem_status launch_m2l_tc(tdbem_ctx* c, const int4* gemm, const int4* ti
 tdbem_status tdbem_m2l_tc(tdbem_ctx* c, int mt, const int4* gemm, const int4* tiles, int ntiles, const uint4* img,
                           int P, int pt, int PS, const int32_t* pO, const int32_t* pC, const int16_t* psym,
                           const int16_t* smap, const float* pk, int k, float* loc, int Q, int R, int prec,
-                          const float* opinv, const float* pkinv, int32_t* err) {
+                          const float* opinv, const float* pkinv, const unsigned long long* live, int32_t* err) {
   if (mt == 2)
     return launch_m2l_tc<2>(c, gemm, tiles, ntiles, img, P, pt, PS, pO, pC, psym, smap, pk, k, loc, Q, R, prec, opinv,
-                            pkinv, err);
+                            pkinv, live, err);
   return launch_m2l_tc<1>(c, gemm, tiles, ntiles, img, P, pt, PS, pO, pC, psym, smap, pk, k, loc, Q, R, prec, opinv,
-                          pkinv, err);
+                          pkinv, live, err);
 }
 
 // Convert the FP32 operators of one level into the tensor-core images read by
 // k_m2l_tc (allocated here, owned by the context).  The FP16 form scales each
 // operator by a power of two first; *opinv (allocated here, 2 nop floats)
-// then holds the inverse scales, and is null for the other forms.
+// then holds the inverse scales, and is null for the other forms.  *live: see
+// k_m2l_live (null where an operator has more than 64 chunks).
 tdbem_status tdbem_m2l_tc_images(tdbem_ctx* c, const float* ops, int nop, int P, int prec, uint4** img,
-                                 float** opinv) {
+                                 float** opinv, unsigned long long** live) {
   using namespace tdbem;
   *img = nullptr;
   *opinv = nullptr;
+  *live = nullptr;
   if (nop == 0) return TDBEM_OK;
   const int fmt = (prec == TDBEM_P_TF32 || prec == TDBEM_P_TF32X3) ? kFmtTf32
                                                                       : (prec == TDBEM_P_F16X3 ? kFmtF16 : kFmtBf16);
@@ -888,6 +933,11 @@ tdbem_status tdbem_m2l_tc_images(tdbem_ctx* c, const float* ops, int nop, int P,
   const int64_t nunits = (int64_t)nop * 2 * nrt * nch * nparts * 1024;
   tdbem_status s = c->dalloc(img, nunits);
   if (s) return s;
+  if (nch <= 64) {
+    if ((s = c->dalloc(live, (size_t)nop * 2 * nrt))) return s;
+    k_m2l_live<<<(unsigned)(nop * 2 * nrt), 256, 0, c->stream>>>(ops, P, nrt, KC, *live);
+    TDBEM_CUDA_TRY(c, cudaGetLastError());
+  }
   float* scale = nullptr;
   if (fmt == kFmtF16) {
     if ((s = c->dalloc(&scale, 2 * (int64_t)nop)) || (s = c->dalloc(opinv, 2 * (int64_t)nop))) return s;
