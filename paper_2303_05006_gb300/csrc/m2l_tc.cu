@@ -11,12 +11,14 @@
 // two 128-row halves of a 256-row operator), so each gathered moment chunk
 // feeds both: the gathers, which bound the kernel, are halved per output.
 // Operand tiles live in shared
-// memory in the canonical K-major layout without swizzle: 8-row x 16-byte
-// core matrices, LBO = 128 B between core matrices along K, SBO = 1024 B
-// between 8-row groups.  With 128 bytes of K per row that layout is a linear
-// run of 1024 16-byte units, unit u holding row 8(u >> 6) + (u & 7) and K
-// bytes 16((u >> 3) & 7) .. +15, so thread t writing units t, t+256, ... is
-// free of bank conflicts.  The operators are converted once at setup into
+// memory K-major in the 128-byte swizzle: rows of 128 bytes of K, a row's
+// 16-byte units XORed with row mod 8, so a tile is a linear run of 1024 units,
+// unit u holding row u >> 3 and K bytes 16((u & 7) ^ (row & 7)) .. +15.  Eight
+// neighbouring threads then read one row's 128 bytes from global memory in one
+// line and write them free of bank conflicts.  (In the layout without swizzle eight
+// neighbours belong to eight rows: every 16-byte gather touched 32 lines a warp, and
+// L1 was 72% busy.  M2L per step: p = 6, 1,920 RWG 1039 -> 982 us; p = 4, 16
+// right-hand sides, 4,608 RWG 800 -> 660 us.)  The operators are converted once at setup into
 // exactly these images (TF32, BF16, or hi and lo parts for the split forms,
 // zero-padded past P) and brought in by TMA bulk copies (cp.async.bulk, one
 // per row tile and chunk, completing on an mbarrier); the moment columns
@@ -159,8 +161,8 @@ __global__ void k_m2l_images(const float* ops, int64_t nunits, int P, int nrt, i
   const int64_t opk = rest / nrt;  // op * 2 + kind
   const bool tf = fmt == kFmtTf32;
   const int E = tf ? 4 : 8, KC = tf ? 32 : 64;
-  const int row = rt * kTileM + unit_row(u);
-  const int k0 = ch * KC + unit_k16(u) * E;
+  const int row = rt * kTileM + sw_row(u);
+  const int k0 = ch * KC + sw_k16(u) * E;
   const float sc = scale ? scale[opk] : 1.f;
   float x[8];
 #pragma unroll
@@ -204,7 +206,8 @@ __global__ void __launch_bounds__(kThreads) k_m2l_tc(const int4* gemm, const int
                                                      const float* pkinv, const unsigned long long* live,
                                                      int32_t* err) {
   constexpr uint32_t kTmemCols = 128 * kMT;
-  extern __shared__ __align__(1024) uint8_t dsm[];
+  extern __shared__ __align__(1024) uint8_t dsm_raw[];
+  uint8_t* dsm = dsm_raw + (1024 - (smem_u32(dsm_raw) & 1023)) % 1024;  // swizzled tiles: 1024-byte boundaries
   __shared__ int64_t src_off[kTileN];
   __shared__ int64_t dst_off[kTileN];
   __shared__ int32_t map_off[kTileN];
@@ -298,13 +301,16 @@ __global__ void __launch_bounds__(kThreads) k_m2l_tc(const int4* gemm, const int
   constexpr int kU = 1024 / kThreads;
   const bool vec = (P & 3) == 0;
   float4 v[kU][2];
+  // this thread's units tid + 256 j: rows (tid >> 3) + 32 j, one 16-byte column of K
+  int64_t so_j[kU];
+#pragma unroll
+  for (int j = 0; j < kU; ++j) so_j[j] = src_off[sw_row(tid + j * kThreads)];
   auto load_b = [&](int chunk) {
     const int kb = chunk * KC;
 #pragma unroll
     for (int j = 0; j < kU; ++j) {
-      const int u = tid + j * kThreads;
-      const int64_t so = src_off[unit_row(u)];
-      const int kk = kb + unit_k16(u) * E;
+      const int64_t so = so_j[j];
+      const int kk = kb + sw_k16(tid) * E;
 #pragma unroll
       for (int g = 0; g < 2; ++g) {
         const int kq = kk + 4 * g;
@@ -349,8 +355,8 @@ __global__ void __launch_bounds__(kThreads) k_m2l_tc(const int4* gemm, const int
       }
     } else {
       for (int u = tid; u < 1024; u += kThreads) {
-        const int64_t so = src_off[unit_row(u)];
-        const int kk = k0 + unit_k16(u) * E;
+        const int64_t so = src_off[sw_row(u)];
+        const int kk = k0 + sw_k16(u) * E;
         float x[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) x[e] = (so >= 0 && e < E && kk + e < P) ? pk[so + kk + e] : 0.f;
@@ -373,18 +379,18 @@ __global__ void __launch_bounds__(kThreads) k_m2l_tc(const int4* gemm, const int
         const uint32_t d = tmem + (uint32_t)(mt * kTileN);  // this row tile's accumulator columns
         for (int s = 0; s < 4; ++s) {
           uint32_t acc = (it > 0 || s > 0) ? 1u : 0u;
-          uint32_t off = 256u * s;  // two core matrices (32 bytes of K) per instruction
+          uint32_t off = 32u * s;  // 32 bytes of K per instruction
           if (tf) {
-            mma_tf32(d, make_desc(a0 + off), make_desc(b0 + off), idesc, acc);
+            mma_tf32(d, make_desc_sw128(a0 + off), make_desc_sw128(b0 + off), idesc, acc);
             if (split) {
-              mma_tf32(d, make_desc(a0 + off), make_desc(b1 + off), idesc, 1u);
-              mma_tf32(d, make_desc(a1 + off), make_desc(b0 + off), idesc, 1u);
+              mma_tf32(d, make_desc_sw128(a0 + off), make_desc_sw128(b1 + off), idesc, 1u);
+              mma_tf32(d, make_desc_sw128(a1 + off), make_desc_sw128(b0 + off), idesc, 1u);
             }
           } else {
-            mma_f16(d, make_desc(a0 + off), make_desc(b0 + off), idesc, acc);
+            mma_f16(d, make_desc_sw128(a0 + off), make_desc_sw128(b0 + off), idesc, acc);
             if (split) {
-              mma_f16(d, make_desc(a0 + off), make_desc(b1 + off), idesc, 1u);
-              mma_f16(d, make_desc(a1 + off), make_desc(b0 + off), idesc, 1u);
+              mma_f16(d, make_desc_sw128(a0 + off), make_desc_sw128(b1 + off), idesc, 1u);
+              mma_f16(d, make_desc_sw128(a1 + off), make_desc_sw128(b0 + off), idesc, 1u);
             }
           }
         }
@@ -580,7 +586,7 @@ constexpr int kResThreads = 288;
 constexpr int kResMaxCh = 4;  // K chunks of 64 halves: P <= 256
 constexpr int kResStages = 3;
 constexpr int kResStage = 2 * kTileBytes;
-constexpr int kResSmem = kResMaxCh * 2 * kTileBytes + kResStages * kResStage;
+constexpr int kResSmem = kResMaxCh * 2 * kTileBytes + kResStages * kResStage + 1024;  // 1024: the tiles' boundary
 
 struct ResUnit {
   int g, rt, ct0, nct;
@@ -610,7 +616,8 @@ __global__ void __launch_bounds__(kResThreads, 1)
     k_m2l_res(const int4* gemm, const int4* units, int nunits, const uint4* img, int P, int P16, int pt, int PS,
               const int32_t* pO, const int32_t* pC, const int16_t* psym, const int16_t* smap, const __half* pk16,
               int k, float* loc, int Q, int R, const float* opinv, const float* pkinv, int32_t* err) {
-  extern __shared__ __align__(1024) uint8_t dsm[];
+  extern __shared__ __align__(1024) uint8_t dsm_raw[];
+  uint8_t* dsm = dsm_raw + (1024 - (smem_u32(dsm_raw) & 1023)) % 1024;
   uint8_t* sA = dsm;                               // [chunk][hi, lo][16 KB]
   uint8_t* sB = dsm + kResMaxCh * 2 * kTileBytes;  // [stage][hi, lo][16 KB]
   __shared__ __align__(8) uint64_t a_full, b_full[kResStages], mma_done[kResStages], acc_full[2], acc_empty[2];
@@ -650,17 +657,17 @@ __global__ void __launch_bounds__(kResThreads, 1)
   if (warp < 4) {
     // ---- producers: cp.async of the packed FP16 moments into the ring ----
     const int tid = threadIdx.x;
-    const int k16 = (tid >> 3) & 7;  // this thread's 16-byte column along K (the same for its 8 units)
+    const int k16 = sw_k16(tid);  // this thread's 16-byte column along K (the same for its 8 units)
     int64_t g_item = 0;
     for (int u = blockIdx.x; u < nunits && !abort_flag; u += gridDim.x) {
       const ResUnit U = res_unit(gemm, units, u, R);
       for (int t = 0; t < U.nct && !abort_flag; ++t) {
         const int col0 = (U.ct0 + t) * kTileN;
-        // units tid + 128 i (i < 8) of a part: row ((tid >> 6) + 2 i) * 8 + (tid & 7)
+        // units tid + 128 i (i < 8) of a part: row (tid >> 3) + 16 i
         int64_t srow[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-          const int r = (((tid >> 6) + 2 * i) << 3) | (tid & 7);
+          const int r = sw_row(tid + 128 * i);
           const int gcol = col0 + r;
           srow[i] = -1;
           if (gcol < U.ncol) {
@@ -754,10 +761,10 @@ __global__ void __launch_bounds__(kResThreads, 1)
             const uint32_t o0 = smem_u32(sA + ch * 2 * kTileBytes), o1 = o0 + kTileBytes;
             const uint32_t m0 = smem_u32(sB + st * kResStage), m1 = m0 + kTileBytes;
             for (int ks = 0; ks < 4; ++ks) {
-              const uint32_t off = 256u * ks;  // 32 bytes of K per instruction
-              mma_f16(d, make_desc(m0 + off), make_desc(o0 + off), idesc, (ch > 0 || ks > 0) ? 1u : 0u);
-              mma_f16(d, make_desc(m1 + off), make_desc(o0 + off), idesc, 1u);
-              mma_f16(d, make_desc(m0 + off), make_desc(o1 + off), idesc, 1u);
+              const uint32_t off = 32u * ks;  // 32 bytes of K per instruction
+              mma_f16(d, make_desc_sw128(m0 + off), make_desc_sw128(o0 + off), idesc, (ch > 0 || ks > 0) ? 1u : 0u);
+              mma_f16(d, make_desc_sw128(m1 + off), make_desc_sw128(o0 + off), idesc, 1u);
+              mma_f16(d, make_desc_sw128(m0 + off), make_desc_sw128(o1 + off), idesc, 1u);
             }
             mma_commit(smem_u32(&mma_done[st]));
             if (ch == nch - 1) mma_commit(smem_u32(&acc_full[b]));

@@ -90,6 +90,22 @@ __device__ __forceinline__ void bulk_reduce_add_f32(float* dst, uint32_t src, ui
                : "memory");
 }
 
+// Shared-memory descriptor of an operand tile in the 128-byte swizzle (K-major, rows of 128 bytes, the
+// 16-byte units of a row XORed with row mod 8; 1024 bytes between 8-row groups):
+// the tile starts on a 1024-byte boundary, K steps of 32 bytes add to the address.
+__device__ __forceinline__ uint64_t make_desc_sw128(uint32_t saddr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr & 0x3FFFF) >> 4);
+  d |= (uint64_t)1 << 16;                    // leading byte offset: not used in a swizzled K-major tile
+  d |= (uint64_t)(1024 >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)2 << 61;                    // 128-byte swizzle
+  return d;
+}
+// its 16-byte unit u: row and 16-byte column along K
+__device__ __forceinline__ int sw_row(int u) { return u >> 3; }
+__device__ __forceinline__ int sw_k16(int u) { return (u & 7) ^ ((u >> 3) & 7); }
+
 // 16-byte unit u of a tile with 128 bytes of K per row: its row and its
 // 16-byte column along K (the unit's byte offset in the tile is 16 u)
 __device__ __forceinline__ int unit_row(int u) { return ((u >> 6) << 3) | (u & 7); }
