@@ -52,6 +52,7 @@
 
 namespace tdbem {
 
+constexpr int kStreamRun = 4;  // most tiles of one k_m2l_stream CTA: the steps beside it get SMs between CTAs
 constexpr int kNC = 7;  // moment components: A x,y,z | phi | mag x,y,z
 
 struct FmmLevel {
@@ -104,17 +105,16 @@ struct FmmLevel {
   unsigned long long* d_live = nullptr;  // K chunks of each operator row tile that are not zero
   // FP16 form with P <= 256: the resident-operator kernel k_m2l_res, its work
   // units {gemm, 128-row tile, first 128-column tile, column tiles} (lag-1
-  // units first) and its packed FP16 hi/lo moments
+  // units first); the packed hi and lo moments of it and of k_m2l_stream
   bool res_ok = false;  // eligible (FP16 form, P <= 256)
   bool res = false;     // chosen by the autotuner
-  float res_ms = 0.f;   // autotuner: mean time of one M2L event of the resident kernel
+  bool str_ok = false, str = false;  // the same two for k_m2l_stream (split forms; tiles of d_tiles_tc[1])
   int4* d_units = nullptr;
   int nunits = 0, nunits_urgent = 0;
-  __half* d_pk16 = nullptr;
+  uint8_t* d_pks = nullptr;
   cudaEvent_t ev_defer = nullptr;   // recorded on the side stream after a deferred M2L
   bool defer_pending = false;       // host: a deferred M2L not yet waited for
   int tc_mt = 1;
-  float tc_ms[2] = {0.f, 0.f};     // autotuner: mean time of one M2L event per shape
   double flops_event = 0;         // M2L flops of one gating event
   // time tables: source/target factors for offsets i = 0..M-1
   float* d_tsrc = nullptr;        // [M][pt]  l_n(s_i)
@@ -1647,6 +1647,11 @@ tdbem_status tdbem_build_fast(tdbem_ctx* c) {
       if (L.nunits)
         TDBEM_CUDA_TRY(c, cudaMemcpy(L.d_units, units.data(), L.nunits * sizeof(int4), cudaMemcpyHostToDevice));
     }
+    // The split forms with both operands streamed (k_m2l_stream).  It keeps a second pack of the moments, so a
+    // context with a memory budget stays with the kernels above; its masks hold 64 K chunks.
+    L.str_ok = (c->p.m2l_prec == TDBEM_P_BF16X3 || c->p.m2l_prec == TDBEM_P_TF32X3 ||
+                c->p.m2l_prec == TDBEM_P_F16X3) &&
+               tdbem_m2l_chunks(P, c->p.m2l_prec) <= 64 && c->p.max_device_bytes == 0;
     if (qmax >= 255) {
       c->set_error("fast: too many time intervals per interaction");
       return TDBEM_EINVAL;
@@ -1772,15 +1777,15 @@ tdbem_status tdbem_build_fast(tdbem_ctx* c) {
       const int64_t npk = std::max<int64_t>(1, (int64_t)F->lev[l].ncombo * 2 * c->R * kNC * P);
       if ((s = c->dalloc(&F->lev[l].d_pack, npk))) return s;
       TDBEM_CUDA_TRY(c, cudaMemset(F->lev[l].d_pack, 0, npk * sizeof(float)));
+      const int64_t nrow = std::max<int64_t>(1, (int64_t)F->lev[l].ncombo * 2 * c->R * kNC);
+      if (F->lev[l].res_ok || F->lev[l].str_ok) {
+        const int64_t nb = nrow * 2 * 128 * tdbem_m2l_chunks(P, c->p.m2l_prec);
+        if ((s = c->dalloc(&F->lev[l].d_pks, nb))) return s;
+        TDBEM_CUDA_TRY(c, cudaMemset(F->lev[l].d_pks, 0, nb));
+      }
       if (c->p.m2l_prec == TDBEM_P_F16X3) {
-        const int64_t nrow = std::max<int64_t>(1, (int64_t)F->lev[l].ncombo * 2 * c->R * kNC);
         if ((s = c->dalloc(&F->lev[l].d_pkinv, nrow))) return s;
         TDBEM_CUDA_TRY(c, cudaMemset(F->lev[l].d_pkinv, 0, nrow * sizeof(float)));
-        if (F->lev[l].res_ok) {
-          const int64_t n16 = nrow * 2 * ((P + 63) / 64 * 64);
-          if ((s = c->dalloc(&F->lev[l].d_pk16, n16))) return s;
-          TDBEM_CUDA_TRY(c, cudaMemset(F->lev[l].d_pk16, 0, n16 * sizeof(__half)));
-        }
       }
     }
   }
@@ -1796,8 +1801,8 @@ tdbem_status tdbem_build_fast(tdbem_ctx* c) {
   TDBEM_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   // M2L autotuner: time one gating event of each level with every kernel
   // shape that applies -- the tiled kernel with one or two 128-row operator
-  // tiles per CTA, and for the FP16 form with P <= 256 the resident-operator
-  // kernel -- on this context's own operators, pairs and right-hand sides,
+  // tiles per CTA, for the FP16 form with P <= 256 the resident-operator
+  // kernel, and for the split forms the streamed one -- on this context's own operators, pairs and right-hand sides,
   // and keep the fastest.  The packed moments are still zero, so the trial
   // launches add nothing to the local coefficients.
   if (c->p.m2l_prec != TDBEM_P_FP32 && c->p.m2l_tile_rows != 0) {
@@ -1812,7 +1817,9 @@ tdbem_status tdbem_build_fast(tdbem_ctx* c) {
     for (int l = 2; l <= F->lmax; ++l) {
       FmmLevel& L = F->lev[l];
       if (!L.ntiles_tc[0]) continue;
-      for (int v = 0; v < (L.res_ok ? 3 : 2); ++v) {
+      float ms[4] = {};  // tiled with 128 and 256 rows, resident, streamed
+      for (int v = 0; v < 4; ++v) {
+        if ((v == 2 && !L.res_ok) || (v == 3 && !L.str_ok)) continue;
         const int reps = 3;
         for (int it = -1; it < reps; ++it) {  // one untimed launch first
           if (it == 0) TDBEM_CUDA_TRY(c, cudaEventRecord(e0, c->stream));
@@ -1820,19 +1827,27 @@ tdbem_status tdbem_build_fast(tdbem_ctx* c) {
             s = tdbem_m2l_tc(c, v + 1, L.d_gemm, L.d_tiles_tc[v], L.ntiles_tc[v], L.ops_img, P, pt, PS, L.d_pO,
                              L.d_pC, L.d_psym, F->d_smap, L.d_pack, 0, L.loc, L.Q, c->R, c->p.m2l_prec, L.d_opinv,
                              L.d_pkinv, L.d_live, F->d_err);
+          else if (v == 3)
+            s = tdbem_m2l_stream(c, L.d_gemm, L.d_tiles_tc[1], L.ntiles_tc[1], L.ops_img, P, pt, PS, L.d_pO, L.d_pC,
+                                 L.d_psym, F->d_smap, L.d_pks, 0, L.loc, L.Q, c->R, c->p.m2l_prec, L.d_opinv,
+                                 L.d_pkinv, L.d_live, F->d_err, kStreamRun);
           else
             s = tdbem_m2l_res(c, L.d_gemm, L.d_units, 0, L.nunits, L.ops_img, P, pt, PS, L.d_pO, L.d_pC, L.d_psym,
-                              F->d_smap, L.d_pk16, 0, L.loc, L.Q, c->R, L.d_opinv, L.d_pkinv, F->d_err, 0);
+                              F->d_smap, L.d_pks, 0, L.loc, L.Q, c->R, L.d_opinv, L.d_pkinv, F->d_err, 0);
           if (s) return s;
         }
         TDBEM_CUDA_TRY(c, cudaEventRecord(e1, c->stream));
         TDBEM_CUDA_TRY(c, cudaEventSynchronize(e1));
-        float ms = 0.f;
-        TDBEM_CUDA_TRY(c, cudaEventElapsedTime(&ms, e0, e1));
-        (v < 2 ? L.tc_ms[v] : L.res_ms) = ms / reps;
+        TDBEM_CUDA_TRY(c, cudaEventElapsedTime(&ms[v], e0, e1));
       }
-      L.tc_mt = L.tc_ms[1] < L.tc_ms[0] ? 2 : 1;
-      L.res = L.res_ok && L.res_ms < std::min(L.tc_ms[0], L.tc_ms[1]);
+      const float tc = std::min(ms[0], ms[1]);
+      L.tc_mt = ms[1] < ms[0] ? 2 : 1;
+      L.res = L.res_ok && ms[2] < tc;
+      L.str = L.str_ok && ms[3] < (L.res ? ms[2] : tc);
+      if (L.str) {
+        L.res = false;
+        L.tc_mt = 2;  // its tiles
+      }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -1903,9 +1918,10 @@ static tdbem_status far_events(tdbem_ctx* c, int32_t alpha, const double* ring, 
       const int v = L.tc_mt - 1;
       if (tc) {
         cudaEvent_t e = c->prof_begin(8);
-        tdbem_status s = L.res ? tdbem_m2l_pack_f16(c, L.d_cS, L.d_csym, L.ncombo, F->d_smap, MOM(l), k, R, PS, pt,
-                                                    L.d_pk16, L.d_pkinv)
-                               : tdbem_m2l_pack(c, L.d_cS, L.d_csym, L.ncombo, F->d_smap, MOM(l), k, R, PS, pt,
+        tdbem_status s = L.res || L.str
+                             ? tdbem_m2l_pack_split(c, L.d_cS, L.d_csym, L.ncombo, F->d_smap, MOM(l), k, R, PS, pt,
+                                                    c->p.m2l_prec, L.d_pks, L.d_pkinv)
+                             : tdbem_m2l_pack(c, L.d_cS, L.d_csym, L.ncombo, F->d_smap, MOM(l), k, R, PS, pt,
                                                 L.d_pack, L.d_pkinv);
         if (s) return s;
         c->prof_end(8, e);
@@ -1922,8 +1938,13 @@ static tdbem_status far_events(tdbem_ctx* c, int32_t alpha, const double* ring, 
           // the deferred launch on the side stream runs one CTA per unit, so
           // that the hardware interleaves it with the steps it overlaps
           tdbem_status s = tdbem_m2l_res(c, L.d_gemm, L.d_units, t0, n, L.ops_img, P, pt, PS, L.d_pO, L.d_pC,
-                                         L.d_psym, F->d_smap, L.d_pk16, k, LOC(l), L.Q, R, L.d_opinv, L.d_pkinv,
+                                         L.d_psym, F->d_smap, L.d_pks, k, LOC(l), L.Q, R, L.d_opinv, L.d_pkinv,
                                          F->d_err, (F->side && c->stream == F->side) ? -1 : 0);
+          if (s) return s;
+        } else if (L.str) {
+          tdbem_status s = tdbem_m2l_stream(c, L.d_gemm, L.d_tiles_tc[v] + t0, n, L.ops_img, P, pt, PS, L.d_pO, L.d_pC,
+                                            L.d_psym, F->d_smap, L.d_pks, k, LOC(l), L.Q, R, c->p.m2l_prec,
+                                            L.d_opinv, L.d_pkinv, L.d_live, F->d_err, kStreamRun);
           if (s) return s;
         } else {
           tdbem_status s = tdbem_m2l_tc(c, L.tc_mt, L.d_gemm, L.d_tiles_tc[v] + t0, n, L.ops_img, P, pt, PS, L.d_pO,

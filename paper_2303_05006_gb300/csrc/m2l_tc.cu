@@ -568,7 +568,7 @@ __global__ void k_m2l_pack_scaled(const int32_t* cS, const int16_t* csym, int64_
 // the unit's operator rows in once (hi and lo parts of every K chunk, by TMA
 // bulk copies) and streams the column tiles through a three-stage ring:
 //  - warps 0-3 copy each (column tile, K chunk) item of the packed moments,
-//    already scaled and split into FP16 hi and lo by k_m2l_pack_f16, into a
+//    already scaled and split into FP16 hi and lo by k_m2l_pack_split, into a
 //    ring stage with 16-byte cp.async copies, up to three items ahead of the
 //    tensor core; each thread's copies arrive on the stage's barrier when
 //    they land (cp.async.mbarrier.arrive), so the producers never wait on
@@ -612,9 +612,48 @@ __device__ __forceinline__ ResUnit res_unit(const int4* gemm, const int4* units,
   return U;
 }
 
+// Adds 16 consecutive operator rows rb .. (v, times ci) of one column, whose coefficients start at dst_off
+// (negative: a column past the GEMM), at the nodes that the column's symmetry map sm gives: pt consecutive
+// rows (the time nodes of one spatial node) are contiguous.  An even pt makes P even, so pairs are aligned.
+__device__ __forceinline__ void add_rows(const uint32_t (&v)[16], float* loc, int64_t dst_off, const int16_t* sm,
+                                         int rb, int P, int pt, float ci) {
+  if (dst_off < 0) {
+  } else if (pt == 4) {
+#pragma unroll
+    for (int gi = 0; gi < 4; ++gi) {
+      const int r = rb + 4 * gi;
+      if (r < P) {
+        float* dst = loc + dst_off + (int64_t)sm[r >> 2] * 4;
+        atomicAdd((float4*)dst,
+                  make_float4(__uint_as_float(v[4 * gi]) * ci, __uint_as_float(v[4 * gi + 1]) * ci,
+                              __uint_as_float(v[4 * gi + 2]) * ci, __uint_as_float(v[4 * gi + 3]) * ci));
+      }
+    }
+  } else if ((pt & 1) == 0) {
+#pragma unroll
+    for (int jj = 0; jj < 16; jj += 2) {
+      const int r = rb + jj;
+      if (r < P) {
+        const int ap = r / pt, m = r - ap * pt;
+        atomicAdd((float2*)(loc + dst_off + (int64_t)sm[ap] * pt + m),
+                  make_float2(__uint_as_float(v[jj]) * ci, __uint_as_float(v[jj + 1]) * ci));
+      }
+    }
+  } else {
+#pragma unroll
+    for (int jj = 0; jj < 16; ++jj) {
+      const int r = rb + jj;
+      if (r < P) {
+        const int ap = r / pt, m = r - ap * pt;
+        atomicAdd(loc + dst_off + (int64_t)sm[ap] * pt + m, __uint_as_float(v[jj]) * ci);
+      }
+    }
+  }
+}
+
 __global__ void __launch_bounds__(kResThreads, 1)
-    k_m2l_res(const int4* gemm, const int4* units, int nunits, const uint4* img, int P, int P16, int pt, int PS,
-              const int32_t* pO, const int32_t* pC, const int16_t* psym, const int16_t* smap, const __half* pk16,
+    k_m2l_res(const int4* gemm, const int4* units, int nunits, const uint4* img, int P, int nch, int pt, int PS,
+              const int32_t* pO, const int32_t* pC, const int16_t* psym, const int16_t* smap, const uint8_t* pk,
               int k, float* loc, int Q, int R, const float* opinv, const float* pkinv, int32_t* err) {
   extern __shared__ __align__(1024) uint8_t dsm_raw[];
   uint8_t* dsm = dsm_raw + (1024 - (smem_u32(dsm_raw) & 1023)) % 1024;
@@ -624,7 +663,7 @@ __global__ void __launch_bounds__(kResThreads, 1)
   __shared__ uint32_t tmem_base;
   __shared__ volatile int abort_flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nch = P16 / 64, nrt = (P + kTileM - 1) / kTileM;
+  const int nrt = (P + kTileM - 1) / kTileM, prow_bytes = nch * 128;
   if (threadIdx.x == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&a_full)));
     for (int i = 0; i < kResStages; ++i) {
@@ -673,7 +712,7 @@ __global__ void __launch_bounds__(kResThreads, 1)
           if (gcol < U.ncol) {
             const int pr = U.pbase + gcol / (U.nk * R), rem = gcol % (U.nk * R);
             const int64_t prow = (((int64_t)pC[pr] * 2 + U.var) * R + rem / U.nk) * kNCmp + U.c0 + rem % U.nk;
-            srow[i] = prow * 2 * P16;
+            srow[i] = prow * 2 * prow_bytes;
           }
         }
         for (int ch = 0; ch < nch && !abort_flag; ++ch, ++g_item) {
@@ -691,7 +730,7 @@ __global__ void __launch_bounds__(kResThreads, 1)
             for (int i = 0; i < 8; ++i) {
               const int uu = tid + 128 * i;
               const bool v = srow[i] >= 0;
-              const __half* src = v ? pk16 + srow[i] + part * P16 + ch * 64 + k16 * 8 : pk16;
+              const uint8_t* src = v ? pk + srow[i] + part * prow_bytes + ch * 128 + k16 * 16 : pk;
               cp_async16_zfill(base + part * kTileBytes + uu * 16, src, v ? 16u : 0u);
             }
           // arrive on the stage's barrier once this thread's copies have landed
@@ -819,29 +858,7 @@ __global__ void __launch_bounds__(kResThreads, 1)
                 "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
               : "r"(addr));
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-          const int rb = row0 + j0;  // operator row of v[0]
-          if (dst_off < 0) {
-          } else if (pt == 4) {
-#pragma unroll
-            for (int gi = 0; gi < 4; ++gi) {
-              const int r = rb + 4 * gi;
-              if (r < P) {
-                float* dst = loc + dst_off + (int64_t)smap[map_off + (r >> 2)] * 4;
-                atomicAdd((float4*)dst, make_float4(__uint_as_float(v[4 * gi]) * ci, __uint_as_float(v[4 * gi + 1]) * ci,
-                                                    __uint_as_float(v[4 * gi + 2]) * ci,
-                                                    __uint_as_float(v[4 * gi + 3]) * ci));
-              }
-            }
-          } else {
-#pragma unroll
-            for (int jj = 0; jj < 16; ++jj) {
-              const int r = rb + jj;
-              if (r < P) {
-                const int ap = r / pt, m = r - ap * pt;
-                atomicAdd(loc + dst_off + (int64_t)smap[map_off + ap] * pt + m, __uint_as_float(v[jj]) * ci);
-              }
-            }
-          }
+          add_rows(v, loc, dst_off, smap + map_off, row0 + j0, P, pt, ci);
         }
         tc_fence_before();
         mbar_arrive(smem_u32(&acc_empty[b]));
@@ -853,13 +870,266 @@ __global__ void __launch_bounds__(kResThreads, 1)
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256u));
 }
 
-// Packed moments of the FP16 form for k_m2l_res: row (as in k_m2l_pack) scaled
-// by a power of two (k_m2l_pack_scaled) and split into FP16 hi and lo parts,
-// pk16[(row * 2 + part) * P16 + e], zero past P up to P16 (a multiple of 64).
-// One warp per row.
-__global__ void k_m2l_pack_f16(const int32_t* cS, const int16_t* csym, int64_t nrows, const int16_t* smap,
-                               const float* mom, int k, int R, int PS, int pt, int P16, __half* pk16,
-                               float* pkinv) {
+// ---------------------------------------------------------------------------
+// The split forms with both operands streamed.
+//
+// A tile is 256 operator rows (two 128-row tiles) by 128 columns.  Per 128 bytes
+// of K it takes 96 KB of operands (operator hi and lo 64 KB, moments hi and lo
+// 32 KB) and 12 MMAs of 128 x 256 x 32 bytes, about as long as the operands take
+// from L2, so the two have to overlap.  k_m2l_tc converts the moments between its loads
+// and its MMAs and waits for each chunk's MMAs before it asks for the next operator
+// rows; with two CTAs per SM the tensor pipe was 33% busy at p = 6.  Here the moments come
+// packed as hi and lo parts (k_m2l_pack_split), and the roles of k_m2l_res run over a ring of
+// two 96 KB stages: warps 0-3 copy the moment columns (cp.async) and thread 0 the
+// operator tiles (bulk copies), one warp issues the MMAs, warps 5-8 drain one of two
+// 256-column accumulators while the other fills.  A CTA does `run` tiles, `side` (one per SM)
+// apart, so that the CTAs at work at one time hold neighbouring tiles, which share operator rows
+// and moment columns in L2 (with `run` consecutive tiles per CTA L2 hit 36% of the reads, not 72%).
+// Every wait is bounded as in k_m2l_res.  M2L per step, before and after: TF32x3, p = 6,
+// 1,920 RWG 982 -> 722 us; TF32x3, p = 4, sphere and cube, 12,864 RWG 311 -> 233 us (asking for the operator
+// chunks in L2 four chunks early made both slower).
+constexpr int kStrStages = 2;
+constexpr int kStrStage = 6 * kTileBytes;  // operator hi (256 rows), operator lo, moments hi, moments lo
+constexpr int kStrSmem = kStrStages * kStrStage + 1024;
+
+struct StrTile {
+  int op, kind, q, nk, c0, var, ncol, pbase, rt0, nmt, col0;
+  unsigned long long todo;  // K chunks that hold anything (k_m2l_live)
+};
+__device__ __forceinline__ StrTile str_tile(const int4* gemm, const int4* tiles, const unsigned long long* live, int u,
+                                            int R, int nrt) {
+  StrTile T;
+  const int4 tl = tiles[u];
+  const int4 gd = gemm[tl.x];
+  T.op = gd.x;
+  T.pbase = gd.y;
+  T.kind = gd.w & 0xff;
+  T.q = (gd.w >> 8) & 0xff;
+  T.var = T.q == ((gd.w >> 16) & 0xff) ? 1 : 0;
+  T.nk = T.kind == 0 ? 3 : 4;
+  T.c0 = T.kind == 0 ? 0 : 3;
+  T.ncol = gd.z * T.nk * R;
+  T.rt0 = 2 * tl.y;
+  T.nmt = min(2, nrt - T.rt0);
+  T.col0 = tl.z * kTileN;
+  const unsigned long long* l = live + ((int64_t)T.op * 2 + T.kind) * nrt + T.rt0;
+  T.todo = l[0] | (T.nmt > 1 ? l[1] : 0ull);
+  return T;
+}
+
+__global__ void __launch_bounds__(kResThreads, 1)
+    k_m2l_stream(const int4* gemm, const int4* tiles, int ntiles, int run, int side, const uint4* img, int P, int nch, int fmt,
+                 int pt, int PS, const int32_t* pO, const int32_t* pC, const int16_t* psym, const int16_t* smap,
+                 const uint8_t* pk, int k, float* loc, int Q, int R, const float* opinv, const float* pkinv,
+                 const unsigned long long* live, int32_t* err) {
+  extern __shared__ __align__(1024) uint8_t dsm_raw[];
+  uint8_t* dsm = dsm_raw + (1024 - (smem_u32(dsm_raw) & 1023)) % 1024;
+  __shared__ __align__(8) uint64_t a_full[kStrStages], b_full[kStrStages], mma_done[kStrStages], acc_full[2],
+      acc_empty[2];
+  __shared__ uint32_t tmem_base;
+  __shared__ volatile int abort_flag;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nrt = (P + kTileM - 1) / kTileM, prow_bytes = nch * 128;
+  const int u0 = (int)(blockIdx.x / side) * side * run + (int)(blockIdx.x % side);
+  const int u1 = min(ntiles, u0 + side * run);
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < kStrStages; ++i) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&a_full[i])));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 128;" ::"r"(smem_u32(&b_full[i])));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mma_done[i])));
+    }
+    for (int i = 0; i < 2; ++i) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&acc_full[i])));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 128;" ::"r"(smem_u32(&acc_empty[i])));
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    abort_flag = 0;
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
+                 "r"(512u));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_base;
+  auto fail = [&]() {
+    if (!abort_flag) {
+      abort_flag = 1;
+      atomicExch(err, 1);
+    }
+  };
+
+  if (warp < 4) {
+    // ---- producers ----
+    const int tid = threadIdx.x;
+    const int k16 = sw_k16(tid);  // this thread's 16-byte column along K (the same for its 8 units)
+    int64_t g_item = 0;
+    for (int u = u0; u < u1 && !abort_flag; u += side) {
+      const StrTile T = str_tile(gemm, tiles, live, u, R, nrt);
+      // units tid + 128 i (i < 8) of a part: row (tid >> 3) + 16 i
+      int64_t srow[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int gcol = T.col0 + sw_row(tid + 128 * i);
+        srow[i] = -1;
+        if (gcol < T.ncol) {
+          const int pr = T.pbase + gcol / (T.nk * R), rem = gcol % (T.nk * R);
+          const int64_t prow = (((int64_t)pC[pr] * 2 + T.var) * R + rem / T.nk) * kNCmp + T.c0 + rem % T.nk;
+          srow[i] = prow * 2 * prow_bytes;
+        }
+      }
+      for (unsigned long long m = T.todo; m && !abort_flag; m &= m - 1, ++g_item) {
+        const int ch = __ffsll((long long)m) - 1;
+        const int st = (int)(g_item % kStrStages);
+        const uint32_t ph = (uint32_t)((g_item / kStrStages) & 1);  // this use's phase of the stage
+        // the stage was last read by the MMAs of item g_item - kStrStages
+        if (g_item >= kStrStages && !mbar_wait(smem_u32(&mma_done[st]), ph ^ 1u)) {
+          fail();
+          break;
+        }
+        const uint32_t base = smem_u32(dsm + st * kStrStage);
+        if (tid == 0) {
+          mbar_expect_tx(smem_u32(&a_full[st]), (uint32_t)(T.nmt * 2 * kTileBytes));
+          for (int mt = 0; mt < T.nmt; ++mt) {
+            const uint4* src = img + ((((int64_t)T.op * 2 + T.kind) * nrt + T.rt0 + mt) * nch + ch) * 2 * 1024;
+            bulk_g2s(base + mt * kTileBytes, src, kTileBytes, smem_u32(&a_full[st]));
+            bulk_g2s(base + (2 + mt) * kTileBytes, src + 1024, kTileBytes, smem_u32(&a_full[st]));
+          }
+        }
+#pragma unroll
+        for (int part = 0; part < 2; ++part)
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const bool v = srow[i] >= 0;
+            const uint8_t* src = v ? pk + srow[i] + part * prow_bytes + ch * 128 + k16 * 16 : pk;
+            cp_async16_zfill(base + (4 + part) * kTileBytes + (tid + 128 * i) * 16, src, v ? 16u : 0u);
+          }
+        // arrive on the stage's barrier once this thread's copies have landed
+        asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&b_full[st])) : "memory");
+      }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    // the operator copies of the stages' last uses (long done unless the loop was given up)
+    if (tid == 0)
+      for (int64_t it = g_item - 1; it >= 0 && it >= g_item - kStrStages; --it)
+        mbar_wait(smem_u32(&a_full[it % kStrStages]), (uint32_t)((it / kStrStages) & 1));
+  } else if (warp == 4) {
+    // ---- the MMA issuer (whole warp, verdicts agreed by vote; lane 0 issues) ----
+    auto wait_all = [&](uint64_t* bar, uint32_t parity) {
+      return __all_sync(0xffffffffu, mbar_wait(smem_u32(bar), parity));
+    };
+    int64_t g_item = 0, j = 0;
+    bool stop = false;
+    for (int u = u0; u < u1 && !stop && !__any_sync(0xffffffffu, abort_flag != 0); u += side) {
+      const StrTile T = str_tile(gemm, tiles, live, u, R, nrt);
+      if (!T.todo) continue;
+      const int b = (int)(j & 1);
+      // the accumulator was last drained by the epilogue of tile j - 2
+      if (j >= 2 && !wait_all(&acc_empty[b], (uint32_t)(((j >> 1) - 1) & 1))) {
+        fail();
+        break;
+      }
+      tc_fence_after();
+      const uint32_t d = tmem + (uint32_t)(b * 2 * kTileN);
+      // D[column][operator row]: the moment columns are the M side, 128 or 256 operator rows the N side
+      const uint32_t ef = fmt == kFmtTf32 ? 2u : fmt == kFmtBf16 ? 1u : 0u;
+      const uint32_t idesc = (1u << 4) | (ef << 7) | (ef << 10) | ((uint32_t)((T.nmt * kTileM) >> 3) << 17) | ((uint32_t)(kTileN >> 4) << 24);
+      uint32_t acc = 0;
+      for (unsigned long long m = T.todo; m; m &= m - 1, ++g_item) {
+        const int st = (int)(g_item % kStrStages);
+        const uint32_t ph = (uint32_t)((g_item / kStrStages) & 1);
+        if (!wait_all(&b_full[st], ph) || !wait_all(&a_full[st], ph)) {
+          fail();
+          stop = true;
+          break;
+        }
+        // the producers' copies (generic proxy) are read by the tensor core (async proxy)
+        fence_async_smem();
+        tc_fence_after();
+        if (lane == 0) {
+          const uint32_t o0 = smem_u32(dsm + st * kStrStage), o1 = o0 + 2 * kTileBytes;
+          const uint32_t m0 = o0 + 4 * kTileBytes, m1 = o0 + 5 * kTileBytes;
+          for (int ks = 0; ks < 4; ++ks) {
+            const uint32_t off = 32u * ks;  // 32 bytes of K per instruction
+            const uint64_t dm0 = make_desc_sw128(m0 + off), dm1 = make_desc_sw128(m1 + off);
+            const uint64_t do0 = make_desc_sw128(o0 + off), do1 = make_desc_sw128(o1 + off);
+            if (fmt == kFmtTf32) {
+              mma_tf32(d, dm0, do0, idesc, acc);
+              mma_tf32(d, dm1, do0, idesc, 1u);
+              mma_tf32(d, dm0, do1, idesc, 1u);
+            } else {
+              mma_f16(d, dm0, do0, idesc, acc);
+              mma_f16(d, dm1, do0, idesc, 1u);
+              mma_f16(d, dm0, do1, idesc, 1u);
+            }
+            acc = 1;
+          }
+          mma_commit(smem_u32(&mma_done[st]));
+          if ((m & (m - 1)) == 0) mma_commit(smem_u32(&acc_full[b]));
+        }
+        __syncwarp();
+      }
+      ++j;
+    }
+    // drain: the last commit covers every MMA issued
+    if (g_item > 0) wait_all(&mma_done[(g_item - 1) % kStrStages], (uint32_t)(((g_item - 1) / kStrStages) & 1));
+  } else {
+    // ---- epilogue, as in k_m2l_res: a lane adds its own column's rows ----
+    const int q4 = warp & 3;  // TMEM lane quarter this warp may read
+    int64_t j = 0;
+    for (int u = u0; u < u1 && !__any_sync(0xffffffffu, abort_flag != 0); u += side) {
+      const StrTile T = str_tile(gemm, tiles, live, u, R, nrt);
+      if (!T.todo) continue;
+      const int b = (int)(j & 1);
+      const int gcol = T.col0 + q4 * 32 + lane;  // this lane's column
+      int64_t dst_off = -1;
+      int32_t map_off = 0;
+      float ci = 0.f;
+      if (gcol < T.ncol) {
+        const int pr = T.pbase + gcol / (T.nk * R), rem = gcol % (T.nk * R), rhs = rem / T.nk, c = T.c0 + rem % T.nk;
+        const int64_t prow = (((int64_t)pC[pr] * 2 + T.var) * R + rhs) * kNCmp + c;
+        dst_off = ((((int64_t)pO[pr] * Q + ((k + T.q) % Q)) * R + rhs) * kNCmp + c) * P;
+        map_off = (int32_t)psym[pr] * PS;
+        ci = pkinv ? opinv[T.op * 2 + T.kind] * pkinv[prow] : 1.f;
+      }
+      if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&acc_full[b]), (uint32_t)((j >> 1) & 1)))) {
+        fail();
+        break;
+      }
+      tc_fence_after();
+      const int row0 = T.rt0 * kTileM;
+      for (int j0 = 0; j0 < T.nmt * kTileM; j0 += 16) {
+        __syncwarp();  // the lanes leave the previous group's adds at different points
+        uint32_t v[16];
+        const uint32_t addr = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(b * 2 * kTileN + j0);
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
+            "%14, %15}, [%16];"
+            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+              "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+            : "r"(addr));
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        add_rows(v, loc, dst_off, smap + map_off, row0 + j0, P, pt, ci);
+      }
+      tc_fence_before();
+      mbar_arrive(smem_u32(&acc_empty[b]));
+      ++j;
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u));
+}
+
+// Packed moments of the split forms for k_m2l_res and k_m2l_stream: row (as in
+// k_m2l_pack) as hi and lo parts in the form's type, nch chunks of 128 bytes each,
+// zero past P: pk[(row * 2 + part) * nch * 128 ..].  The FP16 form scales the row by a
+// power of two first (k_m2l_pack_scaled; pkinv is null for the others).  One warp per row.
+__global__ void k_m2l_pack_split(const int32_t* cS, const int16_t* csym, int64_t nrows, const int16_t* smap,
+                                 const float* mom, int k, int R, int PS, int pt, int nch, int fmt, uint8_t* pk,
+                                 float* pkinv) {
   const int64_t row = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (row >= nrows) return;  // whole warps: a warp's lanes share their row
@@ -868,23 +1138,44 @@ __global__ void k_m2l_pack_f16(const int32_t* cS, const int16_t* csym, int64_t n
   const int P = PS * pt;
   const float* base = mom + (((int64_t)cS[combo] * 2 + (k & 1)) * per + rem) * P;
   const int16_t* sm = smap + csym[combo] * PS;
-  float m = 0.f;
-  for (int e = lane; e < P; e += 32) m = fmaxf(m, fabsf(base[(int64_t)sm[e / pt] * pt + e % pt]));
-  for (int d = 16; d > 0; d >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, d));
-  const int sx = f16_scale_exp(m);
-  const float sc = ldexpf(1.f, sx);
-  __half* hi = pk16 + row * 2 * P16;
-  __half* lo = hi + P16;
-  for (int e = lane; e < P16; e += 32) {
-    const float x = e < P ? sc * base[(int64_t)sm[e / pt] * pt + e % pt] : 0.f;
-    const __half h = __float2half_rn(x);
-    hi[e] = h;
-    lo[e] = __float2half_rn(x - __half2float(h));
+  float sc = 1.f;
+  if (pkinv) {
+    float m = 0.f;
+    for (int e = lane; e < P; e += 32) m = fmaxf(m, fabsf(base[(int64_t)sm[e / pt] * pt + e % pt]));
+    for (int d = 16; d > 0; d >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, d));
+    const int sx = f16_scale_exp(m);
+    sc = ldexpf(1.f, sx);
+    if (lane == 0) pkinv[row] = ldexpf(1.f, -sx);
   }
-  if (lane == 0) pkinv[row] = ldexpf(1.f, -sx);
+  uint4* out = (uint4*)(pk + row * 2 * nch * 128);
+  const int E = fmt == kFmtTf32 ? 4 : 8;
+  for (int u = lane; u < nch * 8; u += 32) {
+    float x[8];
+    int node = u * E / pt, t = u * E - node * pt;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      x[e] = e < E && node < PS ? sc * base[(int64_t)sm[node] * pt + t] : 0.f;
+      if (++t == pt) t = 0, ++node;
+    }
+    uint4 hi, lo;
+    split_any(fmt, x, hi, lo);
+    out[u] = hi;
+    out[nch * 8 + u] = lo;
+  }
 }
 
 }  // namespace tdbem
+
+static int split_fmt(int prec) {
+  return (prec == TDBEM_P_TF32 || prec == TDBEM_P_TF32X3) ? tdbem::kFmtTf32
+                                                            : (prec == TDBEM_P_F16X3 ? tdbem::kFmtF16 : tdbem::kFmtBf16);
+}
+
+// K chunks of 128 bytes that a row of P coefficients takes in the form prec
+int tdbem_m2l_chunks(int P, int prec) {
+  const int KC = split_fmt(prec) == tdbem::kFmtTf32 ? 32 : 64;
+  return (P + KC - 1) / KC;
+}
 
 // Launch the tensor-core M2L of one level event with mt (1 or 2) 128-row
 // operator tiles per CTA; tiles must be the list planned for that mt.
@@ -932,8 +1223,7 @@ tdbem_status tdbem_m2l_tc_images(tdbem_ctx* c, const float* ops, int nop, int P,
   *opinv = nullptr;
   *live = nullptr;
   if (nop == 0) return TDBEM_OK;
-  const int fmt = (prec == TDBEM_P_TF32 || prec == TDBEM_P_TF32X3) ? kFmtTf32
-                                                                      : (prec == TDBEM_P_F16X3 ? kFmtF16 : kFmtBf16);
+  const int fmt = split_fmt(prec);
   const bool split = prec == TDBEM_P_TF32X3 || prec == TDBEM_P_BF16X3 || prec == TDBEM_P_F16X3;
   const int KC = fmt == kFmtTf32 ? 32 : 64;
   const int nrt = (P + kTileM - 1) / kTileM, nch = (P + KC - 1) / KC, nparts = split ? 2 : 1;
@@ -982,7 +1272,7 @@ tdbem_status tdbem_m2l_pack(tdbem_ctx* c, const int32_t* cS, const int16_t* csym
 // unit (the hardware then schedules the units among other streams' work).
 tdbem_status tdbem_m2l_res(tdbem_ctx* c, const int4* gemm, const int4* units, int u0, int n, const uint4* img, int P,
                            int pt, int PS, const int32_t* pO, const int32_t* pC, const int16_t* psym,
-                           const int16_t* smap, const __half* pk16, int k, float* loc, int Q, int R,
+                           const int16_t* smap, const uint8_t* pk, int k, float* loc, int Q, int R,
                            const float* opinv, const float* pkinv, int32_t* err, int max_ctas) {
   using namespace tdbem;
   static bool attr = false;
@@ -993,27 +1283,50 @@ tdbem_status tdbem_m2l_res(tdbem_ctx* c, const int4* gemm, const int4* units, in
     attr = true;
   }
   if (n <= 0) return TDBEM_OK;
-  const int P16 = (P + 63) / 64 * 64;
-  if (P16 > 64 * kResMaxCh) {
+  const int nch = tdbem_m2l_chunks(P, TDBEM_P_F16X3);
+  if (nch > kResMaxCh) {
     c->set_error("fast: resident-operator M2L needs P <= 256");
     return TDBEM_EINVAL;
   }
   const int grid = max_ctas < 0 ? n : std::min(n, max_ctas > 0 ? std::min(max_ctas, nsm) : nsm);
-  k_m2l_res<<<grid, kResThreads, kResSmem, c->stream>>>(gemm, units + u0, n, img, P, P16, pt, PS, pO, pC, psym, smap,
-                                                         pk16, k, loc, Q, R, opinv, pkinv, err);
+  k_m2l_res<<<grid, kResThreads, kResSmem, c->stream>>>(gemm, units + u0, n, img, P, nch, pt, PS, pO, pC, psym, smap,
+                                                         pk, k, loc, Q, R, opinv, pkinv, err);
   TDBEM_CUDA_TRY(c, cudaGetLastError());
   return TDBEM_OK;
 }
 
-tdbem_status tdbem_m2l_pack_f16(tdbem_ctx* c, const int32_t* cS, const int16_t* csym, int ncombo,
-                                const int16_t* smap, const float* mom, int k, int R, int PS, int pt, __half* pk16,
-                                float* pkinv) {
+tdbem_status tdbem_m2l_pack_split(tdbem_ctx* c, const int32_t* cS, const int16_t* csym, int ncombo,
+                                  const int16_t* smap, const float* mom, int k, int R, int PS, int pt, int prec,
+                                  uint8_t* pk, float* pkinv) {
   using namespace tdbem;
   const int64_t nrows = (int64_t)ncombo * 2 * R * kNCmp;
   if (nrows == 0) return TDBEM_OK;
-  const int P16 = (PS * pt + 63) / 64 * 64;
-  k_m2l_pack_f16<<<(unsigned)((nrows * 32 + 255) / 256), 256, 0, c->stream>>>(cS, csym, nrows, smap, mom, k, R, PS,
-                                                                              pt, P16, pk16, pkinv);
+  k_m2l_pack_split<<<(unsigned)((nrows * 32 + 255) / 256), 256, 0, c->stream>>>(
+      cS, csym, nrows, smap, mom, k, R, PS, pt, tdbem_m2l_chunks(PS * pt, prec), split_fmt(prec), pk, pkinv);
+  TDBEM_CUDA_TRY(c, cudaGetLastError());
+  return TDBEM_OK;
+}
+
+// The split forms with both operands streamed (k_m2l_stream, at most 64 K chunks): n tiles of the list for
+// 256 rows, up to max_run of them one after another in a CTA.
+tdbem_status tdbem_m2l_stream(tdbem_ctx* c, const int4* gemm, const int4* tiles, int n, const uint4* img, int P, int pt,
+                              int PS, const int32_t* pO, const int32_t* pC, const int16_t* psym, const int16_t* smap,
+                              const uint8_t* pk, int k, float* loc, int Q, int R, int prec, const float* opinv,
+                              const float* pkinv, const unsigned long long* live, int32_t* err, int max_run) {
+  using namespace tdbem;
+  static bool attr = false;
+  static int nsm = 0;
+  if (!attr) {
+    TDBEM_CUDA_TRY(c, cudaFuncSetAttribute(k_m2l_stream, cudaFuncAttributeMaxDynamicSharedMemorySize, kStrSmem));
+    TDBEM_CUDA_TRY(c, cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
+    attr = true;
+  }
+  if (n <= 0) return TDBEM_OK;
+  const int run = std::max(1, std::min(max_run, n / (2 * nsm)));
+  const int groups = (n + nsm * run - 1) / (nsm * run), rest = n - (groups - 1) * nsm * run;
+  k_m2l_stream<<<(groups - 1) * nsm + std::min(nsm, rest), kResThreads, kStrSmem, c->stream>>>(
+      gemm, tiles, n, run, nsm, img, P, tdbem_m2l_chunks(P, prec), split_fmt(prec), pt, PS, pO, pC, psym, smap, pk, k, loc,
+      Q, R, opinv, pkinv, live, err);
   TDBEM_CUDA_TRY(c, cudaGetLastError());
   return TDBEM_OK;
 }
