@@ -241,7 +241,6 @@ tdbem_status tdbem_create(const double* verts, int64_t nv, const int32_t* tris, 
   }
   if (!s) s = finish_create(c);
   if (!s && p.mode == TDBEM_DIRECT) s = tdbem_direct_split(c);
-  if (!s && p.mode == TDBEM_FAST && tdbem_fast_wants_tiles(c)) s = tdbem_near_tiles_build(c);
   if (s) {
     tdbem_destroy(c);
     return s;
@@ -559,7 +558,7 @@ tdbem_status tdbem_step(tdbem_ctx* c, double* J_out, int32_t* iters) {
   c->total_iters += h[0];
   if (c->p.mode == TDBEM_FAST && (s = tdbem_fast_check(c))) return s;
   if (!h[1]) {
-    if ((s = tdbem_direct_check(c))) return s;
+    if (c->p.mode == TDBEM_DIRECT && (s = tdbem_direct_check(c))) return s;
     c->set_error("step: Z0 solve missed the tolerance");
     return TDBEM_ENOCONV;
   }
@@ -586,7 +585,7 @@ tdbem_status tdbem_step_v(tdbem_ctx* c, const double* V, double* J_out, int32_t*
   c->total_iters += h[0];
   if (c->p.mode == TDBEM_FAST && (s = tdbem_fast_check(c))) return s;
   if (!h[1]) {
-    if ((s = tdbem_direct_check(c))) return s;
+    if (c->p.mode == TDBEM_DIRECT && (s = tdbem_direct_check(c))) return s;
     c->set_error("step: Z0 solve missed the tolerance");
     return TDBEM_ENOCONV;
   }
@@ -607,7 +606,7 @@ tdbem_status tdbem_step_wait(tdbem_ctx* c, int32_t* iters) {
   tdbem_status s;
   if (c->p.mode == TDBEM_FAST && (s = tdbem_fast_check(c))) return s;
   if (!conv) {
-    if ((s = tdbem_direct_check(c))) return s;
+    if (c->p.mode == TDBEM_DIRECT && (s = tdbem_direct_check(c))) return s;
     c->set_error("step: Z0 solve missed the tolerance");
     return TDBEM_ENOCONV;
   }
@@ -687,7 +686,6 @@ static tdbem_status check_misses(tdbem_ctx* c) {
   if (!s) s = tdbem_direct_join(c);
     if (s) return s;
     s = tdbem_fast_check(c);
-    if (!s) s = tdbem_direct_check(c);
     if (s) return s;
   } else {
     tdbem_status s = tdbem_direct_check(c);

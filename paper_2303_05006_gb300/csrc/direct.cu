@@ -664,7 +664,7 @@ __global__ void __launch_bounds__(128) k_direct_reduce(const double* __restrict_
 // 24-bit store adds its own rounding, 2^-16 sum |Zt^(m)_ij| |J_j^{alpha-m}|.
 constexpr int kRtWarps = 8;  // warps per block
 constexpr int kRtB = 4;      // steps per pass of the far pairs where the store is large
-constexpr int64_t kRtBlockBytes = 24ll << 20;  // such a store's bytes
+constexpr int64_t kRtBlockBytes = 64ll << 20;  // such a store's bytes
 
 // A value of the 24-bit store: an FP32 number with its significand rounded
 // to 16 bits (round half away from zero on the dropped byte), kept as its top
@@ -1447,60 +1447,49 @@ tdbem_status tdbem_direct_resplit(tdbem_ctx* c) {
   return c->d_rs ? split_ring(c, c->d_Jring, c->d_rs) : TDBEM_OK;
 }
 
-// The sums of the lags >= 3 of step alpha (for tdbem_fast: of the near field), the
-// context's stream behind them: *pre is [kRedLanes][npos].
-tdbem_status tdbem_rt_pre(tdbem_ctx* c, int32_t alpha, const double* d_ring, const double** pre) {
-  // the march's own ring uses the buffers alpha & 1 (near, pre) and the far
-  // buffers of its blocks, possibly filled ahead during earlier steps; any other
-  // history buffer 2 and the far buffer behind the two
-  const bool march = d_ring == c->d_Jring;
-  const int64_t npos = (int64_t)c->rt_nrt * 32;
-  const float2* rs = march ? c->d_rs : c->d_rs_eval;
-  const int buf = march ? (alpha & 1) : 2;
-  tdbem_status s;
-  if (march && c->dahead[buf] == alpha) {
-    TDBEM_CUDA_TRY(c, cudaStreamWaitEvent(c->stream, c->ev_dahead[buf], 0));
-  } else {
-    if (!march && (s = split_ring(c, d_ring, c->d_rs_eval))) return s;
-    const double* far = far_out(c, 2);
-    int nfar = c->rt_ncb;
-    cudaEvent_t e = c->prof_begin(1);
-    if ((s = direct_near(c, alpha, rs, buf))) return s;
-    if (!march) {
-      for (int q = 0; q < c->rt_B; ++q)
-        if ((s = direct_rt(c, alpha, 1, rs, q, far_out(c, 2)))) return s;
-    } else {
-      const int32_t a0 = far_block(c, alpha);
-      const int fb = far_buf(c, a0);
-      far = far_out(c, fb) + (int64_t)(alpha - a0) * c->rt_ncb * npos;
-      if (!far_any(c, a0)) {
-        nfar = 0;
-      } else {
-        if ((s = far_parts_wait(c, a0))) return s;
-        // the parts not summed ahead, now
-        for (int q = 0; q < c->rt_B; ++q)
-          if (!(c->far_done[fb] >> q & 1) && (s = direct_rt(c, a0, c->rt_B, rs, q, far_out(c, fb)))) return s;
-        c->far_done[fb] = (1 << c->rt_B) - 1;
-      }
-    }
-    if ((s = direct_presum(c, far, nfar, buf))) return s;
-    c->prof_end(1, e);
-  }
-  if (march) c->dahead[buf] = 0;
-  *pre = c->d_pre + buf * kRedLanes * npos;
-  return TDBEM_OK;
-}
-
 tdbem_status tdbem_direct_history(tdbem_ctx* c, int32_t alpha, const double* d_ring, const double* V) {
   const PairStore& st = c->direct;
   if (c->R == 1 && c->rt_prec) {
+    // the march's own ring uses the buffers alpha & 1 (near, pre) and the far
+    // buffers of its blocks, possibly filled ahead during earlier steps; any other
+    // history buffer 2 and the far buffer behind the two
+    const bool march = d_ring == c->d_Jring;
     const int64_t npos = (int64_t)c->rt_nrt * 32;
-    const double* pre = nullptr;
-    tdbem_status s = tdbem_rt_pre(c, alpha, d_ring, &pre);
-    if (s) return s;
+    const float2* rs = march ? c->d_rs : c->d_rs_eval;
+    const int buf = march ? (alpha & 1) : 2;
+    tdbem_status s;
+    if (march && c->dahead[buf] == alpha) {
+      TDBEM_CUDA_TRY(c, cudaStreamWaitEvent(c->stream, c->ev_dahead[buf], 0));
+    } else {
+      if (!march && (s = split_ring(c, d_ring, c->d_rs_eval))) return s;
+      const double* far = far_out(c, 2);
+      int nfar = c->rt_ncb;
+      cudaEvent_t e = c->prof_begin(1);
+      if ((s = direct_near(c, alpha, rs, buf))) return s;
+      if (!march) {
+        for (int q = 0; q < c->rt_B; ++q)
+          if ((s = direct_rt(c, alpha, 1, rs, q, far_out(c, 2)))) return s;
+      } else {
+        const int32_t a0 = far_block(c, alpha);
+        const int fb = far_buf(c, a0);
+        far = far_out(c, fb) + (int64_t)(alpha - a0) * c->rt_ncb * npos;
+        if (!far_any(c, a0)) {
+          nfar = 0;
+        } else {
+          if ((s = far_parts_wait(c, a0))) return s;
+          // the parts not summed ahead, now
+          for (int q = 0; q < c->rt_B; ++q)
+            if (!(c->far_done[fb] >> q & 1) && (s = direct_rt(c, a0, c->rt_B, rs, q, far_out(c, fb)))) return s;
+          c->far_done[fb] = (1 << c->rt_B) - 1;
+        }
+      }
+      if ((s = direct_presum(c, far, nfar, buf))) return s;
+      c->prof_end(1, e);
+    }
+    if (march) c->dahead[buf] = 0;
     cudaEvent_t e = c->prof_begin(10);
     k_direct_reduce<<<(unsigned)((npos * kRedLanes + 127) / 128), 128, 0, c->stream>>>(
-        pre, c->d_rt_row, npos, c->d_l2_ptr, c->d_l2_col, c->d_l2_val, d_ring, c->L, alpha, V, c->d_R);
+        c->d_pre + buf * kRedLanes * npos, c->d_rt_row, npos, c->d_l2_ptr, c->d_l2_col, c->d_l2_val, d_ring, c->L, alpha, V, c->d_R);
     c->prof_end(10, e);
   } else if (c->R == 1) {
     if (!c->d_ring2 || !st.val) {
@@ -1677,7 +1666,8 @@ static std::vector<int32_t> bisected_edges(const tdbem_ctx* c) {
 // Builds the row-tile store of the lags >= 3 from the FP64 store (prec 1: FP32
 // values, 2: (hi, lo) pairs, 3: 24-bit values), frees the FP64 values and sets
 // the grid.
-static tdbem_status build_row_tiles(tdbem_ctx* c, PairStore& st, int prec, int units) {
+static tdbem_status build_row_tiles(tdbem_ctx* c, int prec) {
+  PairStore& st = c->direct;
   const int64_t ne = c->ne, nrt = (ne + 31) / 32, ntc = nrt * ne;
   tdbem_status s;
   // Steps per pass: kRtB where the store is larger than a good part of L2, so
@@ -1692,6 +1682,7 @@ static tdbem_status build_row_tiles(tdbem_ctx* c, PairStore& st, int prec, int u
   TDBEM_CUDA_TRY(c, cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
   TDBEM_CUDA_TRY(c, cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
   TDBEM_CUDA_TRY(c, cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, c->device));
+  const int units = prec != 2;  // FP32 and 24-bit: whole units of 64 columns in edge order
   const int m0 = units ? 3 : rt_m0(B, B - 1), most = prec == 2 ? 2 : 3;  // blocks per SM the registers allow
   int cbw = 64;
   if (!units) {
@@ -1801,6 +1792,8 @@ static tdbem_status build_row_tiles(tdbem_ctx* c, PairStore& st, int prec, int u
   TDBEM_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   c->dfree(d_qst);
   c->dfree(d_qcol);
+  c->dfree(st.val);
+  st.val = nullptr;
   c->rt_B = B;
   c->rt_nrt = (int32_t)nrt;
   c->rt_Lh = Lh;
@@ -1849,81 +1842,6 @@ static tdbem_status build_row_tiles(tdbem_ctx* c, PairStore& st, int prec, int u
   c->rt_cbw = cbw;
   c->rt_ncb = ncb;
   return TDBEM_OK;
-}
-
-// The row tiles' partial sums and split rings, and the side stream.
-static tdbem_status rt_buffers(tdbem_ctx* c) {
-  tdbem_status s;
-  const size_t npos = (size_t)c->rt_nrt * 32, nn = 3 * c->rt_nslot * npos, nf = (2 * c->rt_B + 1) * c->rt_ncb * npos;
-  const size_t nr = (size_t)c->ne * c->L;
-  if ((s = c->dalloc(&c->d_dpart, nn)) || (s = c->dalloc(&c->d_fpart, nf)) || (s = c->dalloc(&c->d_pre, 3 * kRedLanes * npos)) || (s = c->dalloc(&c->d_rs, nr)) ||
-      (s = c->dalloc(&c->d_rs_eval, nr)))
-    return s;
-  // a tile with fewer near chunks than nslot leaves its last slots zero
-  TDBEM_CUDA_TRY(c, cudaMemsetAsync(c->d_dpart, 0, std::max<size_t>(nn, 1) * sizeof(double), c->stream));
-  TDBEM_CUDA_TRY(c, cudaMemsetAsync(c->d_fpart, 0, nf * sizeof(double), c->stream));
-  TDBEM_CUDA_TRY(c, cudaMemsetAsync(c->d_rs, 0, nr * sizeof(float2), c->stream));
-  TDBEM_CUDA_TRY(c, cudaMemsetAsync(c->d_rs_eval, 0, nr * sizeof(float2), c->stream));
-  if (c->p.far_overlap) {
-    // between the library stream's highest priority and the lowest: the
-    // next solve's cluster is dispatched ahead of this stream's blocks
-    int prio_lo = 0, prio_hi = 0;
-    TDBEM_CUDA_TRY(c, cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi));
-    TDBEM_CUDA_TRY(c, cudaStreamCreateWithPriority(&c->dstream, cudaStreamNonBlocking, (prio_lo + prio_hi) / 2));
-    TDBEM_CUDA_TRY(c, cudaEventCreateWithFlags(&c->ev_dsolved, cudaEventDisableTiming));
-    for (int b = 0; b < 2; ++b) {
-      TDBEM_CUDA_TRY(c, cudaEventCreateWithFlags(&c->ev_dahead[b], cudaEventDisableTiming));
-      TDBEM_CUDA_TRY(c, cudaEventCreateWithFlags(&c->ev_far[b], cudaEventDisableTiming));
-    }
-  }
-  return TDBEM_OK;
-}
-
-// Dense lag windows from the near field's CSR (one warp per row; pairs not listed
-// keep no lags).
-__global__ void k_dense_windows(const int64_t* ptr, const int32_t* col, const int16_t* m_lo, const uint8_t* nlag,
-                                const int64_t* off, int64_t ne, int16_t* dm, uint8_t* dn, int64_t* doff) {
-  const int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  if (i >= ne) return;
-  for (int64_t q = ptr[i] + (threadIdx.x & 31); q < ptr[i + 1]; q += 32) {
-    const int64_t p = i * ne + col[q];
-    dm[p] = m_lo[q];
-    dn[p] = nlag[q];
-    doff[p] = off[q];
-  }
-}
-
-// Fast mode, one right-hand side: the row tiles of the near field's lags >= 3, FP32
-// values (see tdbem_fast_wants_tiles).
-tdbem_status tdbem_near_tiles_build(tdbem_ctx* c) {
-  const int64_t *rp, *off;
-  const int32_t* col;
-  const int16_t* ml;
-  const uint8_t* nl;
-  const double* val;
-  tdbem_fast_z0_source(c, &rp, &col, &ml, &nl, &off, &val);
-  const int64_t ne = c->ne, npair = ne * ne, npos = (ne + 31) / 32 * 32;
-  PairStore st;
-  tdbem_status s;
-  std::vector<int32_t> rows = bisected_edges(c), pos(ne);
-  for (int64_t k = 0; k < ne; ++k) pos[rows[k]] = (int32_t)k;
-  rows.resize(npos, -1);
-  if ((s = c->dalloc(&st.m_lo, npair)) || (s = c->dalloc(&st.nlag, npair)) || (s = c->dalloc(&st.off, npair)) ||
-      (s = up(c, &c->d_rt_row, rows)) || (s = up(c, &c->d_rt_pos, pos)))
-    return s;
-  TDBEM_CUDA_TRY(c, cudaMemsetAsync(st.m_lo, 0, npair * sizeof(int16_t), c->stream));
-  TDBEM_CUDA_TRY(c, cudaMemsetAsync(st.nlag, 0, npair, c->stream));
-  k_dense_windows<<<(unsigned)((ne * 32 + 255) / 256), 256, 0, c->stream>>>(rp, col, ml, nl, off, ne, st.m_lo, st.nlag,
-                                                                           st.off);
-  TDBEM_CUDA_TRY(c, cudaGetLastError());
-  st.val = const_cast<double*>(val);  // read only
-  st.nval = tdbem_fast_nval(c);
-  s = build_row_tiles(c, st, 1, 0);
-  TDBEM_CUDA_TRY(c, cudaStreamSynchronize(c->stream));  // before the windows (and rows, pos on the host) go
-  c->dfree(st.m_lo);
-  c->dfree(st.nlag);
-  c->dfree(st.off);
-  return s ? s : rt_buffers(c);
 }
 
 // Single right-hand side, after Z0 and the lag-2 entries have been read from
@@ -1976,15 +1894,34 @@ tdbem_status tdbem_direct_split(tdbem_ctx* c) {
   }
   if (tiled) {
     tdbem_status s =
-        // FP32 and 24-bit: whole units of 64 columns in edge order
-        build_row_tiles(c, st, c->p.p2p_prec == TDBEM_P_FP32 ? 1 : c->p.p2p_prec == TDBEM_P_FP24 ? 3 : 2,
-                        c->p.p2p_prec != TDBEM_P_FP64);
+        build_row_tiles(c, c->p.p2p_prec == TDBEM_P_FP32 ? 1 : c->p.p2p_prec == TDBEM_P_FP24 ? 3 : 2);
     if (s) return s;
   }
   if (c->rt_prec) {
-    c->dfree(st.val);
-    st.val = nullptr;
-    return rt_buffers(c);
+    tdbem_status s;
+    const size_t npos = (size_t)c->rt_nrt * 32, nn = 3 * c->rt_nslot * npos, nf = (2 * c->rt_B + 1) * c->rt_ncb * npos;
+    const size_t nr = (size_t)c->ne * c->L;
+    if ((s = c->dalloc(&c->d_dpart, nn)) || (s = c->dalloc(&c->d_fpart, nf)) || (s = c->dalloc(&c->d_pre, 3 * kRedLanes * npos)) || (s = c->dalloc(&c->d_rs, nr)) ||
+        (s = c->dalloc(&c->d_rs_eval, nr)))
+      return s;
+    // a tile with fewer near chunks than nslot leaves its last slots zero
+    TDBEM_CUDA_TRY(c, cudaMemsetAsync(c->d_dpart, 0, std::max<size_t>(nn, 1) * sizeof(double), c->stream));
+    TDBEM_CUDA_TRY(c, cudaMemsetAsync(c->d_fpart, 0, nf * sizeof(double), c->stream));
+    TDBEM_CUDA_TRY(c, cudaMemsetAsync(c->d_rs, 0, nr * sizeof(float2), c->stream));
+    TDBEM_CUDA_TRY(c, cudaMemsetAsync(c->d_rs_eval, 0, nr * sizeof(float2), c->stream));
+    if (c->p.far_overlap) {
+      // between the library stream's highest priority and the lowest: the
+      // next solve's cluster is dispatched ahead of this stream's blocks
+      int prio_lo = 0, prio_hi = 0;
+      TDBEM_CUDA_TRY(c, cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi));
+      TDBEM_CUDA_TRY(c, cudaStreamCreateWithPriority(&c->dstream, cudaStreamNonBlocking, (prio_lo + prio_hi) / 2));
+      TDBEM_CUDA_TRY(c, cudaEventCreateWithFlags(&c->ev_dsolved, cudaEventDisableTiming));
+      for (int b = 0; b < 2; ++b) {
+        TDBEM_CUDA_TRY(c, cudaEventCreateWithFlags(&c->ev_dahead[b], cudaEventDisableTiming));
+        TDBEM_CUDA_TRY(c, cudaEventCreateWithFlags(&c->ev_far[b], cudaEventDisableTiming));
+      }
+    }
+    return TDBEM_OK;
   }
   k_split_values<<<(unsigned)((st.nval + 255) / 256), 256, 0, c->stream>>>(st.val, st.nval);
   TDBEM_CUDA_TRY(c, cudaGetLastError());

@@ -815,13 +815,11 @@ __global__ void k_l2p(const int32_t* leaf_cells, const int32_t* tri_b, const int
 // column << 8 | lag) entries with coalesced loads; every lane does the same
 // work, and the lags of one column are neighbours in the history ring.
 // R_i = V_i + V2_i + Rfar_i - sum over the row's entries of z J_col^{alpha-m}
-// (V, V2 and Rfar may be null); pre: also the eight sums pre[w * npos + pos[i]]
-// (lanes 0 .. 7 take one each) of the row tiles.
+// (V, V2 and Rfar may be null).
 __global__ void __launch_bounds__(256) k_near_history_flat(const int64_t* hrow, const float* hval, const int32_t* hmeta,
                                                           int64_t ne, const double* ring, int L, int alpha,
                                                           const double* V, const double* V2, double* Rfar_slot,
-                                                          double* R, const double* pre = nullptr,
-                                                          const int32_t* pos = nullptr, int64_t npos = 0) {
+                                                          double* R) {
   int64_t i = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
   int lane = threadIdx.x & 31;
   if (i >= ne) return;
@@ -841,7 +839,6 @@ __global__ void __launch_bounds__(256) k_near_history_flat(const int64_t* hrow, 
     if (b0 >= 0) s0 += __ldg(hval + e) * (float)ring[(int64_t)(q0 >> 8) * L + (b0 & (L - 1))];
   }
   double d = (double)s0 + (double)s1;
-  if (pre && lane < 8) d += pre[(int64_t)lane * npos + pos[i]];
   for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xffffffffu, d, o);
   if (lane == 0) {
     double far = Rfar_slot ? Rfar_slot[i] : 0.0;
@@ -1249,13 +1246,14 @@ tdbem_status tdbem_build_fast(tdbem_ctx* c) {
       std::vector<int64_t> hrow(ne + 1, 0);
       std::vector<float> hval;
       std::vector<int32_t> hmeta;
-      const bool tiles = tdbem_fast_wants_tiles(c);  // the lags >= 3 go to row tiles (direct.cu)
+      hval.reserve(F->nval);
+      hmeta.reserve(F->nval);
       for (int64_t i = 0; i < ne; ++i) {
         hrow[i] = (int64_t)hval.size();
         for (int64_t q = rp[i]; q < rp[i + 1]; ++q)
           for (int w = 0; w < nl[q]; ++w) {
             const int m = ml[q] + w;
-            if (m < 2 || (tiles && m > 2)) continue;
+            if (m < 2) continue;
             hval.push_back(v32[off[q] + w]);
             hmeta.push_back((col[q] << 8) | m);
           }
@@ -1424,7 +1422,7 @@ tdbem_status tdbem_build_fast(tdbem_ctx* c) {
           if (nseg)
             TDBEM_CUDA_TRY(c, cudaMemcpy(F->d_rseg, rseg.data(), nseg * sizeof(int32_t), cudaMemcpyHostToDevice));
         }
-        if (c->p.far_overlap && !tiles) {
+        if (c->p.far_overlap) {
           // between the deferred M2L's lowest priority and the steps' highest:
           // the next solve's cluster, which needs whole SMs, is dispatched ahead
           // of this stream's remaining CTAs
@@ -2020,19 +2018,6 @@ tdbem_status tdbem_fast_history(tdbem_ctx* c, int32_t alpha, const double* ring,
   double* slot = nullptr;
   if (F->lmax >= 2)
     slot = (eval ? F->d_Rfar_eval : F->d_Rfar) + (int64_t)((alpha - 1) & (F->Lr - 1)) * c->ne * c->R;
-  if (c->rt_prec) {
-    // lags >= 3 from the row tiles, summed ahead in the pipelined march; lag 2, V and the far field here
-    const double* pre = nullptr;
-    tdbem_status s = tdbem_rt_pre(c, alpha, ring, &pre);
-    if (s) return s;
-    cudaEvent_t e = c->prof_begin(1);
-    k_near_history_flat<<<(unsigned)((c->ne + 7) / 8), 256, 0, c->stream>>>(
-        F->d_hrow2, F->d_hval2, F->d_hmeta2, c->ne, ring, c->L, alpha, V, nullptr, slot, c->d_R, pre, c->d_rt_pos,
-        (int64_t)c->rt_nrt * 32);
-    c->prof_end(1, e);
-    TDBEM_CUDA_TRY(c, cudaGetLastError());
-    return TDBEM_OK;
-  }
   if (!eval && F->nstream) {
     // pipelined march: -(lags >= 3) was summed ahead on the near stream
     // (it depends on the history only); otherwise it is summed now
@@ -2107,10 +2092,7 @@ static tdbem_status near_lags3(tdbem_ctx* c, const double* ring, int32_t alpha, 
 
 tdbem_status tdbem_fast_after_solve(tdbem_ctx* c, int32_t alpha) {
   FmmPlan* F = c->fmm;
-  if (c->rt_prec) {
-    tdbem_status s = tdbem_direct_after_solve(c, alpha);
-    if (s) return s;
-  } else if (F->nstream && alpha + 2 <= c->Nt - 1) {
+  if (F->nstream && alpha + 2 <= c->Nt - 1) {
     // -(lags >= 3) of step alpha + 2 needs the currents up to J^{alpha-1},
     // which this solve completes; its buffer was last read by the lag-2 pass
     // of step alpha, before the solve.  It runs on the near stream while the
@@ -2217,18 +2199,6 @@ void tdbem_fast_state(tdbem_ctx* c, std::vector<std::pair<void*, size_t>>* bufs)
   }
   bufs->push_back({F->d_Rfar, (size_t)F->Lr * c->ne * c->R * sizeof(double)});
 }
-
-// Whether the single-right-hand-side near field's lags >= 3 are summed by the row
-// tiles (direct.cu: once per four steps for the pairs whose lags allow it) in place
-// of the flat or column-tiled entries.  They are faster wherever their setup, which
-// lays the pairs' windows out densely (11 bytes a pair of functions), stays small: up
-// to 16384 functions; first lags and history must fit their bytes.  A context with a
-// memory budget keeps the forms that budgets were made for.
-bool tdbem_fast_wants_tiles(const tdbem_ctx* c) {
-  return c->p.mode == TDBEM_FAST && c->R == 1 && c->ne <= 16384 && c->fmm && c->fmm->max_near_lag <= 180 &&
-         c->p.max_device_bytes == 0;
-}
-int64_t tdbem_fast_nval(const tdbem_ctx* c) { return c->fmm->nval; }
 
 void tdbem_fast_free(tdbem_ctx* c) {
   FmmPlan* F = c->fmm;

@@ -118,8 +118,7 @@ struct tdbem_ctx {
   double* d_Jring = nullptr;        // [ne][L][R]
   float* d_rf = nullptr;            // fast mode, R > 1: the ring in FP32 [ne][L][R], kept up to date by the solve
   float2* d_ring2 = nullptr;        // direct mode, R = 1: split history [L][ne] (hi, lo) (untiled kernel)
-  // R = 1, row-tile store of the lags >= 3 (direct mode: of all pairs; fast mode: of
-  // the near field; rows in tiles of 32,
+  // direct mode, R = 1, row-tile store of the lags >= 3 (rows in tiles of 32,
   // one lane per row; see k_direct_history_rt): the far pairs by column blocks,
   // rt_B steps per pass, and the near pairs as a list, plus the lag-2 entries in
   // the reduction
@@ -127,7 +126,6 @@ struct tdbem_ctx {
   int32_t rt_B = 1;                 // steps per pass of the far pairs
   int32_t rt_nrt = 0;               // row tiles
   int32_t* d_rt_row = nullptr;      // [nrt * 32] row at a position (-1: padding)
-  int32_t* d_rt_pos = nullptr;      // [ne] position of a row (fast mode)
   unsigned char* d_rt_val = nullptr;  // [groups] of 32 values (128, 256 or 96 bytes)
   uint32_t* d_rt_goff = nullptr;    // [nrt * ne + 1] first group of (tile, column)
   uint8_t* d_rt_lo = nullptr;       // [nrt * ne][32] first stored lag of (row, column)
@@ -244,8 +242,6 @@ tdbem_status tdbem_build_direct(tdbem_ctx* c);
 tdbem_status tdbem_direct_history(tdbem_ctx* c, int32_t alpha, const double* d_ring, const double* V);
 tdbem_status tdbem_direct_split(tdbem_ctx* c);
 tdbem_status tdbem_direct_after_solve(tdbem_ctx* c, int32_t alpha);
-tdbem_status tdbem_rt_pre(tdbem_ctx* c, int32_t alpha, const double* d_ring, const double** pre);
-tdbem_status tdbem_near_tiles_build(tdbem_ctx* c);
 tdbem_status tdbem_direct_resplit(tdbem_ctx* c);  // the split history anew from the ring
 tdbem_status tdbem_direct_join(tdbem_ctx* c);
 tdbem_status tdbem_direct_check(tdbem_ctx* c);
@@ -265,8 +261,6 @@ tdbem_status tdbem_fast_consume_eval_slot(tdbem_ctx* c, int32_t alpha);
 tdbem_status tdbem_fast_eval_reset(tdbem_ctx* c);
 tdbem_status tdbem_fast_reset(tdbem_ctx* c);
 void tdbem_fast_free(tdbem_ctx* c);
-bool tdbem_fast_wants_tiles(const tdbem_ctx* c);
-int64_t tdbem_fast_nval(const tdbem_ctx* c);
 tdbem_status tdbem_fast_join(tdbem_ctx* c);
 tdbem_status tdbem_fast_invalidate(tdbem_ctx* c);
 tdbem_status tdbem_fast_check(tdbem_ctx* c);
