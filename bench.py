@@ -241,9 +241,10 @@ def roofline(args, info, launches, ms, K, W):
                 if args.prec.endswith("x3") else ""}
     if name in ("near_history",):
         if args.mode in ("direct", "direct32", "direct24") and info.history_bytes > 0:
-            # the row-tile store streamed once per launch: the groups of 32 coefficients (8 B pairs
-            # or 4 B FP32, zero-padded to the tile's longest window per column), one first-lag byte
-            # per (row, column) and one 4-byte group offset per (row tile, column)
+            # the store streamed per step: the groups of 32 coefficients (8 B pairs or 4 B FP32,
+            # zero-padded to the tile's longest window per column), one first-lag byte per (row,
+            # column) and one 4-byte group offset per (row tile, column); a fourth of the far
+            # pairs', whose pass serves four steps
             nbytes = info.history_bytes
         elif args.mode in ("direct", "direct32", "direct24"):  # batched kernel: FP64 coefficients and lag windows
             nbytes = info.near_coef_bytes + info.n_near_pairs * (2 + 1)
@@ -257,9 +258,9 @@ def roofline(args, info, launches, ms, K, W):
                 "peak_source": f"{src} hbm_gbs", "bytes_per_launch": nbytes}
     if name == "z0_solve" and info.z0_nnz > 0:
         # algorithmic operand bytes of one solve: per BiCGStab iteration two FP32
-        # ELL SpMVs (value + column, 8 B per non-zero) and 4-byte vector passes
-        # (21 + 2 x 12 with the 5-entry triangle-block preconditioner, 21 + 2 x 2
-        # with the diagonal one); two FP64 residuals (12 B per non-zero, 3 vectors)
+        # SpMVs (value + column, 8 B per non-zero) and 4-byte vector passes (21 + 2 x 12
+        # with a preconditioner of a few entries a row, 21 + 2 x 2 with the diagonal one);
+        # two FP64 residuals (12 B per non-zero, 3 vectors)
         R = args.rhs
         its = info.total_solver_iters / max(W + K, 1)
         vec = 21 + 2 * (12 if args.precond else 2)
@@ -267,8 +268,8 @@ def roofline(args, info, launches, ms, K, W):
         gbs = nbytes / (ms[dom] / launches[dom] / 1e3) / 1e9
         return {"kernel": name, "bound": "hbm", "achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm,
                 "traffic": None, "peak_source": f"{src} hbm_gbs", "bytes_per_launch": nbytes,
-                "note": "latency-bound: one 16-CTA cluster runs about 8 dependent BiCGStab iterations per solve, "
-                        "each with 6 cluster-wide barriers; Z0 (FP32 ELL) and the vectors stay in L2"}
+                "note": "latency-bound: one 16-CTA cluster runs a few dependent BiCGStab iterations per solve, "
+                        "each with cluster-wide barriers; Z0 stays in L2, the vectors on the chip"}
     return {"kernel": name, "bound": "latency", "achieved": None, "peak": None, "unit": None, "frac": None,
             "traffic": None}
 
@@ -632,7 +633,7 @@ def run_ours(args, rank, world, dist):
                    "untimed_before": f"{H['pre']} steps (warm-up, and the history window filled: max lag "
                                      f"{info.max_lag})",
                    "l2": f"inputs larger than L2 ({(info.history_bytes or info.near_coef_bytes) / 1e9:.2f} GB of "
-                         "stored coefficients read every step)",
+                         "stored coefficients read per step)",
                    "setup_s": H["setup_s"]},
         "ns_nt_per_s": H["steps_per_s"] * w.n_tri,
         "roofline": roofline(rf_args, info, launches, ms, K, H["pre"]),

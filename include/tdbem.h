@@ -104,10 +104,14 @@ typedef struct {
                             (0: Krylov only); a sweep that does not cut the residual by 0.7 ends them */
   int32_t m2l_tile_rows; /* tensor-core M2L: rows of the product per CTA, 128 or 256; 0 (default) times
                             both at setup on each level and keeps the faster, with the resident-operator
-                            kernel as a third candidate for the FP16 form (see tdbem_info.m2l_resident);
+                            kernel for the FP16 form (see tdbem_info.m2l_resident) and, for the split forms
+                            without a max_device_bytes, the streamed one as further candidates;
                             1 forces the resident-operator kernel where it applies (128 elsewhere) */
-  int32_t precond;       /* Z0 solve preconditioner: 0 Jacobi; 1 (default) triangle blocks (the inverses of the 3 x 3
-                            blocks of Z0 among the RWG functions of each triangle, summed) */
+  int32_t precond;       /* Z0 solve preconditioner: 0 Jacobi; 1 (default) local inverses: each function's row of the
+                            inverse of Z0 among the functions it couples to most strongly.  The solves on the
+                            cooperative grid, of the FP32 and 24-bit direct marches and after jacobi_sweeps
+                            take triangle blocks in its place (the inverses of the 3 x 3 blocks of Z0 among
+                            the RWG functions of each triangle, summed) */
   int32_t far_overlap;   /* 1 (default): the steps overlap.  Fast mode: the M2L products of a gating event with
                             lag q >= 2, whose local coefficients are first read one interval later, run on a
                             lowest-priority second stream of the context while the next steps proceed; with
@@ -150,10 +154,9 @@ typedef struct {
                             (section 4.3.2): 0 (default) the paper's split, one on the interpolated kernel
                             (dU/dt) and one on the target's time factor; 1 both on the target factor (U
                             interpolated); 2 both on the kernel (d^2U/dt^2, a step in time, interpolated) */
-  int32_t solve_cluster;  /* CTAs of the single-RHS cluster solve: 1, 2, 4, 8 or 16 caps it; 0 (default) the
-                             largest cluster the device schedules (16 on GB300), except in the pipelined direct
-                             march with a history sum streaming at least 3 GB per step, where it is 4: the
-                             solve overlaps that sum there, and a smaller cluster leaves SMs to it */
+  int32_t solve_cluster;  /* CTAs of a right-hand side's solve cluster: 1, 2, 4, 8 or 16 caps it; 0 (default)
+                             chooses by the size of Z0 and the number of right-hand sides (at most the largest
+                             cluster the device schedules, 16 on GB300) */
   int64_t max_device_bytes; /* device memory budget of the context's own allocations (0: none).  An allocation
                                that would exceed it fails as if the device were full: tdbem_create returns
                                TDBEM_ENOMEM with nothing left allocated.  Per-call temporaries of
@@ -360,9 +363,9 @@ typedef struct {
   int64_t device_bytes;            /* device memory held by the context */
   double setup_seconds;            /* wall time of tdbem_create */
   int64_t total_solver_iters;
-  int32_t solver_cluster;          /* CTAs of the single-RHS Z0 solve: one thread-block cluster, or for meshes of
-                                      49152 RWG functions or more a cooperative grid of every SM (0 before the
-                                      first solve) */
+  int32_t solver_cluster;          /* CTAs of a right-hand side's Z0 solve: one thread-block cluster, or with one
+                                      right-hand side and 49152 RWG functions or more a cooperative grid of every
+                                      SM (0 before the first solve) */
   int64_t n_far_pairs;             /* interaction-list cluster pairs over all levels (fast mode) */
   double m2l_flops_per_step;       /* M2L flops per step, averaged over the gating cycle (fast mode) */
   int64_t total_jacobi_sweeps;     /* FP64 Jacobi sweeps of the Z0 solves (per-cluster maximum when batched) */
@@ -377,8 +380,9 @@ typedef struct {
                                       column tiles), chosen at setup against the tiled shapes by timing */
   int64_t device_bytes_peak;       /* the most device memory the context held at once, setup included (a
                                       max_device_bytes at least this large lets tdbem_create succeed) */
-  int64_t history_bytes;           /* direct mode: bytes the history sum of the lags >= 3 streams per step (its
-                                      coefficient store and lag windows); 0 where it runs untiled */
+  int64_t history_bytes;           /* direct mode: bytes the history sum of the lags >= 3 streams per step (coefficient
+                                      store and lag windows; a fourth of the far pairs', which are streamed once
+                                      per four steps); 0 where it runs untiled */
 } tdbem_info;
 tdbem_status tdbem_get_info(const tdbem_ctx* ctx, tdbem_info* info);
 
@@ -393,8 +397,8 @@ tdbem_status tdbem_get_info(const tdbem_ctx* ctx, tdbem_info* info);
    FP32 hi/lo pairs before it), 10 history reduction (direct mode, one
    right-hand side, the tiled history sum: the per-column-block partial sums of
    a row added in a fixed order with the lag-2 entries and V; class 1 is then
-   the row-tile sum of the lags >= 3, launched ahead on the side stream when
-   the steps overlap).  n_classes receives the number of classes (<= 16). */
+   the sum of the lags >= 3, one mark per step: the near pairs' lags and, every
+   fourth step, the far pairs' lags of four steps).  n_classes receives the number of classes (<= 16). */
 tdbem_status tdbem_profile_enable(tdbem_ctx* ctx, int32_t on);
 tdbem_status tdbem_profile_read(tdbem_ctx* ctx, int64_t* launches, double* ms, int32_t* n_classes);
 

@@ -908,15 +908,15 @@ __global__ void k_near_seg_reduce(const int64_t* rseg_ptr, const int32_t* rseg, 
   if (i < ne && sub == 0) R[i] = -t;
 }
 
-// Batched near field on the flattened entries: one block per row, its 8 warps
-// taking interleaved runs of 32 entries.  A lane loads one entry of the run
-// (coalesced); then RL lanes (R rounded up to a power of two, at most 32) share an
-// entry at a time, 32 / RL entries side by side, its coefficient and place passed by
-// shuffles and its history R-vector read contiguously.  What bounds it is the
-// history's L2 traffic and latency: the run's reads are independent of each other,
-// so up to 32 are in flight per warp, and the march reads its ring in FP32 (rf, the
-// values the FP64 ring would be rounded to here; kept by the solve).  A chain of
-// FP32 additions is 1 / (8 * 32 / RL) of the row; the chains meet in FP64.
+// Batched near field on the flattened entries: one block per row.  RL lanes (R
+// rounded up to a power of two, at most 32) share an entry; the block's 256 / RL
+// groups take the row's entries in turn, each adding its own in FP32 in the row's
+// order, and the groups' sums meet in FP64.  256 entries at a time: a lane loads one
+// of the entries of its warp's groups, whose coefficient and place are then passed
+// by shuffles, and the history R-vectors are read contiguously.  What bounds it is the
+// history's L2 traffic and latency: the RL reads of a pass are independent of each
+// other, and the march reads its ring in FP32 (rf, the values the FP64 ring would be
+// rounded to here; kept by the solve).
 template <int RL, typename T>
 __global__ void __launch_bounds__(256) k_near_history_flat_multi(const int64_t* __restrict__ hrow,
                                                                 const float* __restrict__ hval,
@@ -930,8 +930,10 @@ __global__ void __launch_bounds__(256) k_near_history_flat_multi(const int64_t* 
   for (int r0 = 0; r0 < R; r0 += RL) {
     const int r = min(r0 + rr, R - 1);  // lanes past R repeat the last column and are not stored
     float s = 0.f;
-    for (int64_t eb = e0 + warp * 32; eb < e1; eb += 256) {
-      const int64_t e = eb + lane;
+    // lane = m (32 / RL) + g: entry m of the pass of the warp's group g
+    const int first = (lane / (32 / RL)) * (256 / RL) + warp * (32 / RL) + lane % (32 / RL);
+    for (int64_t eb = e0; eb < e1; eb += 256) {
+      const int64_t e = eb + first;
       float z = 0.f;
       int o = 0;  // place in the ring, in units of R
       if (e < e1) {
