@@ -2031,8 +2031,6 @@ tdbem_status tdbem_fast_history(tdbem_ctx* c, int32_t alpha, const double* ring,
     F->ahead[b] = 0;
     cudaEvent_t e = c->prof_begin(1);
     if (!have) {
-      // the first step and the second: the sum ahead of the third may still be using the segments' sums
-      if (F->ahead[b ^ 1]) TDBEM_CUDA_TRY(c, cudaStreamWaitEvent(c->stream, F->ev_near[b ^ 1], 0));
       tdbem_status s = near_lags3(c, ring, alpha, Rp, c->stream);
       if (s) return s;
     }
