@@ -104,8 +104,8 @@ typedef struct {
                             (0: Krylov only); a sweep that does not cut the residual by 0.7 ends them */
   int32_t m2l_tile_rows; /* tensor-core M2L: rows of the product per CTA, 128 or 256; 0 (default) times
                             both at setup on each level and keeps the faster, with the resident-operator
-                            kernel for the FP16 form (see tdbem_info.m2l_resident) and, for the split forms
-                            without a max_device_bytes, the streamed one as further candidates;
+                            kernel for the FP16 form (see tdbem_info.m2l_resident) and, for the split forms,
+                            the streamed one as further candidates;
                             1 forces the resident-operator kernel where it applies (128 elsewhere) */
   int32_t precond;       /* Z0 solve preconditioner: 0 Jacobi; 1 (default) local inverses: each function's row of the
                             inverse of Z0 among the functions it couples to most strongly.  The solves on the
@@ -158,8 +158,9 @@ typedef struct {
                              chooses by the size of Z0 and the number of right-hand sides (at most the largest
                              cluster the device schedules, 16 on GB300) */
   int64_t max_device_bytes; /* device memory budget of the context's own allocations (0: none).  An allocation
-                               that would exceed it fails as if the device were full: tdbem_create returns
-                               TDBEM_ENOMEM with nothing left allocated.  Per-call temporaries of
+                               that would exceed it fails as if the device were full: tdbem_create tries again
+                               without what only saves time (the cluster solve's plan, second copies), then
+                               returns TDBEM_ENOMEM with nothing left allocated.  Per-call temporaries of
                                tdbem_history_eval and the learned warm start's buffers (tdbem_mlp_*) are
                                outside it. */
   int32_t p2p_prec;      /* direct mode, precision of the stored coefficients Zt^(m) of the lags m >= 3 in the

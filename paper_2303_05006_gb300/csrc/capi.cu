@@ -173,7 +173,7 @@ static tdbem_status finish_create(tdbem_ctx* c) {
   if ((s = c->dalloc(&c->d_Jring, NR * L)) || (s = c->dalloc(&c->d_R, NR)) || (s = c->dalloc(&c->d_J, NR)) ||
       (s = c->dalloc(&c->d_pulse, 10 * (int64_t)c->R)) || (c->R > 1 && (s = c->dalloc(&c->d_stage, NR))))
     return s;
-  if (c->p.mode == TDBEM_FAST && c->R > 1) {
+  if (c->p.mode == TDBEM_FAST && c->R > 1 && !c->lean) {
     if ((s = c->dalloc(&c->d_rf, NR * L))) return s;
     TDBEM_CUDA_TRY(c, cudaMemsetAsync(c->d_rf, 0, NR * L * sizeof(float), c->stream));
   }
@@ -183,6 +183,9 @@ static tdbem_status finish_create(tdbem_ctx* c) {
   TDBEM_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   return TDBEM_OK;
 }
+
+static tdbem_status create(const double* verts, int64_t nv, const int32_t* tris, int64_t ntri, double dt, int32_t Nt,
+                           const tdbem_params& p, bool lean, tdbem_ctx** out);
 
 tdbem_status tdbem_create(const double* verts, int64_t nv, const int32_t* tris, int64_t ntri, double dt, int32_t Nt,
                           const tdbem_params* params, tdbem_ctx** out) {
@@ -208,10 +211,19 @@ tdbem_status tdbem_create(const double* verts, int64_t nv, const int32_t* tris, 
       (p.mode == TDBEM_DIRECT && p.p2p_prec != TDBEM_P_FP64 && p.n_rhs != 1) ||
       (p.mode != TDBEM_DIRECT && p.mode != TDBEM_FAST))
     return TDBEM_EINVAL;
+  // where the plans that only save time do not fit (a full device, a tight max_device_bytes): again without them
+  tdbem_status s = create(verts, nv, tris, ntri, dt, Nt, p, false, out);
+  if (s == TDBEM_ENOMEM) s = create(verts, nv, tris, ntri, dt, Nt, p, true, out);
+  return s;
+}
+
+static tdbem_status create(const double* verts, int64_t nv, const int32_t* tris, int64_t ntri, double dt, int32_t Nt,
+                           const tdbem_params& p, bool lean, tdbem_ctx** out) {
   auto t0 = std::chrono::steady_clock::now();
   tdbem_ctx* c = new (std::nothrow) tdbem_ctx();
   if (!c) return TDBEM_ENOMEM;
   c->p = p;
+  c->lean = lean;
   c->dt = dt;
   c->Nt = Nt;
   c->R = p.n_rhs;

@@ -1672,7 +1672,7 @@ static tdbem_status build_row_tiles(tdbem_ctx* c, int prec) {
   tdbem_status s;
   // Steps per pass: kRtB where the store is larger than a good part of L2, so
   // that each pass comes from HBM; below that one step per pass, a step ahead.
-  const int B = st.nval * rt_group_bytes(prec) / 32 >= kRtBlockBytes && ne < (1 << 24) ? kRtB : 1;
+  const int B = st.nval * rt_group_bytes(prec) / 32 >= kRtBlockBytes && ne < (1 << 24) && !c->lean ? kRtB : 1;
   // Columns per block: the width whose blocks fill the SMs best beside the 16 SMs
   // of an overlapped solve (the same width for either order of the steps).  The
   // blocks are small, a row tile per warp, so that tiles passed over early in a

@@ -1647,11 +1647,11 @@ tdbem_status tdbem_build_fast(tdbem_ctx* c) {
       if (L.nunits)
         TDBEM_CUDA_TRY(c, cudaMemcpy(L.d_units, units.data(), L.nunits * sizeof(int4), cudaMemcpyHostToDevice));
     }
-    // The split forms with both operands streamed (k_m2l_stream).  It keeps a second pack of the moments, so a
-    // context with a memory budget stays with the kernels above; its masks hold 64 K chunks.
+    // The split forms with both operands streamed (k_m2l_stream): a second pack of the moments, and masks of 64 K
+    // chunks.
     L.str_ok = (c->p.m2l_prec == TDBEM_P_BF16X3 || c->p.m2l_prec == TDBEM_P_TF32X3 ||
                 c->p.m2l_prec == TDBEM_P_F16X3) &&
-               tdbem_m2l_chunks(P, c->p.m2l_prec) <= 64 && c->p.max_device_bytes == 0;
+               tdbem_m2l_chunks(P, c->p.m2l_prec) <= 64 && !c->lean;
     if (qmax >= 255) {
       c->set_error("fast: too many time intervals per interaction");
       return TDBEM_EINVAL;

@@ -116,6 +116,7 @@ struct tdbem_ctx {
   int32_t R = 1;                    // right-hand sides (params.n_rhs)
   int32_t L = 0;                    // ring length (power of two)
   double* d_Jring = nullptr;        // [ne][L][R]
+  bool lean = false;                // without the plans that only save time (the context would not fit otherwise)
   float* d_rf = nullptr;            // fast mode, R > 1: the ring in FP32 [ne][L][R], kept up to date by the solve
   float2* d_ring2 = nullptr;        // direct mode, R = 1: split history [L][ne] (hi, lo) (untiled kernel)
   // direct mode, R = 1, row-tile store of the lags >= 3 (rows in tiles of 32,

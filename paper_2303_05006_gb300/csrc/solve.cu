@@ -1045,13 +1045,13 @@ static tdbem_status tdbem_z0_f32(tdbem_ctx* c) {
   // 1e-13): they keep k_bicgstab's arithmetic (k_bicgstab_x) and with it
   // their currents.
   const bool f32 = c->p.mode == TDBEM_DIRECT && c->p.p2p_prec != TDBEM_P_FP64;
-  if (c->p.jacobi_sweeps == 0 && !f32 && !(c->R == 1 && use_grid(c))) {
+  if (c->p.jacobi_sweeps == 0 && !f32 && !c->lean && !(c->R == 1 && use_grid(c))) {
     if ((s = tdbem_sc_build(c, c->p.solve_cluster > 0 && c->R == 1 ? c->p.solve_cluster : 16, hp, hc, hv)) || c->sc) return s;
   }
   if (c->p.precond != 1) return TDBEM_OK;
   if ((s = build_triangle_precond(c, hp, hc, hv))) return s;
   // (the same cluster size as k_bicgstab would take: the sums' tree depends on it)
-  if (f32 && c->R == 1 && c->p.jacobi_sweeps == 0 && !use_grid(c) && !(s = pick_cluster(c)))
+  if (f32 && c->R == 1 && c->p.jacobi_sweeps == 0 && !c->lean && !use_grid(c) && !(s = pick_cluster(c)))
     s = tdbem_bx_build(c, c->p.solve_cluster > 0 ? std::min(c->p.solve_cluster, g_cluster) : g_cluster, hp, hc, hv);
   return s;
 }

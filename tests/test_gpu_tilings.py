@@ -183,3 +183,19 @@ def test_m2l_kernels_agree(prec, p, R):
         got = evaluate(m2l_prec=prec, m2l_tile_rows=rows)
         tol = (2e-2 if prec == 3 else 1e-3) * scale  # BF16 hi and lo keep 16 bits of the operands, the others 21 or more
         assert np.abs(got - want).max() <= tol, rows
+
+
+@pytest.mark.parametrize("R", [1, 3])
+def test_a_budget_that_leaves_out_the_optional_plans(R):
+    """A budget one byte below what a context takes with the plans that only save time: the march without them (the
+    near fields' sums are the same, so only the solves' tolerance of 1e-13 a step is between the two)."""
+    from workloads.meshes import mean_edge_length
+
+    v, t = _mesh("ell7")
+    dt = 0.3 * mean_edge_length(v, t)
+    kw = dict(n_rhs=R, mode=1, n_leaf=16, far_kernel=2, far_overlap=0)
+    s, _ = _solver(v, t, dt, 16, **kw)
+    b, _ = _solver(v, t, dt, 16, max_device_bytes=s.info().device_bytes_peak - 1, **kw)
+    assert b.info().device_bytes_peak < s.info().device_bytes_peak
+    J, Jb = s.march(12), b.march(12)
+    assert np.abs(J - Jb).max() <= 1e-10 * np.abs(J).max()
