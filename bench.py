@@ -191,18 +191,10 @@ def batch_pulses(w, n: int, seed: int = 4):
     return [pulse_star(w.verts, k=k, pol=pol) for k, pol in random_plane_waves(n, seed)] if n > 0 else []
 
 
-# dram__bytes_read.sum + dram__bytes_write.sum per k_m2l_tc launch (TF32x3, p = 4, 7680 RWG, two
+# dram__bytes_read.sum + dram__bytes_write.sum per k_m2l_tc launch, zero blocks included (TF32x3, p = 4, 7680 RWG, two
 # 128-row tiles per CTA, lag >= 2 products deferred): two leaf events of 289.5 MB and one level-2
 # event of 152.9 MB per gating period of six launches
 M2L_TRAFFIC_TF32X3 = (2 * 289.5e6 + 152.9e6) / 6
-# DRAM bytes over algorithmic bytes of the direct paths' row-tile history sum,
-# per store precision: FP32 from the ncu launch list of the 7680-RWG march
-# itself (2363.4 MB per launch against 2328.3 MB), the (hi, lo) store from a
-# capture on the 1920-RWG sphere (294.0 MB against 289.4 MB), scaled to the
-# 7680-RWG launch by its own algorithmic bytes (the stream grows with the
-# pairs stored)
-RT_TRAFFIC_RATIO = {"direct": 294.02 / 289.45, "direct32": 2363.4 / 2328.3, "direct24": None}
-RT_TRAFFIC_SOURCE = "profiles/direct_history_rt_sphere7680.md: ncu DRAM bytes of the same kernel over its algorithmic bytes"
 
 PREC = {"fp32": 0, "tf32": 1, "bf16": 2, "bf16x3": 3, "tf32x3": 4, "f16x3": 5}
 KERNELS = ["incident_rhs", "near_history", "z0_solve", "p2m", "m2m", "m2l", "l2l", "l2p", "m2l_pack",
@@ -251,10 +243,8 @@ def roofline(args, info, launches, ms, K, W):
         else:  # flattened entries: FP32 coefficient + (column << 8 | lag), 8 B per stored lag
             nbytes = 2 * info.near_coef_bytes
         gbs = nbytes / (ms[dom] / launches[dom] / 1e3) / 1e9
-        ratio = RT_TRAFFIC_RATIO.get(args.mode) if (info.history_bytes > 0 and args.rhs == 1) else None
-        traffic = ratio * nbytes if ratio else None
         return {"kernel": name, "bound": "hbm", "achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm,
-                "traffic": traffic, "traffic_source": RT_TRAFFIC_SOURCE if traffic else None,
+                "traffic": None, "traffic_source": None,
                 "peak_source": f"{src} hbm_gbs", "bytes_per_launch": nbytes}
     if name == "z0_solve" and info.z0_nnz > 0:
         # algorithmic operand bytes of one solve: per BiCGStab iteration two FP32
