@@ -253,6 +253,10 @@ static tdbem_status create(const double* verts, int64_t nv, const int32_t* tris,
   }
   if (!s) s = finish_create(c);
   if (!s && p.mode == TDBEM_DIRECT) s = tdbem_direct_split(c);
+  // (a budget also has to hold the incident rows that come after)
+  if (!s && !lean && p.max_device_bytes > 0 &&
+      c->device_bytes + (int64_t)Nt * c->ne * c->R * (int64_t)sizeof(double) > p.max_device_bytes)
+    s = TDBEM_ENOMEM;
   if (s) {
     tdbem_destroy(c);
     return s;
