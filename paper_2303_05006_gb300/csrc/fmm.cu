@@ -2069,9 +2069,17 @@ tdbem_status tdbem_fast_history(tdbem_ctx* c, int32_t alpha, const double* ring,
 }
 
 // -(lags >= 3) of step alpha into out[ne] on stream st: the tiled kernel
-// where it was built, else the flat one
+// where it was built, else the flat one.  Every such sum of a context goes
+// through the same segment sums (d_spart).  Those launched ahead follow each
+// other on the near stream, each behind the solve before it and so behind the
+// main stream's own sums; a sum on the main stream (the first two steps of a
+// march, the second one after a load, an evaluation in the middle of a march)
+// waits here for those launched ahead that no step has waited for yet.
 static tdbem_status near_lags3(tdbem_ctx* c, const double* ring, int32_t alpha, double* out, cudaStream_t st) {
   FmmPlan* F = c->fmm;
+  if (st != F->nstream)
+    for (int b = 0; b < 2; ++b)
+      if (F->ahead[b]) TDBEM_CUDA_TRY(c, cudaStreamWaitEvent(st, F->ev_near[b], 0));
   // the staged block holds the lags 0 .. max_near_lag of kNB columns
   const int nlag = F->max_near_lag + 1;
   const int smem = (int)(kNBS * nlag * sizeof(float));

@@ -1,0 +1,66 @@
+"""Sums launched ahead on a second stream, at the steps where a march has to do without them or meets them with
+something else in between: its first steps, the steps after a load, after a load that is refused, and after a
+history evaluation.
+
+Each step is checked by its residual: Z0 J^{a-1} against V^{a-1} minus the history, evaluated by the same context
+(two contexts of the fast method differ in the last bits of their coefficients).  March and evaluation add the same
+terms in the same order, so the solve's tolerance of 1e-13 is all that is left between them; the bar is 1e-10 of the
+right-hand side's scale.  A context's own marches of the same steps are equal to the last bit.
+"""
+import numpy as np
+import pytest
+
+from test_gpu_tilings import _oracle, _solver
+
+pytestmark = pytest.mark.gpu
+
+
+def _residuals_hold(J, Z0, evaluate, steps, bar=1e-10):
+    for a in steps:
+        b = evaluate(a, J[: a - 1])
+        assert np.abs(Z0 @ J[a - 1] - b).max() <= bar * np.abs(b).max(), a
+
+
+# far_kernel = 2: no far field, whose atomics would be above the bar
+def _fast(v, t, dt, n):
+    return _solver(v, t, dt, n + 2, mode=1, n_leaf=8, far_kernel=2)[0]
+
+
+@pytest.mark.parametrize("name,c", [("ell5", 0.3), ("cyl", 0.3)])
+def test_every_step_of_the_fast_march(tmp_path, name, c):
+    v, t, dt, o, mats, Z0 = _oracle(name, c)
+    n, k = 14, 6
+    s = _fast(v, t, dt, n)
+    J = s.march(n)
+    _residuals_hold(J, Z0, s.history_eval, range(1, n + 1))
+    # a state loaded over another march's
+    s.reset()
+    J1 = s.march(k)
+    path = str(tmp_path / "fast.ck")
+    s.save(path)
+    q = _fast(v, t, dt, n)
+    q.march(4)
+    q.load(path)
+    J2 = np.concatenate([J1, q.march(n - k)])
+    _residuals_hold(J2, Z0, q.history_eval, range(k + 1, n + 1))
+    # a load that is refused leaves the march as it was
+    s.reset()
+    J1 = s.march(k)
+    from paper_2303_05006_gb300 import TdbemError
+
+    with pytest.raises(TdbemError):
+        s.load(str(tmp_path / "missing.ck"))
+    assert np.array_equal(np.concatenate([J1, s.march(n - k)]), J)
+
+
+def test_an_evaluation_between_two_steps_of_the_fast_march():
+    v, t, dt, o, mats, Z0 = _oracle("ell5", 0.3)
+    n = 14
+    s = _fast(v, t, dt, n)
+    J = s.march(n)
+    s.reset()
+    for a in range(1, n + 1):
+        b = s.history_eval(a, J[: a - 1])
+        x = s.step()[0]
+        assert np.array_equal(x, J[a - 1]), a
+        assert np.abs(Z0 @ x - b).max() <= 1e-10 * np.abs(b).max(), a
