@@ -1528,12 +1528,22 @@ tdbem_status tdbem_direct_history(tdbem_ctx* c, int32_t alpha, const double* d_r
 // after the solve of step a0 - 1 + q (B = 1: J^{alpha-1} for step alpha + 2).  The
 // steps solved meanwhile write J^{a0-1} .. J^{a0+B-2}: the oldest current read,
 // J^{a0 + B - max_lag}, is at most L - 1 steps older, so no ring slot is shared.
-// The buffers were last read by kernels ordered before this solve.
+// The buffers were last read by kernels ordered before this solve.  A step whose
+// block will not be complete by then (the first block of a march or after a load)
+// sums its near pairs itself, so every launch here lies before an event that is
+// waited for: that of the far part, or that of the step's pre.
 tdbem_status tdbem_direct_after_solve(tdbem_ctx* c, int32_t alpha) {
   if (!c->dstream || !c->rt_prec || c->R != 1) return TDBEM_OK;
   const int32_t a2 = alpha + 2, af = alpha / c->rt_B * c->rt_B + 1 + c->rt_B;
   const bool far = af <= c->Nt - 1 && far_any(c, af);
   if (a2 > c->Nt - 1) return TDBEM_OK;  // af >= a2
+  // step alpha + 2's block, and whether its far sums are complete behind the side stream, this call's part included
+  const int32_t a0 = far_block(c, a2);
+  const int fb0 = far_buf(c, a0), q = alpha % c->rt_B;
+  const bool any = far_any(c, a0);
+  const int done = (c->far_blk[fb0] == a0 ? c->far_done[fb0] : 0) | (far && af == a0 ? 1 << q : 0);
+  const bool whole = !any || done == (1 << c->rt_B) - 1;
+  if (!far && !whole) return TDBEM_OK;
   TDBEM_CUDA_TRY(c, cudaEventRecord(c->ev_dsolved, c->stream));
   TDBEM_CUDA_TRY(c, cudaStreamWaitEvent(c->dstream, c->ev_dsolved, 0));
   cudaStream_t main = c->stream;
@@ -1542,20 +1552,16 @@ tdbem_status tdbem_direct_after_solve(tdbem_ctx* c, int32_t alpha) {
     const int b = a2 & 1;
     tdbem_status s;
     cudaEvent_t e = c->prof_begin(1);
-    if ((s = direct_near(c, a2, c->d_rs, b))) return s;
+    if (whole && (s = direct_near(c, a2, c->d_rs, b))) return s;
     if (far) {
-      const int fb = far_buf(c, af), q = alpha % c->rt_B;
+      const int fb = far_buf(c, af);
       if ((s = far_parts_wait(c, af)) || (s = direct_rt(c, af, c->rt_B, c->d_rs, q, far_out(c, fb)))) return s;
       TDBEM_CUDA_TRY(c, cudaEventRecord(c->ev_far[fb], c->dstream));
       c->far_done[fb] |= 1 << q;
       c->far_wait[fb] = true;
     }
-    // pre of step alpha + 2, if its block's far sums are complete and behind this stream
-    const int32_t a0 = far_block(c, a2);
-    const int fb = far_buf(c, a0), all = (1 << c->rt_B) - 1;
-    const bool any = far_any(c, a0);
-    if (!any || (c->far_blk[fb] == a0 && c->far_done[fb] == all)) {
-      if ((s = direct_presum(c, far_out(c, fb) + (int64_t)(a2 - a0) * c->rt_ncb * c->rt_nrt * 32, any ? c->rt_ncb : 0, b)))
+    if (whole) {
+      if ((s = direct_presum(c, far_out(c, fb0) + (int64_t)(a2 - a0) * c->rt_ncb * c->rt_nrt * 32, any ? c->rt_ncb : 0, b)))
         return s;
       c->dahead[b] = a2;
       TDBEM_CUDA_TRY(c, cudaEventRecord(c->ev_dahead[b], c->dstream));

@@ -64,3 +64,62 @@ def test_an_evaluation_between_two_steps_of_the_fast_march():
         x = s.step()[0]
         assert np.array_equal(x, J[a - 1]), a
         assert np.abs(Z0 @ x - b).max() <= 1e-10 * np.abs(b).max(), a
+
+
+# The direct march forms its far pairs' sums four steps a pass where its store is 64 MiB or more (8, 4 or 3 bytes a
+# coefficient): 1452 RWG.  Every step from its evaluation, solved in the first step of a march of its own, and every
+# other way to the same steps bit for bit.
+@pytest.mark.parametrize("prec,size", [(6, 8), (0, 4), (7, 3)])
+def test_every_step_of_the_blocked_direct_march(tmp_path, prec, size):
+    from paper_2303_05006_gb300 import TdbemError
+    from workloads.meshes import mean_edge_length, octa_ellipsoid
+
+    v, t = octa_ellipsoid(freq=11)
+    dt = 0.25 * mean_edge_length(v, t)
+    n = 27
+    s, pulses = _solver(v, t, dt, n + 2, p2p_prec=prec)
+    assert s.info().near_coef_bytes // 8 * size >= 64 << 20
+    J = s.march(n)
+    z, _ = _solver(v, t, dt, n + 2, p2p_prec=prec)
+    batch = None
+    if prec == 6:  # the batched form's sum reads the ring untiled
+        batch, _ = _solver(v, t, dt, n + 2, n_rhs=2)
+        batch.set_incident_plane(pulses[0], rhs=0)
+    for a in range(1, n + 1):
+        b = [s.history_eval(a, J[: a - 1])]
+        if batch is not None:
+            H = np.zeros((a - 1, 2, s.ne))
+            H[:, 0] = J[: a - 1]
+            b.append(batch.history_eval(a, H)[0])
+        for x in b:
+            V = np.zeros((n + 1, s.ne))
+            V[0] = x
+            z.reset()
+            z.set_rhs(V)
+            x = z.march(1)[0]
+            assert np.abs(J[a - 1] - x).max() <= 1e-10 * (np.abs(x).max() + np.abs(J[:a]).max()), a
+    z.close()
+    missing = str(tmp_path / "missing.ck")
+    q, _ = _solver(v, t, dt, n + 2, p2p_prec=prec)
+    for k in range(1, 14):
+        s.reset()  # whatever is in flight after step k - 1's sums ahead
+        J1 = s.march(k)
+        path = str(tmp_path / f"{k}.ck")
+        s.save(path)
+        with pytest.raises(TdbemError):
+            s.load(missing)
+        s.history_eval(k + 1, J[:k])
+        assert np.array_equal(np.concatenate([J1, s.march(n - k)]), J), k
+        q.reset()
+        q.march(3)
+        q.load(path)
+        assert np.array_equal(q.march(n - k), J[k:]), k
+        s.reset()
+        s.march_dev(k)
+    s.close()
+    for Nt in (7, 8, 9, 10):  # marches that end where a block's sums ahead would begin
+        e, _ = _solver(v, t, dt, Nt, p2p_prec=prec)
+        for _ in range(3):
+            e.reset()
+            assert np.array_equal(e.march(Nt - 1), J[: Nt - 1]), Nt
+        e.close()
