@@ -72,6 +72,7 @@ struct ScArgs {
   float* rf;                 // the ring's values in FP32 (may be null)
   int32_t L, alpha, warm, gpc, passes, npad, ne, maxit, R;
   double tol;
+  double zn2;                // |Z0|_1 |Z0|_inf, a bound of the squared 2-norm of (|Z0_ij|)
   int32_t* status;           // as in SolveArgs (solve.cu)
   double* resid;
 };
@@ -453,44 +454,70 @@ __global__ void __launch_bounds__(kScThreads) k_solve_cluster(const ScArgs A) {
 #pragma unroll
     for (int e = 0; e < RPT; ++e) r[e] = row[e] >= 0 ? b[e] - r[e] : 0.0;
   };
-  auto norm2 = [&](const double(&r)[RPT], double& rr, double& bb) {
-    rr = bb = 0.0;
+  // the sums of r^2 and w^2 over all rows
+  auto norm2 = [&](const double(&r)[RPT], const double(&w)[RPT], double& rr, double& ww) {
+    rr = ww = 0.0;
 #pragma unroll
     for (int e = 0; e < RPT; ++e) {
       rr += r[e] * r[e];
-      bb += b[e] * b[e];
+      ww += w[e] * w[e];
     }
-    S.sums64(rr, bb);
+    S.sums64(rr, ww);
   };
   double rr = 0.0, bb = 0.0;
   int inner_total = 0;
   bool conv = false;
   // The start: the extrapolation; with warm 2 also the caller's guess in A.x,
   // kept only if its FP64 residual is smaller (a NaN never is).
+  // A residual that is carried on (r -= Z0 d) misses the rounding of x, half an
+  // ulp a pass, and that of Z0 d in double-float, 2^-43 with a row's sum; over four
+  // passes |missed|^2 <= 2^-101 zn2 (|x|^2 + 2^18 sum |d|^2).  It decides only where the
+  // tolerance holds with that added, and b - Z0 x is formed anew in FP64 where it does
+  // not.  (Few FP64 operations: each costs a CTA 0.12 us.)
+  constexpr int kScCarry = 4;
+  bool anew = true;
+  int passes = 0;  // carried on since the last FP64 residual, at 2^k0 with
+  float dd = 0.f;  // this thread's share of sum |d|^2 / 4^k0 over them
+  int k0 = 0;
+  double tol2bb = 0.0;
 #pragma unroll 1
   for (int outer = -1;; ++outer) {
-    double nr, nbb;
-    if (outer < 0 || !(rr <= 0x1p-16 * bb)) {
+    const bool carried = !anew && passes < kScCarry && rr <= 0x1p-16 * bb;
+    anew = false;
+    if (!carried) {
       residual(x, w64, r64);
+      norm2(r64, b, rr, bb);
+      tol2bb = A.tol * A.tol * bb;
+      passes = 0;
+      dd = 0.f;
     } else {
-      // The correction (y: its FP32 digits) is at most about 2^-8 of the iterate:
-      // Z0 d in double-float (46 bits) is then as exact as b - Z0 x anew in FP64.
       double zd[RPT];
       sc_spmv<RPT>(LdZdf{A.zhi, A.zlo, A.zcol, sc_X}, zb, ztot, zends, lane, zd);
       const int kx = max((((__double2hiint(rr) >> 20) & 0x7ff) - 1023) >> 1, -500);
       const double sc = __hiloint2double((1023 + kx) << 20, 0);
 #pragma unroll
       for (int e = 0; e < RPT; ++e) r64[e] = row[e] >= 0 ? r64[e] - sc * zd[e] : 0.0;
+      ++passes;
+      double nr = 0.0, xx = (double)(0x1p18f * dd) * __hiloint2double((1023 + 2 * k0) << 20, 0);
+#pragma unroll
+      for (int e = 0; e < RPT; ++e) {
+        nr += r64[e] * r64[e];
+        xx += x[e] * x[e];
+      }
+      S.sums64(nr, xx);
+      rr = nr;
+      if (rr <= tol2bb && rr + 0x1p-101 * A.zn2 * xx > 0.5 * tol2bb) {
+        anew = true;
+        --outer;
+        continue;
+      }
     }
-    norm2(r64, nr, nbb);
-    rr = nr;
-    bb = nbb;
     if (outer < 0 && A.warm == 2) {
       double g[RPT], rg[RPT], gg, b2;
 #pragma unroll
       for (int e = 0; e < RPT; ++e) g[e] = row[e] >= 0 ? A.x[(int64_t)row[e] * R + rhs] : 0.0;
       residual(g, w64 + A.npad, rg);
-      norm2(rg, gg, b2);
+      norm2(rg, b, gg, b2);
       const bool keep = gg < rr;
       if (keep) {
         rr = gg;
@@ -502,7 +529,6 @@ __global__ void __launch_bounds__(kScThreads) k_solve_cluster(const ScArgs A) {
       }
       if (S.rank == 0 && threadIdx.x == 0) atomicAdd(&A.status[keep ? 8 : 9], 1);
     }
-    const double tol2bb = A.tol * A.tol * bb;
     if (rr <= tol2bb) {
       conv = true;
       break;
@@ -586,6 +612,11 @@ __global__ void __launch_bounds__(kScThreads) k_solve_cluster(const ScArgs A) {
     sc_spmv<RPT>(LdA{A.pval, A.pcol, sc_X}, pb, ptot, pends, lane, y);
 #pragma unroll
     for (int e = 0; e < RPT; ++e) x[e] += sc * (double)y[e];
+    float yy = 0.f;
+#pragma unroll
+    for (int e = 0; e < RPT; ++e) yy = fmaf(y[e], y[e], yy);
+    if (passes == 0) k0 = kx;
+    dd = fmaf(ldexpf(1.f, max(2 * (kx - k0), -120)), yy, dd);
     if (rr <= 0x1p-16 * bb) {
       S.sync();  // every CTA has gathered y
       push(y);
@@ -1033,6 +1064,7 @@ struct ScPlan {
   double2* zval = nullptr;
   uint2 *acol = nullptr, *zcol = nullptr, *pcol = nullptr;
   double* w64 = nullptr;
+  double zn2 = 0.0;
   bool bx = false;                 // k_bicgstab_x: rows per CTA, Z0's FP32 blocks, the triangle blocks are the context's
   int rows = 0;
   float4* z32 = nullptr;
@@ -1296,6 +1328,20 @@ tdbem_status tdbem_sc_build(tdbem_ctx* c, int want, const std::vector<int32_t>& 
       }
     np[i + 1] = (int64_t)nc.size();
   }
+  {
+    std::vector<double> colsum(ne, 0.0);
+    double most_row = 0.0, most_col = 0.0;
+    for (int i = 0; i < ne; ++i) {
+      double r = 0.0;
+      for (int64_t k = np[i]; k < np[i + 1]; ++k) {
+        r += std::fabs(nv[k]);
+        colsum[nc[k]] += std::fabs(nv[k]);
+      }
+      most_row = std::max(most_row, r);
+    }
+    for (double v : colsum) most_col = std::max(most_col, v);
+    P.zn2 = most_row * most_col;
+  }
   // P
   std::vector<int64_t> pp(ne + 1, 0);
   std::vector<int32_t> pc;
@@ -1540,6 +1586,7 @@ tdbem_status tdbem_sc_solve(tdbem_ctx* c, int32_t alpha, int32_t warm) {
   A.R = c->R;
   A.maxit = c->p.solve_maxit;
   A.tol = c->p.solve_tol;
+  A.zn2 = P.zn2;
   A.status = c->d_status;
   A.resid = c->d_dots;
   c->cluster = P.cs;
