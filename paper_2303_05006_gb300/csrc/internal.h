@@ -308,9 +308,12 @@ void tdbem_mlp_free(tdbem_ctx* c);
 tdbem_status tdbem_build_z0(tdbem_ctx* c);
 tdbem_status tdbem_build_z0_csr(tdbem_ctx* c);
 tdbem_status tdbem_solve_z0(tdbem_ctx* c, int32_t alpha, int32_t* iters, int32_t warm);
+// the triangle blocks' rows (solve.cu)
+void tdbem_triangle_rows(const tdbem_ctx* c, const std::vector<int32_t>& hp, const std::vector<int32_t>& hc,
+                         const std::vector<double>& hv, std::vector<int32_t>* pcol, std::vector<double>* pval);
 // solve_cluster.cu: the cluster solve, a cluster per right-hand side, for the context's Z0
 // (CSR on the device, and here on the host); want: CTAs of the cluster at most.
-// No plan is made (c->sc stays null) where the mesh does not fit it.
+// No plan is made (c->sc stays null) where the mesh does not fit it or a trial solve does not converge.
 tdbem_status tdbem_sc_build(tdbem_ctx* c, int want, const std::vector<int32_t>& zp, const std::vector<int32_t>& zc,
                             const std::vector<double>& zv);
 // the same for the FP32 and 24-bit direct marches: k_bicgstab's own arithmetic

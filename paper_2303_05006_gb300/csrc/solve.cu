@@ -955,17 +955,19 @@ static bool use_grid(const tdbem_ctx* c) {
 // and P = sum over triangles of the inverses scattered to their rows and
 // columns.  Row i of P couples edge i with the other sides of its two
 // triangles (at most kPc entries).  A triangle whose block is singular adds
-// its diagonal reciprocals instead.
-static tdbem_status build_triangle_precond(tdbem_ctx* c, const std::vector<int32_t>& hp, const std::vector<int32_t>& hc,
-                                           const std::vector<double>& hv) {
+// its diagonal reciprocals instead.  pcol, pval: ELL [kPc][ne], unused entries zero.
+void tdbem_triangle_rows(const tdbem_ctx* c, const std::vector<int32_t>& hp, const std::vector<int32_t>& hc,
+                         const std::vector<double>& hv, std::vector<int32_t>* pcol_out, std::vector<double>* pval_out) {
   const int64_t ne = c->ne;
   auto z = [&](int32_t i, int32_t j) {
     for (int32_t k = hp[i]; k < hp[i + 1]; ++k)
       if (hc[k] == j) return hv[k];
     return 0.0;
   };
-  std::vector<int32_t> pcol(kPc * ne, 0);
-  std::vector<double> pval(kPc * ne, 0.0);
+  std::vector<int32_t>& pcol = *pcol_out;
+  std::vector<double>& pval = *pval_out;
+  pcol.assign(kPc * ne, 0);
+  pval.assign(kPc * ne, 0.0);
   std::vector<int> used(ne, 0);
   auto add = [&](int32_t i, int32_t j, double v) {
     for (int k = 0; k < used[i]; ++k)
@@ -1001,6 +1003,14 @@ static tdbem_status build_triangle_precond(tdbem_ctx* c, const std::vector<int32
       for (int a = 0; a < 3; ++a)
         if (B[a][a] != 0.0) add(e[a], e[a], 1.0 / B[a][a]);
   }
+}
+
+static tdbem_status build_triangle_precond(tdbem_ctx* c, const std::vector<int32_t>& hp, const std::vector<int32_t>& hc,
+                                           const std::vector<double>& hv) {
+  const int64_t ne = c->ne;
+  std::vector<int32_t> pcol;
+  std::vector<double> pval;
+  tdbem_triangle_rows(c, hp, hc, hv, &pcol, &pval);
   std::vector<float> pv32(kPc * ne);
   for (int64_t k = 0; k < kPc * ne; ++k) pv32[k] = (float)pval[k];
   tdbem_status s;

@@ -51,6 +51,8 @@ constexpr int kScPasses = 24;       // groups per warp at most: 6 rows per threa
 constexpr double kScInner2 = 1e-10; // squared relative residual an inner solve stops at
 constexpr int kScDepth = 4;          // blocks a warp keeps in flight
 constexpr int kScInnerMax = 80;     // iterations of one inner solve
+constexpr int kScTrial = 2 * kScInnerMax;  // most iterations to 1e-5 that a plan may take: 1e-13 is then six of eight inner solves
+constexpr int kScGood = 24;         // above these another preconditioner is tried
 
 struct ScArgs {
   const int32_t* perm;       // [npad] row at a position, -1: padding
@@ -1277,6 +1279,136 @@ __global__ void __launch_bounds__(kLiWarps * 32) k_local_inverse(const int32_t* 
   pval[(int64_t)i * kScK + lane] = lane < n ? y : 0.f;
 }
 
+// The plan's arrays for a preconditioner P: A = Z0 P and the order of its rows.
+static tdbem_status sc_arrays(tdbem_ctx* c, ScPlan* out, const ScMat& Z, const ScMat& M) {
+  ScPlan& P = *out;
+  const int ne = (int)c->ne;
+  const std::vector<int64_t>&np = Z.ptr, &pp = M.ptr;
+  const std::vector<int32_t>&nc = Z.col, &pc = M.col;
+  const std::vector<double>&nv = Z.val, &pv = M.val;
+  tdbem_status s;
+  // A = Z0 P, row by row
+  std::vector<int64_t> ap(ne + 1, 0);
+  std::vector<int32_t> ac, at(ne, -1), rowc;
+  std::vector<double> av, acc(ne, 0.0);
+  for (int i = 0; i < ne; ++i) {
+    rowc.clear();
+    for (int64_t k = np[i]; k < np[i + 1]; ++k) {
+      const double z = nv[k];
+      const int j = nc[k];
+      for (int64_t m = pp[j]; m < pp[j + 1]; ++m) {
+        const int l = pc[m];
+        if (at[l] != i) {
+          at[l] = i;
+          acc[l] = 0.0;
+          rowc.push_back(l);
+        }
+        acc[l] += z * pv[m];
+      }
+    }
+    for (int l : rowc)
+      if (std::fabs(acc[l]) > kScDrop) {
+        ac.push_back(l);
+        av.push_back(acc[l]);
+      }
+    ap[i + 1] = (int64_t)ac.size();
+  }
+  // order: rows by their blocks of A, longest first (stable), in groups of 8 dealt over the CTAs
+  std::vector<int32_t> ord(ne);
+  for (int i = 0; i < ne; ++i) ord[i] = i;
+  std::stable_sort(ord.begin(), ord.end(), [&](int32_t a, int32_t b) {
+    return (ap[a + 1] - ap[a] + 15) / 16 > (ap[b + 1] - ap[b] + 15) / 16;
+  });
+  std::vector<int32_t> perm(P.npad, -1), at_pos(ne);
+  int next = 0;
+  for (int j = 0; j < P.passes && next < ne; ++j)
+    for (int u = 0; u < P.cs * kScWarps && next < ne; ++u) {
+      const int f = j & 1 ? P.cs * kScWarps - 1 - u : u;  // there and back: long and short groups meet
+      const int k = f % P.cs, g = j * kScWarps + f / P.cs;
+      if (g >= P.gpc) continue;
+      for (int t = 0; t < 8 && next < ne; ++t, ++next) {
+        const int64_t p = ((int64_t)k * P.gpc + g) * 8 + t;
+        perm[p] = ord[next];
+        at_pos[ord[next]] = (int32_t)p;
+      }
+    }
+  if ((s = sc_upload(c, &P.perm, perm)) ||
+      (s = sc_matrix(c, P, perm, at_pos, {ap, ac, av}, &P.ab, &P.ae, &P.aval, nullptr, nullptr, &P.acol)) ||
+      (s = sc_matrix(c, P, perm, at_pos, M, &P.pb, &P.pe, &P.pval, nullptr, nullptr, &P.pcol)) ||
+      (s = sc_matrix(c, P, perm, at_pos, Z, &P.zb, &P.ze, &P.zhi, &P.zlo, &P.zval, &P.zcol)) ||
+      (s = c->dalloc(&P.w64, 2 * (size_t)P.npad * c->R)))
+    return s;
+  TDBEM_CUDA_TRY(c, cudaMemsetAsync(P.w64, 0, 2 * (size_t)P.npad * c->R * sizeof(double), c->stream));
+  return TDBEM_OK;
+}
+
+static void sc_drop(tdbem_ctx* c, ScPlan* P) {
+  for (void* d : {(void*)P->perm, (void*)P->ab, (void*)P->ae, (void*)P->aval, (void*)P->acol, (void*)P->zb, (void*)P->ze,
+                  (void*)P->zval, (void*)P->zhi, (void*)P->zlo, (void*)P->zcol, (void*)P->pb, (void*)P->pe,
+                  (void*)P->pval, (void*)P->pcol, (void*)P->w64})
+    if (d) c->dfree(d);
+}
+
+static ScArgs sc_args(const tdbem_ctx* c, const ScPlan& P) {
+  ScArgs A = {};
+  A.perm = P.perm;
+  A.ab = P.ab;
+  A.ae = P.ae;
+  A.aval = P.aval;
+  A.acol = P.acol;
+  A.zb = P.zb;
+  A.ze = P.ze;
+  A.zval = P.zval;
+  A.zhi = P.zhi;
+  A.zlo = P.zlo;
+  A.zcol = P.zcol;
+  A.pb = P.pb;
+  A.pe = P.pe;
+  A.pval = P.pval;
+  A.pcol = P.pcol;
+  A.w64 = P.w64;
+  A.gpc = P.gpc;
+  A.passes = P.passes;
+  A.npad = P.npad;
+  A.ne = (int32_t)c->ne;
+  A.zn2 = P.zn2;
+  A.status = c->d_status;
+  A.resid = c->d_dots;
+  return A;
+}
+
+// Iterations that the plan takes to 1e-5 for one right-hand side of every frequency, kScTrial where that is not enough.
+static tdbem_status sc_trial(tdbem_ctx* c, const ScPlan& P, int* its) {
+  const int64_t ne = c->ne;
+  std::vector<double> b(ne);
+  uint64_t h = 1;
+  for (double& v : b) {
+    h = h * 6364136223846793005ull + 1442695040888963407ull;
+    v = (double)(int64_t)h * 0x1p-63;
+  }
+  // d_work serves the solves that have no plan; the ring is one step long here
+  TDBEM_CUDA_TRY(c, cudaMemcpyAsync(c->d_work, b.data(), ne * sizeof(double), cudaMemcpyHostToDevice, c->stream));
+  TDBEM_CUDA_TRY(c, cudaMemsetAsync(c->d_status, 0, 16 * sizeof(int32_t), c->stream));
+  ScArgs A = sc_args(c, P);
+  A.b = c->d_work;
+  A.x = c->d_work + ne;
+  A.ring = c->d_work + 2 * ne;
+  A.L = 1;
+  A.alpha = 1;
+  A.R = 1;
+  A.maxit = kScTrial;
+  A.tol = 2e-5;
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute at;
+  sc_config(&cfg, &at, P.cs, P.cs, sc_smem(P), c->stream);
+  TDBEM_CUDA_TRY(c, cudaLaunchKernelEx(&cfg, sc_fn(P.passes), A));
+  int32_t st[2];
+  TDBEM_CUDA_TRY(c, cudaMemcpyAsync(st, c->d_status, sizeof(st), cudaMemcpyDeviceToHost, c->stream));
+  TDBEM_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  *its = st[1] ? st[0] : kScTrial;
+  return TDBEM_OK;
+}
+
 tdbem_status tdbem_sc_build(tdbem_ctx* c, int want, const std::vector<int32_t>& zp, const std::vector<int32_t>& zc,
                             const std::vector<double>& zv) {
   const int ne = (int)c->ne;
@@ -1342,6 +1474,8 @@ tdbem_status tdbem_sc_build(tdbem_ctx* c, int want, const std::vector<int32_t>& 
     for (double v : colsum) most_col = std::max(most_col, v);
     P.zn2 = most_row * most_col;
   }
+  const ScPlan base = P;
+  const ScMat Z = {np, nc, nv};
   // P
   std::vector<int64_t> pp(ne + 1, 0);
   std::vector<int32_t> pc;
@@ -1380,58 +1514,40 @@ tdbem_status tdbem_sc_build(tdbem_ctx* c, int want, const std::vector<int32_t>& 
       pp[i + 1] = (int64_t)pc.size();
     }
   }
-  // A = Z0 P, row by row
-  std::vector<int64_t> ap(ne + 1, 0);
-  std::vector<int32_t> ac, at(ne, -1), rowc;
-  std::vector<double> av, acc(ne, 0.0);
-  for (int i = 0; i < ne; ++i) {
-    rowc.clear();
-    for (int64_t k = np[i]; k < np[i + 1]; ++k) {
-      const double z = nv[k];
-      const int j = nc[k];
-      for (int64_t m = pp[j]; m < pp[j + 1]; ++m) {
-        const int l = pc[m];
-        if (at[l] != i) {
-          at[l] = i;
-          acc[l] = 0.0;
-          rowc.push_back(l);
+  // Rows of local inverses do best where Z0 couples near neighbours: 1 to 11 iterations to 1e-5 at time steps up to half
+  // an edge length, on spheres and slivers.  At steps of many edge lengths Z0 is full, and where a sliver's
+  // pole gathers more strong couplings than a row takes, the truncated blocks' inverses spoil it (UV
+  // ellipsoid of 2880 RWG, steps of 32 edge lengths: 174 iterations against 66 with the triangle blocks; 1e-13 not
+  // reached).  So where the trial takes more than kScGood, the triangle blocks are tried too; the better one is kept,
+  // and where neither converges there is no plan and the general kernel solves.
+  int its = kScTrial;
+  if ((s = sc_arrays(c, &P, Z, {pp, pc, pv})) || (s = sc_trial(c, P, &its))) return s;
+  if (c->p.precond == 1 && its > kScGood) {
+    std::vector<int32_t> ec;
+    std::vector<double> ev;
+    tdbem_triangle_rows(c, zp, zc, zv, &ec, &ev);
+    std::vector<int64_t> tp(ne + 1, 0);
+    std::vector<int32_t> tc;
+    std::vector<double> tv;
+    for (int i = 0; i < ne; ++i) {
+      for (size_t k = i; k < ec.size(); k += ne)
+        if (ev[k] != 0.0) {
+          tc.push_back(ec[k]);
+          tv.push_back(ev[k]);
         }
-        acc[l] += z * pv[m];
-      }
+      tp[i + 1] = (int64_t)tc.size();
     }
-    for (int l : rowc)
-      if (std::fabs(acc[l]) > kScDrop) {
-        ac.push_back(l);
-        av.push_back(acc[l]);
-      }
-    ap[i + 1] = (int64_t)ac.size();
+    ScPlan T = base;
+    int its2 = kScTrial;
+    if ((s = sc_arrays(c, &T, Z, {tp, tc, tv})) || (s = sc_trial(c, T, &its2))) return s;
+    if (its2 < its) std::swap(P, T);
+    its = std::min(its, its2);
+    sc_drop(c, &T);
   }
-  // order: rows by their blocks of A, longest first (stable), in groups of 8 dealt over the CTAs
-  std::vector<int32_t> ord(ne);
-  for (int i = 0; i < ne; ++i) ord[i] = i;
-  std::stable_sort(ord.begin(), ord.end(), [&](int32_t a, int32_t b) {
-    return (ap[a + 1] - ap[a] + 15) / 16 > (ap[b + 1] - ap[b] + 15) / 16;
-  });
-  std::vector<int32_t> perm(P.npad, -1), at_pos(ne);
-  int next = 0;
-  for (int j = 0; j < P.passes && next < ne; ++j)
-    for (int u = 0; u < P.cs * kScWarps && next < ne; ++u) {
-      const int f = j & 1 ? P.cs * kScWarps - 1 - u : u;  // there and back: long and short groups meet
-      const int k = f % P.cs, g = j * kScWarps + f / P.cs;
-      if (g >= P.gpc) continue;
-      for (int t = 0; t < 8 && next < ne; ++t, ++next) {
-        const int64_t p = ((int64_t)k * P.gpc + g) * 8 + t;
-        perm[p] = ord[next];
-        at_pos[ord[next]] = (int32_t)p;
-      }
-    }
-  if ((s = sc_upload(c, &P.perm, perm)) ||
-      (s = sc_matrix(c, P, perm, at_pos, {ap, ac, av}, &P.ab, &P.ae, &P.aval, nullptr, nullptr, &P.acol)) ||
-      (s = sc_matrix(c, P, perm, at_pos, {pp, pc, pv}, &P.pb, &P.pe, &P.pval, nullptr, nullptr, &P.pcol)) ||
-      (s = sc_matrix(c, P, perm, at_pos, {np, nc, nv}, &P.zb, &P.ze, &P.zhi, &P.zlo, &P.zval, &P.zcol)) ||
-      (s = c->dalloc(&P.w64, 2 * (size_t)P.npad * c->R)))
-    return s;
-  TDBEM_CUDA_TRY(c, cudaMemsetAsync(P.w64, 0, 2 * (size_t)P.npad * c->R * sizeof(double), c->stream));
+  if (its == kScTrial) {
+    sc_drop(c, &P);
+    return TDBEM_OK;
+  }
   c->sc = new (std::nothrow) ScPlan(P);
   return c->sc ? TDBEM_OK : TDBEM_ENOMEM;
 }
@@ -1554,23 +1670,7 @@ static tdbem_status bx_solve(tdbem_ctx* c, int32_t alpha, int32_t warm) {
 tdbem_status tdbem_sc_solve(tdbem_ctx* c, int32_t alpha, int32_t warm) {
   if (c->sc->bx) return bx_solve(c, alpha, warm);
   const ScPlan& P = *c->sc;
-  ScArgs A;
-  A.perm = P.perm;
-  A.ab = P.ab;
-  A.ae = P.ae;
-  A.aval = P.aval;
-  A.acol = P.acol;
-  A.zb = P.zb;
-  A.ze = P.ze;
-  A.zval = P.zval;
-  A.zhi = P.zhi;
-  A.zlo = P.zlo;
-  A.zcol = P.zcol;
-  A.pb = P.pb;
-  A.pe = P.pe;
-  A.pval = P.pval;
-  A.pcol = P.pcol;
-  A.w64 = P.w64;
+  ScArgs A = sc_args(c, P);
   A.b = c->d_R;
   A.x = c->d_J;
   A.ring = c->d_Jring;
@@ -1579,16 +1679,9 @@ tdbem_status tdbem_sc_solve(tdbem_ctx* c, int32_t alpha, int32_t warm) {
   A.L = c->L;
   A.alpha = alpha;
   A.warm = warm;
-  A.gpc = P.gpc;
-  A.passes = P.passes;
-  A.npad = P.npad;
-  A.ne = (int32_t)c->ne;
   A.R = c->R;
   A.maxit = c->p.solve_maxit;
   A.tol = c->p.solve_tol;
-  A.zn2 = P.zn2;
-  A.status = c->d_status;
-  A.resid = c->d_dots;
   c->cluster = P.cs;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute at;

@@ -52,3 +52,14 @@ def test_a_tolerance_above_it_is_met(name, tol, R):
     y = _solver(v, t, 0.5, 4, R, solve_tol=tol, jacobi_sweeps=1).march(4)
     # both residuals are below tol |b|; the condition number is below 4000 on the slivers, 100 elsewhere
     assert np.abs(x - y).max() <= 2 * (4000 if name == "uv13" else 100) * tol * np.abs(y).max()
+
+
+# Steps of many edge lengths: Z0 is full, and the rows of local inverses no longer precondition it.
+@pytest.mark.parametrize("name,c", [("uv13", 32.0), ("uv13", 256.0), ("cyl", 256.0), ("ico1", 64.0)])
+@pytest.mark.parametrize("R,precond", [(1, 1), (2, 1), (1, 0)])
+def test_steps_of_many_edge_lengths(name, c, R, precond):
+    v, t = _mesh(name)
+    x = _solver(v, t, c, 4, R, precond=precond).march(4)
+    y = _solver(v, t, c, 4, R, precond=precond, jacobi_sweeps=1).march(4)
+    # as above: both residuals below 1e-13 |b|
+    assert np.abs(x - y).max() <= 2 * (4000 if name == "uv13" else 100) * 1e-13 * np.abs(y).max()
