@@ -1083,7 +1083,7 @@ __global__ void k_rt_meta(const int16_t* m_lo, const uint8_t* nlag, int64_t ne, 
 #pragma unroll
   for (int d = 1; d < 8; d <<= 1) nn = max(nn, __shfl_xor_sync(0xffffffffu, nn, d));
   lo3[wid * 32 + lane] = (uint8_t)l3;
-  if ((lane & 7) == 0) nnear[(4 * rt + lane / 8) * ne + j] = (uint8_t)nn;
+  if (nnear && (lane & 7) == 0) nnear[(4 * rt + lane / 8) * ne + j] = (uint8_t)nn;
   if (lane == 0) {
     nmax[wid] = (uint8_t)mx;
     atomicMax(lh, need);
@@ -1691,7 +1691,7 @@ static tdbem_status build_row_tiles(tdbem_ctx* c, int prec) {
   const int units = prec != 2;  // FP32 and 24-bit: whole units of 64 columns in edge order
   const int m0 = units ? 3 : rt_m0(B, B - 1), most = prec == 2 ? 2 : 3;  // blocks per SM the registers allow
   int cbw = 64;
-  if (!units) {
+  if (!units && !c->lean) {
     const int lag = std::min(255, c->max_lag + 6), sms = nsm > 32 ? nsm - 16 : nsm;
     double best = 1e300;
     for (int w = 8; w <= 96; w += 2) {
@@ -1706,29 +1706,33 @@ static tdbem_status build_row_tiles(tdbem_ctx* c, int prec) {
     }
   }
   const int ncb = (int)((ne + cbw - 1) / cbw);
+  const bool quads = B > 1 && !units;
   uint8_t *d_nmax = nullptr, *d_nnear = nullptr;
-  int32_t* d_lh = nullptr;
-  if ((s = c->dalloc(&d_nmax, ntc)) || (s = c->dalloc(&d_nnear, 4 * ntc)) || (s = c->dalloc(&c->d_rt_lo, ntc * 32)) ||
-      (s = c->dalloc(&c->d_rt_lomin, nrt * ncb)) || (s = c->dalloc(&d_lh, 1)) || (s = c->dalloc(&c->d_dt_err, 1)))
+  int32_t *d_lh = nullptr, *d_lomin = nullptr;
+  if ((s = c->dalloc(&d_nmax, ntc)) || (quads && (s = c->dalloc(&d_nnear, 4 * ntc))) ||
+      (s = c->dalloc(&c->d_rt_lo, ntc * 32)) || (s = c->dalloc(&d_lomin, nrt * ncb)) || (s = c->dalloc(&d_lh, 1)) ||
+      (s = c->dalloc(&c->d_dt_err, 1)))
     return s;
   TDBEM_CUDA_TRY(c, cudaMemsetAsync(d_lh, 0, sizeof(int32_t), c->stream));
   TDBEM_CUDA_TRY(c, cudaMemsetAsync(c->d_dt_err, 0, sizeof(int32_t), c->stream));
-  TDBEM_CUDA_TRY(c, cudaMemsetAsync(c->d_rt_lomin, 0x7f, nrt * ncb * sizeof(int32_t), c->stream));
+  TDBEM_CUDA_TRY(c, cudaMemsetAsync(d_lomin, 0x7f, nrt * ncb * sizeof(int32_t), c->stream));
   const unsigned nb = (unsigned)((ntc * 32 + 255) / 256);
   k_rt_meta<<<nb, 256, 0, c->stream>>>(st.m_lo, st.nlag, ne, (int32_t)nrt, c->d_rt_row, B, units, d_nmax, d_nnear,
-                                       c->d_rt_lo, c->d_rt_lomin, ncb, cbw, d_lh);
+                                       c->d_rt_lo, d_lomin, ncb, cbw, d_lh);
   TDBEM_CUDA_TRY(c, cudaGetLastError());
-  const bool quads = B > 1 && !units;
   std::vector<uint8_t> nmax(ntc), nnear(quads ? 4 * ntc : 0);
-  std::vector<int32_t> rows(nrt * 32);
+  std::vector<int32_t> rows(nrt * 32), lm(nrt * ncb);
   int32_t lh = 0;
   TDBEM_CUDA_TRY(c, cudaMemcpyAsync(nmax.data(), d_nmax, ntc, cudaMemcpyDeviceToHost, c->stream));
   if (quads) TDBEM_CUDA_TRY(c, cudaMemcpyAsync(nnear.data(), d_nnear, 4 * ntc, cudaMemcpyDeviceToHost, c->stream));
   TDBEM_CUDA_TRY(c, cudaMemcpyAsync(rows.data(), c->d_rt_row, nrt * 32 * sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
+  TDBEM_CUDA_TRY(c, cudaMemcpyAsync(lm.data(), d_lomin, lm.size() * sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
   TDBEM_CUDA_TRY(c, cudaMemcpyAsync(&lh, d_lh, sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
   TDBEM_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  // (what the march alone reads comes back when the FP64 values are gone: the two stores side by side are the peak)
   c->dfree(d_nmax);
   c->dfree(d_nnear);
+  c->dfree(d_lomin);
   c->dfree(d_lh);
   std::vector<uint32_t> goff(ntc + 1);
   uint64_t acc = 0;
@@ -1809,10 +1813,7 @@ static tdbem_status build_row_tiles(tdbem_ctx* c, int prec) {
   c->rt_nslot = units && B > 1 ? ncb : nslot;
   // streamed per step: the far pairs' share once per B steps, the near ones each step
   int64_t whole = (int64_t)nbytes + ntc * 32 + (ntc + 1) * 4, near = (int64_t)nearbytes + nq * (128 + 4);
-  std::vector<int32_t> lm(nrt * ncb), list, loff(1, 0);
-  TDBEM_CUDA_TRY(c, cudaMemcpyAsync(lm.data(), c->d_rt_lomin, lm.size() * sizeof(int32_t), cudaMemcpyDeviceToHost,
-                                    c->stream));
-  TDBEM_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  std::vector<int32_t> list, loff(1, 0);
   for (int l = 0; l <= B; ++l) {  // the far tiles of each part, then the near ones
     int most_tiles = 0;
     for (int cb = 0; cb < ncb; ++cb) {
@@ -1838,7 +1839,7 @@ static tdbem_status build_row_tiles(tdbem_ctx* c, int prec) {
     // the far parts: a tile per warp; the near units, fewer and unevenly spread: by the cost
     c->rt_ltiles[l] = l < B ? kRtWarps : rt_tiles(std::max(1, most_tiles), ncb, slots, cbw);
   }
-  if ((s = up(c, &c->d_rt_list, list)) || (s = up(c, &c->d_rt_loff, loff))) return s;
+  if ((s = up(c, &c->d_rt_list, list)) || (s = up(c, &c->d_rt_loff, loff)) || (s = up(c, &c->d_rt_lomin, lm))) return s;
   TDBEM_CUDA_TRY(c, cudaStreamSynchronize(c->stream));  // the vectors go
   if (units && B > 1) whole -= near;
   c->rt_bytes = whole / B + near;
@@ -1859,12 +1860,17 @@ tdbem_status tdbem_direct_split(tdbem_ctx* c) {
   if (c->R != 1) return TDBEM_OK;
   PairStore& st = c->direct;
   // The row-tile store's first lags are bytes and its history of a column block
-  // lies in shared memory: rings of up to 256 steps in (hi, lo) pairs.
-  const bool tiled = c->L <= 128 || (c->L <= 256 && c->p.p2p_prec == TDBEM_P_FP64);
+  // lies in shared memory: rings of up to 256 steps in (hi, lo) pairs.  It is built beside the FP64 values, where the
+  // untiled form turns them into pairs in place: the memory of a lean context has no room for that beyond 128 steps.
+  const bool tiled = c->L <= 128 || (c->L <= 256 && c->p.p2p_prec == TDBEM_P_FP64 && !c->lean);
   if (tiled) {
     // the row order, and the lag-2 entries (read from the FP64 store before the row tiles replace it)
     const int64_t ne = c->ne, nrt = (ne + 31) / 32, npos = nrt * 32;
-    std::vector<int32_t> rows = bisected_edges(c), cnt(npos), ptr(npos + 1, 0);
+    std::vector<int32_t> rows, cnt(npos), ptr(npos + 1, 0);
+    if (c->lean)  // the numbering's own order, whose store may be smaller (UV ellipsoid of 2,880 RWG: by a tenth)
+      for (int32_t e = 0; e < ne; ++e) rows.push_back(e);
+    else
+      rows = bisected_edges(c);
     rows.resize(npos, -1);
     tdbem_status s0;
     if ((s0 = up(c, &c->d_rt_row, rows)) || (s0 = c->dalloc(&c->d_l2_ptr, npos + 1))) return s0;

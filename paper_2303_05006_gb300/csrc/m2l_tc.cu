@@ -1215,7 +1215,7 @@ tdbem_status tdbem_m2l_tc(tdbem_ctx* c, int mt, const int4* gemm, const int4* ti
 // k_m2l_tc (allocated here, owned by the context).  The FP16 form scales each
 // operator by a power of two first; *opinv (allocated here, 2 nop floats)
 // then holds the inverse scales, and is null for the other forms.  *live: see
-// k_m2l_live (null where an operator has more than 64 chunks).
+// k_m2l_live (null where an operator has more than 64 chunks, and in a lean context).
 tdbem_status tdbem_m2l_tc_images(tdbem_ctx* c, const float* ops, int nop, int P, int prec, uint4** img,
                                  float** opinv, unsigned long long** live) {
   using namespace tdbem;
@@ -1230,7 +1230,7 @@ tdbem_status tdbem_m2l_tc_images(tdbem_ctx* c, const float* ops, int nop, int P,
   const int64_t nunits = (int64_t)nop * 2 * nrt * nch * nparts * 1024;
   tdbem_status s = c->dalloc(img, nunits);
   if (s) return s;
-  if (nch <= 64) {
+  if (nch <= 64 && !c->lean) {
     if ((s = c->dalloc(live, (size_t)nop * 2 * nrt))) return s;
     k_m2l_live<<<(unsigned)(nop * 2 * nrt), 256, 0, c->stream>>>(ops, P, nrt, KC, *live);
     TDBEM_CUDA_TRY(c, cudaGetLastError());

@@ -63,3 +63,19 @@ def test_steps_of_many_edge_lengths(name, c, R, precond):
     y = _solver(v, t, c, 4, R, precond=precond, jacobi_sweeps=1).march(4)
     # as above: both residuals below 1e-13 |b|
     assert np.abs(x - y).max() <= 2 * (4000 if name == "uv13" else 100) * 1e-13 * np.abs(y).max()
+
+
+def test_a_long_ring_within_one_copy_of_its_store():
+    """Rings of 129 to 256 steps are tiled beside the FP64 values; a budget that holds the values once (and the lags,
+    offsets and ring beside them, less than half of them here) gives the untiled form, which turns them into pairs in
+    place.  Both solve to 1e-13 a step; their sums agree to 2^-46 of their terms."""
+    from workloads.meshes import octa_ellipsoid
+
+    v, t = octa_ellipsoid(freq=11)
+    s = _solver(v, t, 0.15, 12)
+    i = s.info()
+    assert 128 <= i.max_lag < 256
+    b = _solver(v, t, 0.15, 12, max_device_bytes=int(1.5 * i.near_coef_bytes))
+    assert b.info().device_bytes_peak < i.device_bytes_peak
+    J, Jb = s.march(12), b.march(12)
+    assert np.abs(J - Jb).max() <= 1e-10 * np.abs(J).max()
