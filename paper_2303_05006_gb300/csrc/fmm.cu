@@ -938,15 +938,21 @@ __global__ void __launch_bounds__(256) k_near_history_flat_multi(const int64_t* 
     for (int64_t eb = e0; eb < e1; eb += 256) {
       const int64_t e = eb + first;
       float z = 0.f;
-      int o = 0;  // place in the ring, in units of R
+      int o = -1;  // place in the ring, in units of R
       if (e < e1) {
         const int q = __ldg(hmeta + e);
         const int b = alpha - (q & 0xff);
-        if (b >= 0) {  // (no history yet: a zero coefficient at a place that exists)
+        if (b >= 0) {
           z = __ldg(hval + e);
           o = (q >> 8) * L + (b & (L - 1));
         }
       }
+      // no entry, or no history yet: a zero coefficient at a place that the row reads anyway, so that a value that is
+      // not finite stays in the rows that have it (skipping such entries one by one took 1.4% of the 16-wave march)
+      const unsigned have = __ballot_sync(0xffffffffu, o >= 0);
+      if (!have) continue;
+      const int any = __shfl_sync(0xffffffffu, o, __ffs(have) - 1);
+      if (o < 0) o = any;
 #pragma unroll 8
       for (int k = 0; k < 32; k += 32 / RL) {
         const float zk = __shfl_sync(0xffffffffu, z, k + sub);

@@ -123,3 +123,19 @@ def test_every_step_of_the_blocked_direct_march(tmp_path, prec, size):
             e.reset()
             assert np.array_equal(e.march(Nt - 1), J[: Nt - 1]), Nt
         e.close()
+
+
+# what is not finite in the history reaches the rows that have an entry there, in its own right-hand side, and no other
+@pytest.mark.parametrize("R", [2, 3, 17])
+@pytest.mark.parametrize("value", [np.nan, np.inf, 1e200])
+def test_values_that_are_not_finite_stay_in_their_rows(R, value):
+    v, t, dt, o, mats, Z0 = _oracle("ell5", 0.3)
+    one, _ = _solver(v, t, dt, 6, mode=1, n_leaf=8, far_kernel=2, far_overlap=0)
+    s, _ = _solver(v, t, dt, 6, n_rhs=R, mode=1, n_leaf=8, far_kernel=2)
+    H = np.random.default_rng(1).standard_normal((1, R, s.ne))
+    H[0, 1, 0] = value
+    got = s.history_eval(2, H)
+    want = np.stack([one.history_eval(2, H[:, r]) for r in range(R)])
+    reached = np.nonzero(~np.isfinite(want[1]))[0]
+    assert 0 < len(reached) < s.ne // 4 and np.isfinite(want[[r for r in range(R) if r != 1]]).all()
+    assert np.array_equal(np.isfinite(got), np.isfinite(want))
