@@ -1136,7 +1136,8 @@ __global__ void k_near_fill(const int16_t* m_lo, const uint8_t* nlag, const int6
   int l3 = 3;
   const int n3 = j < 0 ? 0 : rt_window(m_lo, nlag, ne, i, j, rt_m0(B, rt_part(st / 4, nrt, B)), false, &l3);
   const int64_t src = n3 > 0 ? off[i * ne + j] + (l3 - m_lo[i * ne + j]) : 0;
-  meta[q * 32 + lane] = (uint32_t)(j < 0 ? 0 : j) | (uint32_t)l3 << 24;
+  // (an absent column reads the quad's first one with zero coefficients: what is not finite there stays beside its rows)
+  meta[q * 32 + lane] = (uint32_t)(j < 0 ? qcol[4 * q] : j) | (uint32_t)l3 << 24;
   for (uint32_t u = 0; u < nm; ++u)
     rt_put(Coef{}, out + ((size_t)g0 + u) * RtPrec<Coef>::kGroupBytes, lane, (int)u < n3 ? val[src + u] : 0.0);
 }

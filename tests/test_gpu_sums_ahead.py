@@ -139,3 +139,24 @@ def test_values_that_are_not_finite_stay_in_their_rows(R, value):
     reached = np.nonzero(~np.isfinite(want[1]))[0]
     assert 0 < len(reached) < s.ne // 4 and np.isfinite(want[[r for r in range(R) if r != 1]]).all()
     assert np.array_equal(np.isfinite(got), np.isfinite(want))
+
+
+def test_a_value_that_is_not_finite_stays_on_its_side_of_the_body():
+    """The direct march's stores pad the windows of 32 neighbouring rows to the longest, with zero coefficients, so
+    what is not finite may reach rows beside those that have an entry there, but no row across the body."""
+    from workloads.meshes import mean_edge_length, octa_ellipsoid
+
+    v, t = octa_ellipsoid(freq=11)
+    s, _ = _solver(v, t, 0.25 * mean_edge_length(v, t), 6)
+    assert s.info().near_coef_bytes >= 64 << 20  # four steps a pass, near pairs apart
+    ev = s.edges()[0]
+    mid = v[ev].mean(axis=1)
+    far = np.linalg.norm(mid - mid[0], axis=1)
+    far = np.nonzero(far > 0.7 * far.max())[0]
+    H = np.random.default_rng(1).standard_normal((1, s.ne))
+    for value in (np.nan, np.inf):
+        H[0, 0] = value
+        for a in (3, 4, 5):
+            got = s.history_eval(a, H)
+            assert not np.isfinite(got).all() or a == 3
+            assert np.isfinite(got[far]).all(), a
