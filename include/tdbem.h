@@ -106,7 +106,8 @@ typedef struct {
                             both at setup on each level and keeps the faster, with the resident-operator
                             kernel for the FP16 form (see tdbem_info.m2l_resident) and, for the split forms,
                             the streamed one as further candidates;
-                            1 forces the resident-operator kernel where it applies (128 elsewhere) */
+                            1 forces the resident-operator kernel where it applies (128 elsewhere),
+                            2 the streamed one (256 elsewhere; see tdbem_info.m2l_streamed) */
   int32_t precond;       /* Z0 solve preconditioner: 0 Jacobi; 1 (default) local inverses: each function's row of the
                             inverse of Z0 among the functions it couples to most strongly.  The solves on the
                             cooperative grid, of the FP32 and 24-bit direct marches and after jacobi_sweeps
@@ -384,6 +385,12 @@ typedef struct {
   int64_t history_bytes;           /* direct mode: bytes the history sum of the lags >= 3 streams per step (coefficient
                                       store and lag windows; a fourth of the far pairs', which are streamed once
                                       per four steps); 0 where it runs untiled */
+  int32_t m2l_streamed;            /* bit l set where level l's M2L runs the streamed kernel (split forms, at most 64
+                                      chunks of 128 bytes a row of the operator) */
+  int32_t solve_plan;              /* Z0 solve: 1 the cluster solve; 2 the FP32 and 24-bit direct marches' form of it;
+                                      0 the general kernels */
+  int32_t lean;                    /* 1: made without the plans that only save time, which did not fit the device
+                                      or max_device_bytes */
 } tdbem_info;
 tdbem_status tdbem_get_info(const tdbem_ctx* ctx, tdbem_info* info);
 

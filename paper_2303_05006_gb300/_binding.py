@@ -46,7 +46,8 @@ class Info(ctypes.Structure):
                 ("m2l_flops_per_step", ctypes.c_double), ("total_jacobi_sweeps", ctypes.c_int64),
                 ("m2l_tile_rows", ctypes.c_int32 * 8), ("z0_nnz", ctypes.c_int64), ("max_lag", ctypes.c_int32),
                 ("m2l_resident", ctypes.c_int32), ("device_bytes_peak", ctypes.c_int64),
-                ("history_bytes", ctypes.c_int64)]
+                ("history_bytes", ctypes.c_int64), ("m2l_streamed", ctypes.c_int32),
+                ("solve_plan", ctypes.c_int32), ("lean", ctypes.c_int32)]
 
 
 class TdbemError(RuntimeError):

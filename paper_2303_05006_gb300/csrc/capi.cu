@@ -201,7 +201,7 @@ tdbem_status tdbem_create(const double* verts, int64_t nv, const int32_t* tris, 
       p.m2l_prec < TDBEM_P_FP32 || p.m2l_prec > TDBEM_P_F16X3 ||
       !(p.mu > 0) || !(p.theta >= 0) || !(p.chi >= 0) || !(p.solve_tol > 0) || p.solve_maxit < 1 || p.n_rhs < 1 ||
       p.n_rhs > TDBEM_MAX_RHS || p.jacobi_sweeps < 0 ||
-      (p.m2l_tile_rows != 0 && p.m2l_tile_rows != 1 && p.m2l_tile_rows != 128 && p.m2l_tile_rows != 256) || p.precond < 0 ||
+      (p.m2l_tile_rows < 0 || (p.m2l_tile_rows > 2 && p.m2l_tile_rows != 128 && p.m2l_tile_rows != 256)) || p.precond < 0 ||
       p.precond > 1 || (p.far_overlap != 0 && p.far_overlap != 1) || p.solve_grid < 0 || p.solve_grid > 2 ||
       p.far_kernel < 0 || p.far_kernel > 3 || p.max_device_bytes < 0 || p.s_interp < 0 || p.s_interp > 1 ||
       p.t_interp < 0 || p.t_interp > 1 || p.a_deriv < 0 || p.a_deriv > 2 ||
@@ -925,6 +925,8 @@ tdbem_status tdbem_get_info(const tdbem_ctx* c, tdbem_info* info) {
   info->total_jacobi_sweeps = c->total_sweeps;
   info->z0_nnz = c->z0_nnz;
   info->solver_cluster = c->cluster;
+  info->solve_plan = tdbem_sc_kind(c);
+  info->lean = c->lean ? 1 : 0;
   info->max_lag = c->max_lag;
   if (c->p.mode == TDBEM_FAST) tdbem_fast_info(c, info);
   return TDBEM_OK;

@@ -1660,7 +1660,8 @@ tdbem_status tdbem_build_fast(tdbem_ctx* c) {
     // chunks.
     L.str_ok = (c->p.m2l_prec == TDBEM_P_BF16X3 || c->p.m2l_prec == TDBEM_P_TF32X3 ||
                 c->p.m2l_prec == TDBEM_P_F16X3) &&
-               tdbem_m2l_chunks(P, c->p.m2l_prec) <= 64 && !c->lean;
+               tdbem_m2l_chunks(P, c->p.m2l_prec) <= 64 && !c->lean &&
+               (c->p.m2l_tile_rows == 0 || c->p.m2l_tile_rows == 2);
     if (qmax >= 255) {
       c->set_error("fast: too many time intervals per interaction");
       return TDBEM_EINVAL;
@@ -1816,8 +1817,9 @@ tdbem_status tdbem_build_fast(tdbem_ctx* c) {
   // launches add nothing to the local coefficients.
   if (c->p.m2l_prec != TDBEM_P_FP32 && c->p.m2l_tile_rows != 0) {
     for (int l = 2; l <= F->lmax; ++l) {
-      F->lev[l].tc_mt = c->p.m2l_tile_rows == 256 ? 2 : 1;
+      F->lev[l].tc_mt = c->p.m2l_tile_rows == 256 || c->p.m2l_tile_rows == 2 ? 2 : 1;
       F->lev[l].res = c->p.m2l_tile_rows == 1 && F->lev[l].res_ok;
+      F->lev[l].str = c->p.m2l_tile_rows == 2 && F->lev[l].str_ok;
     }
   } else if (c->p.m2l_prec != TDBEM_P_FP32) {
     cudaEvent_t e0, e1;
@@ -2258,6 +2260,7 @@ void tdbem_fast_info(const tdbem_ctx* c, tdbem_info* info) {
                                  ? (F->lev[l].res ? 128 : 128 * F->lev[l].tc_mt)
                                  : 0;
     if (F->lev[l].res) info->m2l_resident |= 1 << l;
+    if (F->lev[l].str && F->lev[l].ntiles_tc[0]) info->m2l_streamed |= 1 << l;
   }
 }
 

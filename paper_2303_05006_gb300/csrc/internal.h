@@ -321,3 +321,4 @@ tdbem_status tdbem_bx_build(tdbem_ctx* c, int want, const std::vector<int32_t>& 
                             const std::vector<double>& zv);
 tdbem_status tdbem_sc_solve(tdbem_ctx* c, int32_t alpha, int32_t warm);
 void tdbem_sc_free(tdbem_ctx* c);
+int tdbem_sc_kind(const tdbem_ctx* c);  // tdbem_info.solve_plan

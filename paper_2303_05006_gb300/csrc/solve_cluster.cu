@@ -1691,6 +1691,8 @@ tdbem_status tdbem_sc_solve(tdbem_ctx* c, int32_t alpha, int32_t warm) {
   return TDBEM_OK;
 }
 
+int tdbem_sc_kind(const tdbem_ctx* c) { return !c->sc ? 0 : c->sc->bx ? 2 : 1; }
+
 void tdbem_sc_free(tdbem_ctx* c) {
   delete c->sc;
   c->sc = nullptr;
