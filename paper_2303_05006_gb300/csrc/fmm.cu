@@ -859,6 +859,7 @@ __global__ void __launch_bounds__(256) k_near_history_flat(const int64_t* hrow, 
 constexpr int kNB = 128;              // columns per block
 constexpr int kNBS = kNB + 1;         // row stride of the staged block (no bank conflicts when staging)
 constexpr int kNTaskEntries = 16384;  // entries per task (about)
+constexpr int kNearTileSmem = 160 * 1024;  // most that the staged block may take
 
 __global__ void __launch_bounds__(256) k_near_tile(const int4* tasks, const int32_t* corder, const int64_t* seg_ptr,
                                                    const float* cval, const uint16_t* cmeta, int64_t ne,
@@ -1422,6 +1423,8 @@ tdbem_status tdbem_build_fast(tdbem_ctx* c) {
               (s = c->dalloc(&F->d_rseg, std::max<int64_t>(1, nseg))) ||
               (s = c->dalloc(&F->d_spart, std::max<int64_t>(1, nseg))))
             return s;
+          // (as tdbem_m2l_limits)
+          TDBEM_CUDA_TRY(c, cudaFuncSetAttribute(k_near_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, kNearTileSmem));
           TDBEM_CUDA_TRY(c, cudaMemcpy(F->d_corder, corder.data(), ne * sizeof(int32_t), cudaMemcpyHostToDevice));
           TDBEM_CUDA_TRY(c, cudaMemcpy(F->d_seg_ptr, seg_ptr.data(), (nseg + 1) * sizeof(int64_t),
                                        cudaMemcpyHostToDevice));
@@ -1459,6 +1462,7 @@ tdbem_status tdbem_build_fast(tdbem_ctx* c) {
   TDBEM_CUDA_TRY(c, cudaFuncSetAttribute(k_p2m, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
   TDBEM_CUDA_TRY(c, cudaFuncSetAttribute(k_m2m_fact, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   TDBEM_CUDA_TRY(c, cudaFuncSetAttribute(k_l2l_fact, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+  if ((s = tdbem_m2l_limits(c))) return s;
 
   std::vector<double> tbox(4 * nt);
   for (int l = 0; l <= lmax; ++l) {
@@ -2091,12 +2095,7 @@ static tdbem_status near_lags3(tdbem_ctx* c, const double* ring, int32_t alpha, 
   // the staged block holds the lags 0 .. max_near_lag of kNB columns
   const int nlag = F->max_near_lag + 1;
   const int smem = (int)(kNBS * nlag * sizeof(float));
-  if (F->d_seg_ptr && smem <= 160 * 1024) {
-    static int smem_set = 0;
-    if (smem > smem_set) {
-      TDBEM_CUDA_TRY(c, cudaFuncSetAttribute(k_near_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-      smem_set = smem;
-    }
+  if (F->d_seg_ptr && smem <= kNearTileSmem) {
     if (F->ntask)
       k_near_tile<<<(unsigned)F->ntask, 256, smem, st>>>(
           F->d_ntasks, F->d_corder, F->d_seg_ptr, F->d_cval, F->d_cmeta, c->ne, ring, c->L, nlag, alpha, 3,

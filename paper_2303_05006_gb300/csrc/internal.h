@@ -116,6 +116,7 @@ struct tdbem_ctx {
   int32_t R = 1;                    // right-hand sides (params.n_rhs)
   int32_t L = 0;                    // ring length (power of two)
   double* d_Jring = nullptr;        // [ne][L][R]
+  int nsm = 0;                      // SMs of the device (fast mode)
   bool lean = false;                // without the plans that only save time (the context would not fit otherwise)
   float* d_rf = nullptr;            // fast mode, R > 1: the ring in FP32 [ne][L][R], kept up to date by the solve
   float2* d_ring2 = nullptr;        // direct mode, R = 1: split history [L][ne] (hi, lo) (untiled kernel)
@@ -292,6 +293,7 @@ tdbem_status tdbem_m2l_pack_split(tdbem_ctx* c, const int32_t* cS, const int16_t
                                   const int16_t* smap, const float* mom, int k, int R, int PS, int pt, int prec,
                                   uint8_t* pk, float* pkinv);
 int tdbem_m2l_chunks(int P, int prec);
+tdbem_status tdbem_m2l_limits(tdbem_ctx* c);
 void tdbem_fast_info(const tdbem_ctx* c, tdbem_info* info);
 void tdbem_fast_state(tdbem_ctx* c, std::vector<std::pair<void*, size_t>>* bufs);
 tdbem_status tdbem_fast_z0_source(const tdbem_ctx* c, const int64_t** row_ptr, const int32_t** col,

@@ -1177,6 +1177,19 @@ int tdbem_m2l_chunks(int P, int prec) {
   return (P + KC - 1) / KC;
 }
 
+// The kernels' shared-memory limits, for the context's device, at its creation: a first launch that sets them once per
+// process misses other devices and races with other contexts' threads.
+tdbem_status tdbem_m2l_limits(tdbem_ctx* c) {
+  using namespace tdbem;
+  const auto lim = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  TDBEM_CUDA_TRY(c, cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, c->device));
+  TDBEM_CUDA_TRY(c, cudaFuncSetAttribute(k_m2l_tc<1>, lim, smem_tiles<1>() + kSmapSmem + 1024));
+  TDBEM_CUDA_TRY(c, cudaFuncSetAttribute(k_m2l_tc<2>, lim, smem_tiles<2>() + kSmapSmem + 1024));
+  TDBEM_CUDA_TRY(c, cudaFuncSetAttribute(k_m2l_res, lim, kResSmem));
+  TDBEM_CUDA_TRY(c, cudaFuncSetAttribute(k_m2l_stream, lim, kStrSmem));
+  return TDBEM_OK;
+}
+
 // Launch the tensor-core M2L of one level event with mt (1 or 2) 128-row
 // operator tiles per CTA; tiles must be the list planned for that mt.
 template <int kMT>
@@ -1186,12 +1199,6 @@ static tdbem_status launch_m2l_tc(tdbem_ctx* c, const int4* gemm, const int4* ti
                                   const float* opinv, const float* pkinv, const unsigned long long* live,
                                   int32_t* err) {
   using namespace tdbem;
-  static bool attr = false;
-  if (!attr) {
-    TDBEM_CUDA_TRY(c, cudaFuncSetAttribute(k_m2l_tc<kMT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           smem_tiles<kMT>() + kSmapSmem + 1024));
-    attr = true;
-  }
   if (ntiles == 0) return TDBEM_OK;
   const size_t smem = smem_tiles<kMT>() + (48 * PS * 2 <= kSmapSmem ? 48 * PS * 2 : 0) + 1024;
   k_m2l_tc<kMT><<<ntiles, kThreads, smem, c->stream>>>(gemm, tiles, img, P, pt, PS, pO, pC, psym, smap, pk, k, loc,
@@ -1275,19 +1282,13 @@ tdbem_status tdbem_m2l_res(tdbem_ctx* c, const int4* gemm, const int4* units, in
                            const int16_t* smap, const uint8_t* pk, int k, float* loc, int Q, int R,
                            const float* opinv, const float* pkinv, int32_t* err, int max_ctas) {
   using namespace tdbem;
-  static bool attr = false;
-  static int nsm = 0;
-  if (!attr) {
-    TDBEM_CUDA_TRY(c, cudaFuncSetAttribute(k_m2l_res, cudaFuncAttributeMaxDynamicSharedMemorySize, kResSmem));
-    TDBEM_CUDA_TRY(c, cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
-    attr = true;
-  }
   if (n <= 0) return TDBEM_OK;
   const int nch = tdbem_m2l_chunks(P, TDBEM_P_F16X3);
   if (nch > kResMaxCh) {
     c->set_error("fast: resident-operator M2L needs P <= 256");
     return TDBEM_EINVAL;
   }
+  const int nsm = c->nsm;
   const int grid = max_ctas < 0 ? n : std::min(n, max_ctas > 0 ? std::min(max_ctas, nsm) : nsm);
   k_m2l_res<<<grid, kResThreads, kResSmem, c->stream>>>(gemm, units + u0, n, img, P, nch, pt, PS, pO, pC, psym, smap,
                                                          pk, k, loc, Q, R, opinv, pkinv, err);
@@ -1314,15 +1315,8 @@ tdbem_status tdbem_m2l_stream(tdbem_ctx* c, const int4* gemm, const int4* tiles,
                               const uint8_t* pk, int k, float* loc, int Q, int R, int prec, const float* opinv,
                               const float* pkinv, const unsigned long long* live, int32_t* err, int max_run) {
   using namespace tdbem;
-  static bool attr = false;
-  static int nsm = 0;
-  if (!attr) {
-    TDBEM_CUDA_TRY(c, cudaFuncSetAttribute(k_m2l_stream, cudaFuncAttributeMaxDynamicSharedMemorySize, kStrSmem));
-    TDBEM_CUDA_TRY(c, cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
-    attr = true;
-  }
   if (n <= 0) return TDBEM_OK;
-  const int run = std::max(1, std::min(max_run, n / (2 * nsm)));
+  const int nsm = c->nsm, run = std::max(1, std::min(max_run, n / (2 * nsm)));
   const int groups = (n + nsm * run - 1) / (nsm * run), rest = n - (groups - 1) * nsm * run;
   k_m2l_stream<<<(groups - 1) * nsm + std::min(nsm, rest), kResThreads, kStrSmem, c->stream>>>(
       gemm, tiles, n, run, nsm, img, P, tdbem_m2l_chunks(P, prec), split_fmt(prec), pt, PS, pO, pC, psym, smap, pk, k, loc,
