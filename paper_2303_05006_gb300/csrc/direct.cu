@@ -938,7 +938,7 @@ __global__ void __launch_bounds__(kRtWarps * 32, MINB)
   }
 }
 
-// Near store and kernel, one step.  The near pairs of 32 rows would fill a third
+// Near store of the (hi, lo) pairs and its kernel, one step.  The near pairs of 32 rows would fill a third
 // of a tile's lanes (the rows' near columns differ), so the near tier takes 8
 // positions and 4 of their columns at a time: a quad owns as many groups of 32
 // values as its longest window has lags, lane 8 s + r holding the coefficients of
@@ -951,46 +951,12 @@ __global__ void __launch_bounds__(kRtWarps * 32, MINB)
 constexpr int kNearGroups = 64;  // groups per chunk (about)
 constexpr int kNearAhead = 8;
 
-template <typename Coef>
-struct NearVal;
-template <>
-struct NearVal<float> {
-  float v;
-  __device__ void load(const unsigned char* val, size_t g, int lane) {
-    v = __ldg(reinterpret_cast<const float*>(val) + g * 32 + lane);
-  }
-  __device__ float get() const { return v; }
-};
-template <>
-struct NearVal<float2> {
-  float2 v;
-  __device__ void load(const unsigned char* val, size_t g, int lane) {
-    v = __ldg(reinterpret_cast<const float2*>(val) + g * 32 + lane);
-  }
-  __device__ float2 get() const { return v; }
-};
-template <>
-struct NearVal<F24> {
-  uint32_t h, l;
-  __device__ void load(const unsigned char* val, size_t g, int lane) {
-    const unsigned char* p = val + g * 96;
-    h = __ldg(reinterpret_cast<const uint16_t*>(p) + lane);
-    l = __ldg(p + 64 + lane);
-  }
-  __device__ float get() const { return __uint_as_float(__byte_perm(l, h, 0x5401)); }
-};
-__device__ __forceinline__ void near_hist(float* x, const float2* p) { *x = p->x; }
-__device__ __forceinline__ void near_hist(float2* x, const float2* p) { *x = *p; }
-
-template <typename Coef>
-__global__ void __launch_bounds__(256) k_direct_near(const unsigned char* __restrict__ val,
+__global__ void __launch_bounds__(256) k_direct_near(const float2* __restrict__ val,
                                                      const uint32_t* __restrict__ qoff,
                                                      const uint32_t* __restrict__ meta,
                                                      const int4* __restrict__ chunks, int32_t nchunk, const float2* rs,
                                                      int32_t L, int32_t alpha, int64_t npos,
                                                      double* __restrict__ partial) {
-  using Hist = typename RtPrec<Coef>::Hist;
-  constexpr bool kF32 = !std::is_same<Coef, float2>::value;
   const int wid = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (wid >= nchunk) return;  // whole warps
   const int4 ch = chunks[wid];
@@ -1003,26 +969,18 @@ __global__ void __launch_bounds__(256) k_direct_near(const unsigned char* __rest
     // the slot of a step not there yet holds zero; one of a lag past the window
     // (zero coefficient) is finite
     int b = alpha - (int)(mt >> 24);
-    float a = 0.f;
     for (; g < ge; g += kNearAhead, b -= kNearAhead) {
-      NearVal<Coef> z[kNearAhead];
-      Hist x[kNearAhead];
+      float2 z[kNearAhead], x[kNearAhead];
 #pragma unroll
       for (int i = 0; i < kNearAhead; ++i)
         if (g + i < ge) {
-          z[i].load(val, (size_t)g + i, lane);
-          near_hist(&x[i], h + ((b - i) & (L - 1)));
+          z[i] = __ldg(val + ((size_t)g + i) * 32 + lane);
+          x[i] = h[(b - i) & (L - 1)];
         }
 #pragma unroll
       for (int i = 0; i < kNearAhead; ++i)
-        if (g + i < ge) {
-          if constexpr (kF32)
-            a = __fmaf_rn(z[i].get(), x[i], a);
-          else
-            df_fma_acc(sh, sl, z[i].get(), x[i]);
-        }
+        if (g + i < ge) df_fma_acc(sh, sl, z[i], x[i]);
     }
-    if constexpr (kF32) df_add(sh, sl, a, 0.f);
     g = ge;
     ge = gn;
     mt = mn;
@@ -1124,10 +1082,9 @@ __global__ void k_rt_fill(const int16_t* m_lo, const uint8_t* nlag, const int64_
 
 // The near pairs' quads: one warp per quad q of sub-tile qst[q]; qcol[4 q + s] its
 // columns (edges; -1: none).
-template <typename Coef>
 __global__ void k_near_fill(const int16_t* m_lo, const uint8_t* nlag, const int64_t* off, const double* val,
                             int64_t ne, int32_t nrt, int64_t nq, const int32_t* rows, int B, const int32_t* qst,
-                            const int32_t* qcol, const uint32_t* qoff, uint32_t* meta, unsigned char* out) {
+                            const int32_t* qcol, const uint32_t* qoff, uint32_t* meta, float2* out) {
   const int64_t q = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (q >= nq) return;  // whole warps
@@ -1139,7 +1096,7 @@ __global__ void k_near_fill(const int16_t* m_lo, const uint8_t* nlag, const int6
   // (an absent column reads the quad's first one with zero coefficients: what is not finite there stays beside its rows)
   meta[q * 32 + lane] = (uint32_t)(j < 0 ? qcol[4 * q] : j) | (uint32_t)l3 << 24;
   for (uint32_t u = 0; u < nm; ++u)
-    rt_put(Coef{}, out + ((size_t)g0 + u) * RtPrec<Coef>::kGroupBytes, lane, (int)u < n3 ? val[src + u] : 0.0);
+    out[((size_t)g0 + u) * 32 + lane] = (int)u < n3 ? split_pair(val[src + u]) : make_float2(0.f, 0.f);
 }
 
 // Lag-2 entries of the direct store, as a CSR over the positions of the row
@@ -1395,8 +1352,7 @@ static double* near_out(const tdbem_ctx* c, int buf) {
 static tdbem_status direct_near(tdbem_ctx* c, int32_t alpha, const float2* rs, int buf) {
   if (c->rt_units) return c->rt_B > 1 ? direct_rt(c, alpha, 1, rs, c->rt_B, near_out(c, buf)) : TDBEM_OK;
   if (!c->rt_nchunk) return TDBEM_OK;
-  auto fn = c->rt_prec == 1 ? k_direct_near<float> : c->rt_prec == 3 ? k_direct_near<F24> : k_direct_near<float2>;
-  fn<<<(unsigned)((c->rt_nchunk + 7) / 8), 256, 0, c->stream>>>(c->d_nt_val, c->d_nt_qoff, c->d_nt_meta, c->d_nt_chunk,
+  k_direct_near<<<(unsigned)((c->rt_nchunk + 7) / 8), 256, 0, c->stream>>>(c->d_nt_val, c->d_nt_qoff, c->d_nt_meta, c->d_nt_chunk,
                                                                 c->rt_nchunk, rs, c->L, alpha, (int64_t)c->rt_nrt * 32,
                                                                 near_out(c, buf));
   TDBEM_CUDA_TRY(c, cudaGetLastError());
@@ -1782,19 +1738,18 @@ static tdbem_status build_row_tiles(tdbem_ctx* c, int prec) {
     return TDBEM_EINVAL;
   }
   goff[ntc] = (uint32_t)acc;
-  const size_t nbytes = (size_t)acc * rt_group_bytes(prec), nearbytes = (size_t)nacc * rt_group_bytes(prec);
+  const size_t nbytes = (size_t)acc * rt_group_bytes(prec), nearbytes = (size_t)nacc * 32 * sizeof(float2);
   const int64_t nq = (int64_t)qst.size();
   int32_t *d_qst = nullptr, *d_qcol = nullptr;
   if ((s = up(c, &c->d_rt_goff, goff)) || (s = c->dalloc(&c->d_rt_val, nbytes)) || (s = up(c, &d_qst, qst)) ||
       (s = up(c, &d_qcol, qcol)) || (s = up(c, &c->d_nt_qoff, qoff)) || (s = up(c, &c->d_nt_chunk, chunks)) ||
-      (s = c->dalloc(&c->d_nt_meta, (size_t)nq * 32)) || (s = c->dalloc(&c->d_nt_val, nearbytes)))
+      (s = c->dalloc(&c->d_nt_meta, (size_t)nq * 32)) || (s = c->dalloc(&c->d_nt_val, (size_t)nacc * 32)))
     return s;
   auto fill = prec == 1 ? k_rt_fill<float> : prec == 3 ? k_rt_fill<F24> : k_rt_fill<float2>;
   fill<<<nb, 256, 0, c->stream>>>(st.m_lo, st.nlag, st.off, st.val, ne, (int32_t)nrt, c->d_rt_row, B, units, c->d_rt_goff,
                                   c->d_rt_val);
   if (nq) {
-    auto nfill = prec == 1 ? k_near_fill<float> : prec == 3 ? k_near_fill<F24> : k_near_fill<float2>;
-    nfill<<<(unsigned)((nq * 32 + 255) / 256), 256, 0, c->stream>>>(st.m_lo, st.nlag, st.off, st.val, ne, (int32_t)nrt,
+    k_near_fill<<<(unsigned)((nq * 32 + 255) / 256), 256, 0, c->stream>>>(st.m_lo, st.nlag, st.off, st.val, ne, (int32_t)nrt,
                                                                     nq, c->d_rt_row, B, d_qst, d_qcol, c->d_nt_qoff,
                                                                     c->d_nt_meta, c->d_nt_val);
   }

@@ -139,7 +139,7 @@ struct tdbem_ctx {
   int32_t rt_units = 0;             // tiers by whole (tile, column block) units of one store, columns in edge order
   int64_t rt_bytes = 0;             // bytes streamed per step (values, lag bytes, group offsets)
   int32_t* d_rt_lomin = nullptr;    // [nrt][ncb] smallest far lag of (tile, column block)
-  unsigned char* d_nt_val = nullptr;  // near pairs: groups of the quads (8 rows x 4 columns)
+  float2* d_nt_val = nullptr;       // near pairs of the (hi, lo) store: groups of the quads (8 rows x 4 columns)
   uint32_t* d_nt_qoff = nullptr;    // first group of a quad
   uint32_t* d_nt_meta = nullptr;    // [quads][32] column | first lag << 24
   int4* d_nt_chunk = nullptr;       // [rt_nchunk] {sub-tile, first quad, end, partial slot}
