@@ -17,6 +17,7 @@
   do {                                                                                  \
     cudaError_t e__ = (call);                                                           \
     if (e__ != cudaSuccess) {                                                           \
+      cudaGetLastError(); /* reported here: not once more by the next launch's check */ \
       (ctx)->set_error(std::string(#call) + ": " + cudaGetErrorString(e__));            \
       return (e__ == cudaErrorMemoryAllocation) ? TDBEM_ENOMEM : TDBEM_ECUDA;           \
     }                                                                                   \
@@ -210,6 +211,7 @@ struct tdbem_ctx {
     }
     cudaError_t e = cudaMalloc((void**)ptr, count * sizeof(T));
     if (e != cudaSuccess) {
+      cudaGetLastError();  // as TDBEM_CUDA_TRY
       set_error(std::string("cudaMalloc: ") + cudaGetErrorString(e));
       *ptr = nullptr;
       return TDBEM_ENOMEM;
