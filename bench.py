@@ -191,10 +191,11 @@ def batch_pulses(w, n: int, seed: int = 4):
     return [pulse_star(w.verts, k=k, pol=pol) for k, pol in random_plane_waves(n, seed)] if n > 0 else []
 
 
-# dram__bytes_read.sum + dram__bytes_write.sum per k_m2l_tc launch, zero blocks included (TF32x3, p = 4, 7680 RWG, two
-# 128-row tiles per CTA, lag >= 2 products deferred): two leaf events of 289.5 MB and one level-2
-# event of 152.9 MB per gating period of six launches
-M2L_TRAFFIC_TF32X3 = (2 * 289.5e6 + 152.9e6) / 6
+# dram__bytes_read.sum + dram__bytes_write.sum per M2L launch (TF32x3, p = 4, 7680 RWG, lag >= 2 products deferred): two
+# leaf events and one level-2 event per gating period of six launches, with k_m2l_tc (two 128-row tiles per CTA) and with
+# k_m2l_stream
+M2L_TRAFFIC_TF32X3 = (2 * 271.0e6 + 141.1e6) / 6
+M2L_TRAFFIC_TF32X3_STREAMED = (2 * 454.8e6 + 158.2e6) / 6
 
 PREC = {"fp32": 0, "tf32": 1, "bf16": 2, "bf16x3": 3, "tf32x3": 4, "f16x3": 5}
 KERNELS = ["incident_rhs", "near_history", "z0_solve", "p2m", "m2m", "m2l", "l2l", "l2p", "m2l_pack",
@@ -220,12 +221,13 @@ def roofline(args, info, launches, ms, K, W):
         peak = bf16 if args.prec in ("bf16", "bf16x3", "f16x3") else bf16 * 1.1 / 2.25
         how = f"{src} bf16_tflops" + ("" if not args.prec.startswith("tf32") else " x 1.1/2.25 (nominal TF32/BF16)")
         # DRAM bytes of one launch from the committed ncu capture of this kernel and configuration
-        traffic = (M2L_TRAFFIC_TF32X3 if (M2L_TRAFFIC_TF32X3 and args.prec == "tf32x3" and args.p == 4
-                                          and args.rhs == 1 and args.workload == "sphere7680" and args.far_overlap
-                                          and list(info.m2l_tile_rows)[2:4] == [256, 256]) else None)
+        traffic = None
+        if (args.prec == "tf32x3" and args.p == 4 and args.rhs == 1 and args.workload == "sphere7680"
+                and args.far_overlap and list(info.m2l_tile_rows)[2:4] == [256, 256]):
+            traffic = {0: M2L_TRAFFIC_TF32X3, 0b1100: M2L_TRAFFIC_TF32X3_STREAMED}.get(getattr(info, "m2l_streamed", 0))
         return {"kernel": name, "bound": "tensor", "achieved": tflops, "peak": peak, "unit": "TFLOP/s",
                 "frac": tflops / peak, "traffic": traffic,
-                "traffic_source": "profiles/m2l_tc_sphere7680_tf32x3.md (mean of one gating period's launches)"
+                "traffic_source": "profiles/m2l_stream_tf32x3.md (mean of one gating period's launches)"
                 if traffic else None,
                 "peak_source": how,
                 "flops_per_launch": flops / max(launches[dom], 1),
@@ -246,8 +248,14 @@ def roofline(args, info, launches, ms, K, W):
         return {"kernel": name, "bound": "hbm", "achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm,
                 "traffic": None, "traffic_source": None,
                 "peak_source": f"{src} hbm_gbs", "bytes_per_launch": nbytes}
+    if name == "z0_solve" and getattr(info, "solve_plan", 0):
+        # the cluster solve reads its own matrices (Z0 P, P, Z0 without its stored zeros) from L2 and keeps the
+        # vectors on the chip: no byte count of Z0 describes it
+        return {"kernel": name, "bound": "latency", "achieved": None, "peak": None, "unit": None, "frac": None,
+                "traffic": None, "note": "one cluster runs a few dependent BiCGStab iterations per solve, each with "
+                                         "cluster-wide barriers; its matrices stay in L2, the vectors on the chip"}
     if name == "z0_solve" and info.z0_nnz > 0:
-        # algorithmic operand bytes of one solve: per BiCGStab iteration two FP32
+        # the general kernels: algorithmic operand bytes of one solve: per BiCGStab iteration two FP32
         # SpMVs (value + column, 8 B per non-zero) and 4-byte vector passes (21 + 2 x 12
         # with a preconditioner of a few entries a row, 21 + 2 x 2 with the diagonal one);
         # two FP64 residuals (12 B per non-zero, 3 vectors)

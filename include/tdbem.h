@@ -112,7 +112,9 @@ typedef struct {
                             inverse of Z0 among the functions it couples to most strongly.  The solves on the
                             cooperative grid, of the FP32 and 24-bit direct marches and after jacobi_sweeps
                             take triangle blocks in its place (the inverses of the 3 x 3 blocks of Z0 among
-                            the RWG functions of each triangle, summed) */
+                            the RWG functions of each triangle, summed), and so does a solve whose trial at
+                            setup converges faster with them (long thin triangles at time steps of many edge
+                            lengths) */
   int32_t far_overlap;   /* 1 (default): the steps overlap.  Fast mode: the M2L products of a gating event with
                             lag q >= 2, whose local coefficients are first read one interval later, run on a
                             lowest-priority second stream of the context while the next steps proceed; with
@@ -155,13 +157,15 @@ typedef struct {
                             (section 4.3.2): 0 (default) the paper's split, one on the interpolated kernel
                             (dU/dt) and one on the target's time factor; 1 both on the target factor (U
                             interpolated); 2 both on the kernel (d^2U/dt^2, a step in time, interpolated) */
-  int32_t solve_cluster;  /* CTAs of a right-hand side's solve cluster: 1, 2, 4, 8 or 16 caps it; 0 (default)
-                             chooses by the size of Z0 and the number of right-hand sides (at most the largest
-                             cluster the device schedules, 16 on GB300) */
+  int32_t solve_cluster;  /* CTAs of the solve cluster with one right-hand side: 1, 2, 4, 8 or 16 caps it; 0
+                             (default) chooses by the size of Z0 (at most the largest cluster the device
+                             schedules, 16 on GB300).  With several right-hand sides, a cluster each, it is not
+                             read: their number and the size of Z0 choose. */
   int64_t max_device_bytes; /* device memory budget of the context's own allocations (0: none).  An allocation
                                that would exceed it fails as if the device were full: tdbem_create tries again
-                               without what only saves time (the cluster solve's plan, second copies), then
-                               returns TDBEM_ENOMEM with nothing left allocated.  Per-call temporaries of
+                               without what only saves time (the cluster solve's plan, second copies; they also
+                               have to leave room for incident rows, Nt x ne x n_rhs values; tdbem_info.lean
+                               says so), then returns TDBEM_ENOMEM with nothing left allocated.  Per-call temporaries of
                                tdbem_history_eval and the learned warm start's buffers (tdbem_mlp_*) are
                                outside it. */
   int32_t p2p_prec;      /* direct mode, precision of the stored coefficients Zt^(m) of the lags m >= 3 in the

@@ -1809,7 +1809,7 @@ static tdbem_status build_row_tiles(tdbem_ctx* c, int prec) {
 
 // Single right-hand side, after Z0 and the lag-2 entries have been read from
 // the FP64 store: the row-tile store of the lags >= 3 in the precision of
-// p2p_prec (ring length L <= 128), which replaces the FP64 values; else the
+// p2p_prec (rings of up to 128 steps, 256 in (hi, lo) pairs), which replaces the FP64 values; else the
 // FP64 values split in place into (hi, lo) pairs for the untiled kernel and
 // its split ring.
 tdbem_status tdbem_direct_split(tdbem_ctx* c) {

@@ -16,8 +16,8 @@
 // unit u holding row u >> 3 and K bytes 16((u & 7) ^ (row & 7)) .. +15.  Eight
 // neighbouring threads then read one row's 128 bytes from global memory in one
 // line and write them free of bank conflicts.  (In the layout without swizzle eight
-// neighbours belong to eight rows: every 16-byte gather touched 32 lines a warp, and
-// L1 was 72% busy.  M2L per step: p = 6, 1,920 RWG 1039 -> 982 us; p = 4, 16
+// neighbours belong to eight rows: every 16-byte gather touched 32 lines a warp.
+// M2L per step: p = 6, 1,920 RWG 1039 -> 982 us; p = 4, 16
 // right-hand sides, 4,608 RWG 800 -> 660 us.)  The operators are converted once at setup into
 // exactly these images (TF32, BF16, or hi and lo parts for the split forms,
 // zero-padded past P) and brought in by TMA bulk copies (cp.async.bulk, one
@@ -878,16 +878,16 @@ __global__ void __launch_bounds__(kResThreads, 1)
 // 32 KB) and 12 MMAs of 128 x 256 x 32 bytes, about as long as the operands take
 // from L2, so the two have to overlap.  k_m2l_tc converts the moments between its loads
 // and its MMAs and waits for each chunk's MMAs before it asks for the next operator
-// rows; with two CTAs per SM the tensor pipe was 33% busy at p = 6.  Here the moments come
+// rows; its tensor pipe is 25% busy at p = 6, this kernel's 51%.  Here the moments come
 // packed as hi and lo parts (k_m2l_pack_split), and the roles of k_m2l_res run over a ring of
 // two 96 KB stages: warps 0-3 copy the moment columns (cp.async) and thread 0 the
 // operator tiles (bulk copies), one warp issues the MMAs, warps 5-8 drain one of two
 // 256-column accumulators while the other fills.  A CTA does `run` tiles, `side` (one per SM)
 // apart, so that the CTAs at work at one time hold neighbouring tiles, which share operator rows
-// and moment columns in L2 (with `run` consecutive tiles per CTA L2 hit 36% of the reads, not 72%).
+// and moment columns in L2 (71% of its reads hit; `run` consecutive tiles per CTA took 789 us a step at p = 6).
 // Every wait is bounded as in k_m2l_res.  M2L per step, before and after: TF32x3, p = 6,
-// 1,920 RWG 982 -> 722 us; TF32x3, p = 4, sphere and cube, 12,864 RWG 311 -> 233 us (asking for the operator
-// chunks in L2 four chunks early made both slower).
+// 1,920 RWG 982 -> 722 us; one deferred launch of TF32x3, p = 4, 7,680 RWG 649 -> 492 us (asking for the operator
+// chunks in L2 four chunks early made it slower).
 constexpr int kStrStages = 2;
 constexpr int kStrStage = 6 * kTileBytes;  // operator hi (256 rows), operator lo, moments hi, moments lo
 constexpr int kStrSmem = kStrStages * kStrStage + 1024;

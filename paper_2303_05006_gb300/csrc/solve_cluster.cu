@@ -5,14 +5,15 @@
 // Scheme.  Iterative refinement: an FP64 residual r = b - Z0 x around an FP32
 // BiCGStab on the right-preconditioned matrix A = Z0 P, which is formed once at
 // setup.  Row i of P is row i of the inverse of the block of Z0 among edge i and
-// its kScK - 1 strongest couplings (k_local_inverse), or the diagonal's inverse.
-// Against the triangle blocks used before, 32 couplings take a third of the
+// its kScK - 1 strongest couplings (k_local_inverse), or where a trial at setup says so of
+// the triangle blocks, or the diagonal's inverse.
+// Against the triangle blocks, 32 couplings take a third of the
 // iterations (to 1e-5: 7680-RWG sphere 3 to 1, cone-capped cylinder 14.5 to 3.5,
 // octahedral ellipsoid 12.5 to 4.5, UV ellipsoid 44.5 to 10.5), and A has about as
 // many entries, as it is close to the identity: entries below 1e-6 are left out
 // (they would change a correction by less than the 1e-5 it is computed to; the
 // FP64 residual decides).  The Krylov vectors live in
-// registers, each thread owning kScRows rows; only the vector that the next
+// registers, each thread owning 1 to 6 rows; only the vector that the next
 // product gathers from travels: every owner stores its values into all CTAs'
 // copies through distributed shared memory, so the gathers are shared-memory
 // reads and an iteration meets at four cluster barriers (p, alpha's dots, s,
@@ -22,9 +23,14 @@
 // four blocks of 8 rows x 16 entries per warp keeps about 50 KB in flight per
 // SM), the reductions are dependent shuffles.  FP64 issues at 1/64 of FP32's
 // rate here (2 per clock and SM), so FP64 is left to the residuals and the
-// iterate; the dots are summed in double-float (FP32 pairs, 48 bits), the
-// Krylov scalars are FP32 and the refinement's scale is a power of two, which
-// needs no FP64 division or square root.
+// iterate.  Inside the FP32 correction the dots are FP32 over a thread's rows and
+// double-float (FP32 pairs, 48 bits) from there, the Krylov scalars are FP32, and
+// |s|^2 and |r|^2 follow from the same dots (k_bicgstab has FP64 for all of these); the
+// refinement's scale is a power of two, which needs no FP64 division or square root.
+// What the correction is worth is decided by the FP64 residual, or by the one carried
+// on where the tolerance leaves room for what that misses.
+// 1920 RWG, 16 CTAs, alone under ncu: 64 us, 25% of issue slots, waiting for shared-memory
+// gathers first and barriers third.
 //
 // Layout.  Rows are put in an order of their own (`perm`): sorted by length,
 // cut into groups of 8 (four lanes per row, so that a warp takes one group at a
@@ -46,7 +52,7 @@ namespace tdbem {
 
 constexpr int kScThreads = 512, kScWarps = kScThreads / 32;
 constexpr int kScK = 32;            // entries per row of P at most
-constexpr double kScDrop = 1e-6;    // entries of A left out (A is close to the identity)
+constexpr double kScDrop = 1e-6;    // entries of A left out (A's diagonal is about 1)
 constexpr int kScPasses = 24;       // groups per warp at most: 6 rows per thread
 constexpr double kScInner2 = 1e-10; // squared relative residual an inner solve stops at
 constexpr int kScDepth = 4;          // blocks a warp keeps in flight
