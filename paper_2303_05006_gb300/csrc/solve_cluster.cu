@@ -487,6 +487,7 @@ __global__ void __launch_bounds__(kScThreads) k_solve_cluster(const ScArgs A) {
   int passes = 0;  // carried on since the last FP64 residual, at 2^k0 with
   float dd = 0.f;  // this thread's share of sum |d|^2 / 4^k0 over them
   int k0 = 0;
+  bool last = false;  // the correction was made for the tolerance: only then is |missed| summed
   double tol2bb = 0.0;
 #pragma unroll 1
   for (int outer = -1;; ++outer) {
@@ -506,15 +507,17 @@ __global__ void __launch_bounds__(kScThreads) k_solve_cluster(const ScArgs A) {
 #pragma unroll
       for (int e = 0; e < RPT; ++e) r64[e] = row[e] >= 0 ? r64[e] - sc * zd[e] : 0.0;
       ++passes;
-      double nr = 0.0, xx = (double)(0x1p18f * dd) * __hiloint2double((1023 + 2 * k0) << 20, 0);
+      double nr = 0.0, xx = 0.0;
 #pragma unroll
-      for (int e = 0; e < RPT; ++e) {
-        nr += r64[e] * r64[e];
-        xx += x[e] * x[e];
+      for (int e = 0; e < RPT; ++e) nr += r64[e] * r64[e];
+      if (last) {
+        xx = (double)(0x1p18f * dd) * __hiloint2double((1023 + 2 * k0) << 20, 0);
+#pragma unroll
+        for (int e = 0; e < RPT; ++e) xx += x[e] * x[e];
       }
       S.sums64(nr, xx);
       rr = nr;
-      if (rr <= tol2bb && rr + 0x1p-101 * A.zn2 * xx > 0.5 * tol2bb) {
+      if (rr <= tol2bb && (!last || rr + 0x1p-101 * A.zn2 * xx > 0.5 * tol2bb)) {
         anew = true;
         --outer;
         continue;
@@ -555,7 +558,9 @@ __global__ void __launch_bounds__(kScThreads) k_solve_cluster(const ScArgs A) {
     // inner target: the reduction that brings the FP64 residual to half the outer
     // tolerance, within [1e-5, 0.5] (1e-5: what FP32 reliably reaches)
     const float rin = (float)(rr * inv * inv);
-    const float tin2 = fminf(fmaxf(0.25f * (float)(tol2bb * inv * inv) / rin, (float)kScInner2), 0.25f) * rin;
+    const float want2 = 0.25f * (float)(tol2bb * inv * inv) / rin;
+    const float tin2 = fminf(fmaxf(want2, (float)kScInner2), 0.25f) * rin;
+    last = want2 >= (float)kScInner2;
 #pragma unroll
     for (int e = 0; e < RPT; ++e) {
       u[e] = rh[e] = p[e] = (float)(r64[e] * inv);
